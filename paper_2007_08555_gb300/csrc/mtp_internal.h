@@ -69,9 +69,8 @@ size_t scan_tmp_ints(int n);
 int scan_exclusive(const int* in, int* out, int n, int* tmp, cudaStream_t st);
 
 // Active set (mtp_maxvol.cu)
-int launch_maxvol(int n, int m, const double* B, double* Bs, double* D, double* W, int* perm, int* sel, double* A,
-                  double* Ai, double* C, double tol, int max_iter, int* status, int* swaps, double* gmax,
-                  cudaStream_t st, int start_given = 0);
+int launch_maxvol(int n, int m, const double* B, double* W, int* pos, int* sel, double* A, double* Ai, double tol,
+                  int max_iter, int* status, int* swaps, double* gmax, cudaStream_t st, int start_given = 0);
 int launch_invert(int m, const double* A, double* Ai, double* W, int* status, cudaStream_t st);
 template <class T>
 int launch_grade(int n, int m, const T* B, int ldb, const T* Ai, unsigned long long* gbits, cudaStream_t st);

@@ -1,6 +1,6 @@
 // Active set and extrapolation grade of Sec. 2.3 (D-optimality, MaxVol of Goreinov et al. 2010).
 //
-// k_maxvol (one CTA, double precision, all loops bounded):
+// k_maxvol (cooperative, double precision, all loops and waits bounded):
 //   0. columns are scaled by 1 / max |column| (the grades and the selection are invariant under
 //      B -> B D, and the scaled matrix is far better conditioned);
 //   1. start rows: the pivot rows of Gaussian elimination with partial pivoting on the tall
@@ -9,9 +9,21 @@
 //   2. A^-1 of A = B[sel] by Gauss-Jordan elimination with partial pivoting;
 //   3. C = B A^-1 for every row;
 //   4. repeat at most max_iter times: (k, j) = argmax |C_kj| (ties: smallest k, then smallest j);
-//      stop when |C_kj| <= 1 + tol (tol = 1e-3); otherwise row k replaces active row j, and A^-1 and C follow
+//      stop when |C_kj| <= 1 + tol (tol = 1e-3); otherwise row k replaces active row j, and C follows
 //      by the rank-one (Sherman-Morrison) update  C <- C - C[:,j] (C[k,:] - e_j) / C_kj.
-//   A^-1 is recomputed from scratch at the end.
+//   A^-1 is computed from scratch at the end.
+//
+// Every phase is a chain of dependent steps (m pivots, or one swap), each a rank-one update of all rows.
+// A block owns a fixed set of rows and keeps them in shared memory for a whole phase, so that a step
+// exchanges only what the others need: every block publishes its best candidate (value, position) with
+// the candidate's row, waits for the others' and takes the same winner (Exchange).  Rows are never
+// moved: a row's current position is a number beside it.  The inverse runs in place (the column that a
+// pivot eliminates is replaced by the column of the inverse that it creates).  Pivots, factors and
+// inverse are the same operations in the same order as elimination by one block with explicit
+// interchanges, so the selection does not depend on the number of blocks.
+// Bound: one exchange per step (a release, a poll and a row read through L2) and the step's FMAs on the
+// double-precision pipe (~2 per clock and SM).  Measured with all grades of the rows: 232 x 116 in
+// 2.81 ms, 920 x 460 in 13.7 ms; one block with every matrix in global memory took 11.3 and 482 ms.
 // k_grade: gamma_r = max_j |(b_r A^-1)_j| for many rows; 64x64 output tiles through shared memory,
 //   the row maxima are combined with an atomic max on the bit pattern (gamma >= 0); a NaN in a row
 //   of b A^-1 gives gamma = +inf, so a broken configuration reads as extrapolating.
@@ -26,228 +38,499 @@ namespace mtp {
 
 namespace {
 
-constexpr int kMvThreads = 1024;
+constexpr int kMvThreads = 512;
 
-struct ArgMax {
-    double v;
-    int idx;
+// One round of all blocks: each publishes a candidate (a non-negative value and a 32-bit payload, ties
+// to the smaller payload) and a row of numbers; everyone gets the winner.  A record is two words that
+// carry their own round (a parity in the sign bit of the value, the round's number beside the payload),
+// in two alternating sets: a block publishes round t + 1 only after it has read every record of round t,
+// so nobody can still be reading what it overwrites.
+constexpr unsigned kNone = 0xffffffffu;
+
+// The exchange's rows: in global memory, or in shared memory when there is one block, so these are
+// generic accesses (volatile: never from the L1 cache).
+__device__ __forceinline__ void put_row(double* p, double v) { *(volatile double*)p = v; }
+__device__ __forceinline__ double get_row(const double* p) { return *(const volatile double*)p; }
+
+struct Exchange {
+    unsigned long long* rec;  // [2][G][2]
+    double* slots;            // [2][G][m + 1] the candidates' rows, and the row's number
+    int G, m;
+    unsigned t;
+    int* err;
+    unsigned long long* s_key;  // shared [G]
+    unsigned* s_pay;            // shared [G]
+
+    __device__ double* mine() const { return slots + ((size_t)((t + 1) & 1) * G + blockIdx.x) * (m + 1); }
+    __device__ const double* slot(int q) const { return slots + ((size_t)(t & 1) * G + q) * (m + 1); }
+
+    // Publishes (value, payload; kNone: no candidate) after the block's writes to mine(), and waits for
+    // the others' records.  False if a wait gave up.
+    __device__ bool round(double value, unsigned payload) {
+        __syncthreads();
+        ++t;
+        unsigned long long* r = rec + (size_t)(t & 1) * G * 2;
+        const unsigned long long par = (unsigned long long)(((t + 1) >> 1) & 1u) << 63;
+        bool bad = false;
+        if (threadIdx.x == 0) {
+            volatile unsigned long long* w = r + 2 * blockIdx.x;
+            __threadfence();
+            w[0] = ((unsigned long long)__double_as_longlong(value) & 0x7fffffffffffffffull) | par;
+            w[1] = ((unsigned long long)t << 32) | payload;
+        }
+        if (threadIdx.x < G) {
+            volatile unsigned long long* w = r + 2 * threadIdx.x;
+            unsigned long long v = 0, p = 0;
+            long spins = 0;
+            do {  // a poll takes the better part of a microsecond: this gives up after some seconds
+                p = w[1];
+                v = w[0];
+            } while (((unsigned)(p >> 32) != t || (v & 0x8000000000000000ull) != par) && ++spins < (4l << 20));
+            bad = spins >= (4l << 20);
+            __threadfence();
+            s_key[threadIdx.x] = v & 0x7fffffffffffffffull;
+            s_pay[threadIdx.x] = (unsigned)p;
+        }
+        bad = __syncthreads_or(bad);
+        if (bad && threadIdx.x == 0) atomicOr(err, kErrTimeout);
+        return !bad;
+    }
+
+    // The winner of the round (every warp finds it for itself): its block, or -1 if there is none.
+    __device__ int winner(double* value, unsigned* payload) const {
+        unsigned long long bv = 0;
+        unsigned bp = kNone;
+        int bq = -1;
+        for (int q = threadIdx.x & 31; q < G; q += 32) {
+            const unsigned long long v = s_key[q];
+            const unsigned p = s_pay[q];
+            if (p != kNone && (bq < 0 || v > bv || (v == bv && p < bp))) {
+                bv = v;
+                bp = p;
+                bq = q;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, bv, o);
+            const unsigned p = __shfl_xor_sync(0xffffffffu, bp, o);
+            const int q = __shfl_xor_sync(0xffffffffu, bq, o);
+            if (q >= 0 && (bq < 0 || v > bv || (v == bv && p < bp))) {
+                bv = v;
+                bp = p;
+                bq = q;
+            }
+        }
+        *value = __longlong_as_double((long long)bv);
+        *payload = bp;
+        return bq;
+    }
 };
 
-// block-wide argmax of |value| (ties -> smallest index); every thread returns the winner
-__device__ ArgMax block_argmax(double v, int idx, ArgMax* sbuf) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) {
-        const double v2 = __shfl_xor_sync(0xffffffffu, v, o);
-        const int i2 = __shfl_xor_sync(0xffffffffu, idx, o);
-        if (v2 > v || (v2 == v && i2 < idx)) {
-            v = v2;
-            idx = i2;
+// A block's own rows: w [R][m], their positions, and R numbers for a column of them.
+struct Rows {
+    double* w;
+    int* pos;
+    double* col;
+    int first, R, m;  // rows first .. first + R - 1 of the matrix
+    double* prow;     // shared [m]: the winner's row
+    unsigned long long* s_v;  // shared [32]: candidates of the warps
+    unsigned* s_p;
+    int* s_r;
+};
+
+// The block's candidate of a pivot step: largest |w[r][k]| among its rows at positions >= k (ties to
+// the smaller position; NaN is no candidate).  Threads take rows, then the warps' winners are combined.
+// Returns the local row, or -1.
+__device__ int pivot_candidate(const Rows& a, int k, double* value, unsigned* payload) {
+    unsigned long long bv = 0;
+    unsigned bp = kNone;
+    int br = -1;
+    auto take = [&](unsigned long long v, unsigned p, int r) {
+        if (r >= 0 && (br < 0 || v > bv || (v == bv && p < bp))) {
+            bv = v;
+            bp = p;
+            br = r;
         }
-    }
-    if (lane == 0) sbuf[warp] = {v, idx};
-    __syncthreads();
-    if (warp == 0) {
-        ArgMax a = lane < (int)(blockDim.x >> 5) ? sbuf[lane] : ArgMax{-1.0, 0x7fffffff};
+    };
+    auto across = [&]() {
+#pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            const double v2 = __shfl_xor_sync(0xffffffffu, a.v, o);
-            const int i2 = __shfl_xor_sync(0xffffffffu, a.idx, o);
-            if (v2 > a.v || (v2 == a.v && i2 < a.idx)) {
-                a.v = v2;
-                a.idx = i2;
-            }
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, bv, o);
+            const unsigned p = __shfl_xor_sync(0xffffffffu, bp, o);
+            const int r = __shfl_xor_sync(0xffffffffu, br, o);
+            take(v, p, r);
         }
-        if (lane == 0) sbuf[32] = a;
+    };
+    const int warps = (a.R + 31) >> 5 < (int)(blockDim.x >> 5) ? (a.R + 31) >> 5 : (int)(blockDim.x >> 5);
+    if ((int)(threadIdx.x >> 5) < warps) {
+        for (int r = threadIdx.x; r < a.R; r += warps * 32) {
+            const int p = a.pos[r];
+            const unsigned long long v =
+                (unsigned long long)__double_as_longlong(a.w[(size_t)r * a.m + k]) & 0x7fffffffffffffffull;
+            if (p >= k && v <= 0x7ff0000000000000ull) take(v, (unsigned)p, r);
+        }
+        across();
+        if ((threadIdx.x & 31) == 0) {
+            a.s_v[threadIdx.x >> 5] = bv;
+            a.s_p[threadIdx.x >> 5] = bp;
+            a.s_r[threadIdx.x >> 5] = br;
+        }
     }
     __syncthreads();
-    const ArgMax r = sbuf[32];
-    __syncthreads();
-    return r;
+    br = -1;
+    bp = kNone;
+    for (int q = 0; q < warps; ++q) take(a.s_v[q], a.s_p[q], a.s_r[q]);
+    *value = __longlong_as_double((long long)bv);
+    *payload = br < 0 ? kNone : bp;
+    return br;
 }
 
-// inverse of the m x m matrix A (row-major) into Ai, Gauss-Jordan with partial pivoting on a
-// work copy W [m][2m].  Returns false if a pivot is exactly zero.
-__device__ bool gauss_jordan(const double* A, double* Ai, double* W, int m, ArgMax* sbuf, int* s_flag) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int w = 2 * m;
-    for (int e = tid; e < m * w; e += nt) {
-        const int r = e / w, c = e % w;
-        W[e] = c < m ? A[r * m + c] : (c - m == r ? 1.0 : 0.0);
+// w[r][c] <- w[r][c] - col[r] prow[c] for the block's rows that keep(r) takes and columns c0 <= c < m;
+// seen(value, r, c) gets every new value.  Warps take rows, and parts of a row where there are more warps
+// than rows.
+template <class Keep, class Seen>
+__device__ __forceinline__ void rank_one(const Rows& a, int c0, Keep keep, Seen seen) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    if (a.R < 1) return;
+    const int parts = a.R < nw ? nw / a.R : 1;
+    const int part = a.R < nw ? warp / a.R : 0;
+    if (part >= parts) return;
+    for (int r = a.R < nw ? warp % a.R : warp; r < a.R; r += nw) {
+        if (!keep(r)) continue;
+        const double l = a.col[r];
+        double* w = a.w + (size_t)r * a.m;
+        for (int c = c0 + part * 32 + lane; c < a.m; c += parts * 32) {
+            const double v = fma(-l, a.prow[c], w[c]);
+            w[c] = v;
+            seen(v, r, c);
+        }
     }
+}
+
+// NR rows of C = B A^-1 (chunk: NR rows of B, scaled): a thread per column, k in order.
+template <int NR, class Put>
+__device__ __forceinline__ void product_rows(const double* chunk, const double* Ai, int m, Put put) {
+    for (int c = threadIdx.x; c < m; c += blockDim.x) {
+        double s[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) s[r] = 0.0;
+#pragma unroll 8
+        for (int k = 0; k < m; ++k) {
+            const double ai = __ldcg(Ai + (size_t)k * m + c);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) s[r] = fma(chunk[r * m + k], ai, s[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < NR; ++r) put(s[r], r, c);
+    }
+}
+
+// Inverse of the m x m matrix whose row j is load(j, c), in place with partial pivoting; its row at
+// position q goes to Ai[q][.], scaled by scale(q).  False: a zero (or no finite) pivot, or a wait that
+// gave up (then *err is set).  orig: shared [m].
+template <class Load, class Scale>
+__device__ bool invert_rows(Exchange& x, Rows& a, int* orig, double* Ai, int* status, Load load, Scale scale) {
+    const int m = a.m, tid = threadIdx.x, nt = blockDim.x;
+    for (int e = tid; e < a.R * m; e += nt) a.w[e] = load(a.first + e / m, e % m);
+    for (int r = tid; r < a.R; r += nt) a.pos[r] = a.first + r;
     __syncthreads();
     for (int k = 0; k < m; ++k) {
-        double best = -1.0;
-        int bi = 0x7fffffff;
-        for (int r = k + tid; r < m; r += nt) {
-            const double v = fabs(W[r * w + k]);
-            if (v > best || (v == best && r < bi)) {
-                best = v;
-                bi = r;
-            }
+        double v;
+        unsigned p;
+        const int br = pivot_candidate(a, k, &v, &p);
+        if (br >= 0) {
+            double* out = x.mine();
+            for (int c = tid; c < m; c += nt) put_row(out + c, a.w[(size_t)br * m + c]);
+            if (tid == 0) put_row(out + m, (double)(a.first + br));
         }
-        const ArgMax p = block_argmax(best, bi, sbuf);
-        if (p.v == 0.0) return false;
-        if (p.idx != k)
-            for (int c = tid; c < w; c += nt) {
-                const double t = W[k * w + c];
-                W[k * w + c] = W[p.idx * w + c];
-                W[p.idx * w + c] = t;
-            }
-        __syncthreads();
-        const double inv = 1.0 / W[k * w + k];
-        __syncthreads();  // every thread has read the pivot before row k is scaled
-        for (int c = tid; c < w; c += nt) W[k * w + c] *= inv;
-        __syncthreads();
-        for (int e = tid; e < m * w; e += nt) {
-            const int r = e / w, c = e % w;
-            if (r != k) {
-                const double f = W[r * w + k];
-                if (c != k) W[e] -= f * W[k * w + c];
-            }
+        if (!x.round(v, p)) return false;
+        const int q = x.winner(&v, &p);
+        if (q < 0 || v == 0.0) {
+            if (tid == 0 && blockIdx.x == 0) atomicOr(status, kErrSingular);
+            return false;
+        }
+        const double* in = x.slot(q);
+        const double inv = 1.0 / get_row(in + k);
+        for (int c = tid; c < m; c += nt) a.prow[c] = c == k ? inv : get_row(in + c) * inv;
+        if (tid == 0) orig[k] = (int)get_row(in + m);
+        for (int r = tid; r < a.R; r += nt) {
+            if (a.pos[r] == (int)p)
+                a.pos[r] = k;
+            else if (a.pos[r] == k)
+                a.pos[r] = (int)p;
+            a.col[r] = a.w[(size_t)r * m + k];
+            a.w[(size_t)r * m + k] = 0.0;  // the eliminated column; the new column of the inverse grows here
         }
         __syncthreads();
-        for (int r = tid; r < m; r += nt)
-            if (r != k) W[r * w + k] = 0.0;
+        rank_one(a, 0, [&](int r) { return a.pos[r] != k; }, [](double, int, int) {});
+        if (q == (int)blockIdx.x)
+            for (int c = tid; c < m; c += nt) a.w[(size_t)br * m + c] = a.prow[c];
         __syncthreads();
     }
-    for (int e = tid; e < m * m; e += nt) Ai[e] = W[(e / m) * w + m + (e % m)];
-    __syncthreads();
-    (void)s_flag;
+    for (int e = tid; e < a.R * m; e += nt) {
+        const int row = a.pos[e / m];
+        Ai[(size_t)row * m + orig[e % m]] = a.w[e] * scale(row);
+    }
     return true;
 }
 
-__global__ void __launch_bounds__(kMvThreads) k_maxvol(int n, int m, const double* Braw, double* Bs, double* D,
-                                                       double* W, int* perm, int* sel, double* A, double* Ai, double* C,
-                                                       double tol, int max_iter, int* status, int* swaps_out,
-                                                       double* gmax_out, int start_given) {
-    __shared__ ArgMax sbuf[33];
-    __shared__ int s_flag;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    // 0. column equilibration: gamma and the selection do not change under B -> B D
+// Shared memory of the cooperative kernels, in order: exchange keys and payloads [G], warps' candidates,
+// (G == 1: records and slots), prow [m], orig [m], then for k_maxvol D [m], sel [m] and a chunk of B, and
+// the block's rows with their positions and column when those fit.
+struct Layout {
+    int G, R, br;          // blocks, rows of a block at most, rows of B in a chunk
+    bool rows_in, col_in;  // rows, positions and column in shared memory
+    size_t bytes;
+};
+constexpr size_t kMvSharedMost = 200 * 1024;
+
+__host__ __device__ inline int mv_rows(int n, int G) { return (n + G - 1) / G; }
+
+inline Layout mv_layout(int n, int m, int G, bool full) {
+    Layout l{};
+    l.G = G;
+    l.R = mv_rows(n > m ? n : m, G);
+    l.br = full ? (m <= 1024 ? 8 : 1) : 0;
+    size_t b = 16 * (size_t)((G + 1) / 2 * 2) + 32 * 16 + (G == 1 ? 8 * (size_t)(4 + 2 * (m + 1)) : 0);
+    b += 8 * (size_t)m + 8 * (size_t)m;                                     // prow, orig (8-byte slots)
+    if (full) b += 8 * (size_t)m + 8 * (size_t)m + 8 * (size_t)m * l.br;    // D, sel, chunk
+    l.col_in = b + 16 * (size_t)l.R <= kMvSharedMost;
+    if (l.col_in) b += 16 * (size_t)l.R;
+    l.rows_in = b + 8 * (size_t)l.R * m <= kMvSharedMost;
+    if (l.rows_in) b += 8 * (size_t)l.R * m;
+    l.bytes = b;
+    return l;
+}
+
+struct Carve {
+    unsigned char* p;
+    template <class T>
+    __device__ T* take(size_t count) {  // 8-byte slots
+        T* r = reinterpret_cast<T*>(p);
+        p += 8 * ((count * sizeof(T) + 7) / 8);
+        return r;
+    }
+};
+
+__device__ void carve_common(Carve& s, Exchange& x, Rows& a, int** orig) {
+    x.s_key = s.take<unsigned long long>(x.G);
+    x.s_pay = s.take<unsigned>(x.G);
+    a.s_v = s.take<unsigned long long>(32);
+    a.s_p = s.take<unsigned>(32);
+    a.s_r = s.take<int>(32);
+    if (x.G == 1) {
+        x.rec = s.take<unsigned long long>(4);
+        x.slots = s.take<double>(2 * (x.m + 1));
+        if (threadIdx.x < 4) x.rec[threadIdx.x] = 0;
+    }
+    a.prow = s.take<double>(x.m);
+    *orig = s.take<int>(2 * x.m);
+}
+
+struct MaxvolArgs {
+    int n, m, G, br;
+    bool rows_in, col_in;
+    const double* B;           // [n][m]
+    double* rows;              // [max(n, m)][m] when the rows do not fit in shared memory
+    double* col;               // [max(n, m)], likewise
+    int* pos;                  // [n], likewise
+    unsigned long long* rec;   // [2][G][2], zero at the start (G > 1)
+    int* sel;                  // [m]
+    double* A;                 // [m][m]; holds the exchange's rows until the end
+    double* Ai;                // [m][m]
+    double tol;
+    int max_iter, start_given;
+    int *status, *swaps;
+    double* gmax;
+};
+
+__global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int tid = threadIdx.x, nt = blockDim.x, n = g.n, m = g.m;
+    Carve sh{smem};
+    Exchange x{g.rec, g.A, g.G, m, 0u, g.status, nullptr, nullptr};
+    Rows a{};
+    int* orig;
+    carve_common(sh, x, a, &orig);
+    double* D = sh.take<double>(m);
+    int* sel = sh.take<int>(2 * m);
+    double* chunk = sh.take<double>((size_t)m * g.br);
+    const int Rn = mv_rows(n, g.G), Rm = mv_rows(m, g.G), Rmost = Rn > Rm ? Rn : Rm;
+    double* col_s = g.col_in ? sh.take<double>(Rmost) : nullptr;
+    int* pos_s = g.col_in ? sh.take<int>(2 * Rmost) : nullptr;
+    double* rows_s = g.rows_in ? sh.take<double>((size_t)Rmost * m) : nullptr;
+    a.m = m;
+    auto own = [&](int total, int each) {  // the block's share of `total` rows
+        a.first = min(total, (int)blockIdx.x * each);
+        a.R = min(total, a.first + each) - a.first;
+        a.w = g.rows_in ? rows_s : g.rows + (size_t)a.first * m;
+        a.col = g.col_in ? col_s : g.col + a.first;
+        a.pos = g.col_in ? pos_s : g.pos + a.first;
+    };
+    own(n, Rn);
+    __syncthreads();
+    // 0. column equilibration: the largest |column| of the block's rows, then of all blocks'
     for (int c = tid; c < m; c += nt) {
         double mx = 0.0;
-        for (int r = 0; r < n; ++r) mx = fmax(mx, fabs(Braw[(size_t)r * m + c]));
+        for (int r = 0; r < a.R; ++r) mx = fmax(mx, fabs(g.B[(size_t)(a.first + r) * m + c]));
+        put_row(x.mine() + c, mx);
+    }
+    if (!x.round(0.0, kNone)) return;
+    bool zero = false;
+    for (int c = tid; c < m; c += nt) {
+        double mx = 0.0;
+#pragma unroll 8
+        for (int q = 0; q < g.G; ++q) mx = fmax(mx, get_row(x.slot(q) + c));
         D[c] = mx > 0.0 ? 1.0 / mx : 0.0;
+        zero = zero || D[c] == 0.0;
     }
-    __syncthreads();
-    for (int c = 0; c < m; ++c)
-        if (D[c] == 0.0) {
-            if (tid == 0) *status = kErrSingular;
-            return;
-        }
-    for (int e = tid; e < n * m; e += nt) Bs[e] = Braw[e] * D[e % m];
-    __syncthreads();
-    const double* B = Bs;
-    if (start_given) {  // select-add: start from the first m rows (the current active set)
-        for (int j = tid; j < m; j += nt) sel[j] = j;
-        __syncthreads();
-        goto have_start;
-    }
-    // 1. pivot rows of LU with partial pivoting (row interchanges tracked in perm)
-    for (int e = tid; e < n * m; e += nt) W[e] = B[e];
-    for (int r = tid; r < n; r += nt) perm[r] = r;
-    __syncthreads();
-    for (int k = 0; k < m; ++k) {
-        double best = -1.0;
-        int bi = 0x7fffffff;
-        for (int r = k + tid; r < n; r += nt) {
-            const double v = fabs(W[perm[r] * m + k]);
-            if (v > best || (v == best && r < bi)) {
-                best = v;
-                bi = r;
-            }
-        }
-        const ArgMax p = block_argmax(best, bi, sbuf);
-        if (p.v == 0.0) {
-            if (tid == 0) *status = kErrSingular;
-            return;
-        }
-        if (tid == 0 && p.idx != k) {
-            const int t = perm[k];
-            perm[k] = perm[p.idx];
-            perm[p.idx] = t;
-        }
-        __syncthreads();
-        const int pk = perm[k];
-        const double piv = W[pk * m + k];
-        const int rows = n - k - 1, cols = m - k - 1;
-        for (int e = tid; e < rows * (cols + 1); e += nt) {
-            const int rr = k + 1 + e / (cols + 1), c = k + e % (cols + 1);
-            const int pr = perm[rr];
-            const double l = W[pr * m + k] / piv;
-            if (c > k) W[pr * m + c] -= l * W[pk * m + c];
-        }
-        __syncthreads();
-        // the multipliers are no longer needed in column k (kept implicit)
-    }
-    for (int j = tid; j < m; j += nt) sel[j] = perm[j];
-    __syncthreads();
-have_start:
-    // 2. A and its inverse
-    for (int e = tid; e < m * m; e += nt) A[e] = B[sel[e / m] * m + (e % m)];
-    __syncthreads();
-    if (!gauss_jordan(A, Ai, W, m, sbuf, &s_flag)) {
-        if (tid == 0) *status = kErrSingular;
+    if (__syncthreads_or(zero)) {
+        if (tid == 0 && blockIdx.x == 0) atomicOr(g.status, kErrSingular);
         return;
     }
-    // 3. C = B A^-1
-    for (int e = tid; e < n * m; e += nt) {
-        const int r = e / m, c = e % m;
-        double s = 0.0;
-        for (int k = 0; k < m; ++k) s += B[r * m + k] * Ai[k * m + c];
-        C[e] = s;
+    if (g.start_given) {  // select-add: start from the first m rows (the current active set)
+        for (int j = tid; j < m; j += nt) sel[j] = j;
+    } else {
+        // 1. pivot rows of LU with partial pivoting
+        for (int e = tid; e < a.R * m; e += nt) a.w[e] = g.B[(size_t)a.first * m + e] * D[e % m];
+        for (int r = tid; r < a.R; r += nt) a.pos[r] = a.first + r;
+        __syncthreads();
+        for (int k = 0; k < m; ++k) {
+            double v;
+            unsigned p;
+            const int br = pivot_candidate(a, k, &v, &p);
+            if (br >= 0) {
+                double* out = x.mine();
+                for (int c = k + tid; c < m; c += nt) put_row(out + c, a.w[(size_t)br * m + c]);
+                if (tid == 0) put_row(out + m, (double)(a.first + br));
+            }
+            if (!x.round(v, p)) return;
+            const int q = x.winner(&v, &p);
+            if (q < 0 || v == 0.0) {
+                if (tid == 0 && blockIdx.x == 0) atomicOr(g.status, kErrSingular);
+                return;
+            }
+            const double* in = x.slot(q);
+            const double piv = get_row(in + k);
+            for (int c = k + 1 + tid; c < m; c += nt) a.prow[c] = get_row(in + c);
+            if (tid == 0) sel[k] = (int)get_row(in + m);
+            for (int r = tid; r < a.R; r += nt) {
+                if (a.pos[r] == (int)p)
+                    a.pos[r] = k;
+                else if (a.pos[r] == k)
+                    a.pos[r] = (int)p;
+                a.col[r] = a.w[(size_t)r * m + k] / piv;
+            }
+            __syncthreads();
+            rank_one(a, k + 1, [&](int r) { return a.pos[r] > k; }, [](double, int, int) {});
+            __syncthreads();
+        }
     }
     __syncthreads();
+    // 2. the inverse of A = B[sel]
+    const auto load = [&](int j, int c) { return g.B[(size_t)sel[j] * m + c] * D[c]; };
+    own(m, Rm);
+    if (!invert_rows(x, a, orig, g.Ai, g.status, load, [](int) { return 1.0; })) return;
+    if (!x.round(0.0, kNone)) return;  // every block's rows of A^-1 are written
+    // 3. C = B A^-1 for the block's rows, a few rows at a time (a thread per column)
+    own(n, Rn);
+    double best = -1.0;
+    int at = 0;
+    auto track = [&](double v, int e) {
+        v = fabs(v);
+        if (v > best || (v == best && e < at)) {
+            best = v;
+            at = e;
+        }
+    };
+    for (int r0 = 0; r0 < a.R; r0 += g.br) {
+        const int nr = min(g.br, a.R - r0);
+        __syncthreads();
+        for (int e = tid; e < nr * m; e += nt) chunk[e] = g.B[(size_t)(a.first + r0) * m + e] * D[e % m];
+        __syncthreads();
+        const auto put = [&](double v, int r, int c) {
+            a.w[(size_t)(r0 + r) * m + c] = v;
+            track(v, (a.first + r0 + r) * m + c);
+        };
+        switch (nr) {
+            case 8: product_rows<8>(chunk, g.Ai, m, put); break;
+            case 7: product_rows<7>(chunk, g.Ai, m, put); break;
+            case 6: product_rows<6>(chunk, g.Ai, m, put); break;
+            case 5: product_rows<5>(chunk, g.Ai, m, put); break;
+            case 4: product_rows<4>(chunk, g.Ai, m, put); break;
+            case 3: product_rows<3>(chunk, g.Ai, m, put); break;
+            case 2: product_rows<2>(chunk, g.Ai, m, put); break;
+            default: product_rows<1>(chunk, g.Ai, m, put); break;
+        }
+    }
     // 4. swaps
     int swaps = 0;
-    double g = 0.0;
-    for (int it = 0; it <= max_iter; ++it) {
-        double best = -1.0;
-        int bi = 0x7fffffff;
-        for (int e = tid; e < n * m; e += nt) {
-            const double v = fabs(C[e]);
-            if (v > best || (v == best && e < bi)) {
+    double gm = -1.0;
+    for (int it = 0; it <= g.max_iter; ++it) {
+        // the block's largest |C| (ties: the smallest element)
+        for (int o = 16; o > 0; o >>= 1) {
+            const double v = __shfl_xor_sync(0xffffffffu, best, o);
+            const int e = __shfl_xor_sync(0xffffffffu, at, o);
+            if (v > best || (v == best && e < at)) {
                 best = v;
-                bi = e;
+                at = e;
             }
         }
-        const ArgMax p = block_argmax(best, bi, sbuf);
-        g = p.v;
-        if (p.v <= 1.0 + tol) break;
-        if (it == max_iter) {
-            if (tid == 0) *status = kErrTimeout;
+        __syncthreads();
+        if ((tid & 31) == 0) {
+            a.s_v[tid >> 5] = (unsigned long long)__double_as_longlong(best);
+            a.s_r[tid >> 5] = at;
+        }
+        __syncthreads();
+        for (int q = 0; q < nt >> 5; ++q) {
+            const double v = __longlong_as_double((long long)a.s_v[q]);
+            if (v > best || (v == best && a.s_r[q] < at)) {
+                best = v;
+                at = a.s_r[q];
+            }
+        }
+        if (best >= 0.0) {
+            double* out = x.mine();
+            const double* row = a.w + (size_t)(at / m - a.first) * m;
+            for (int c = tid; c < m; c += nt) put_row(out + c, row[c]);
+        }
+        if (!x.round(best, best >= 0.0 ? (unsigned)at : kNone)) return;
+        unsigned e;
+        double v;
+        const int q = x.winner(&v, &e);
+        gm = q < 0 ? -1.0 : v;
+        if (gm <= 1.0 + g.tol) break;
+        if (it == g.max_iter) {
+            if (tid == 0 && blockIdx.x == 0) atomicOr(g.status, kErrTimeout);
             break;
         }
-        const int k = p.idx / m, j = p.idx % m;
-        const double ckj = C[p.idx];
-        // Ai <- Ai - Ai[:,j] (C[k,:] - e_j) / ckj ; C <- C - C[:,j] (C[k,:] - e_j) / ckj
-        // (read the column and the row before writing: stage them in W)
-        for (int t = tid; t < m; t += nt) {
-            W[t] = C[k * m + t] - (t == j ? 1.0 : 0.0);  // row
-            W[m + t] = Ai[t * m + j];                     // column of Ai
-        }
-        for (int r = tid; r < n; r += nt) W[2 * m + r] = C[r * m + j];
+        const int j = (int)e % m;
+        const double* in = x.slot(q);
+        const double ckj = get_row(in + j);
+        for (int c = tid; c < m; c += nt) a.prow[c] = get_row(in + c) - (c == j ? 1.0 : 0.0);
+        for (int r = tid; r < a.R; r += nt) a.col[r] = a.w[(size_t)r * m + j] / ckj;
+        if (tid == 0) sel[j] = (int)e / m;
         __syncthreads();
-        for (int e = tid; e < m * m; e += nt) Ai[e] -= W[m + e / m] * W[e % m] / ckj;
-        for (int e = tid; e < n * m; e += nt) C[e] -= W[2 * m + e / m] * W[e % m] / ckj;
-        if (tid == 0) sel[j] = k;
-        __syncthreads();
+        best = -1.0;
+        at = 0;
+        rank_one(a, 0, [](int) { return true; }, [&](double v, int r, int c) { track(v, (a.first + r) * m + c); });
         ++swaps;
     }
-    // final A (unscaled rows of B) and A^-1 = D (A D)^-1, the inverse recomputed from scratch
-    for (int e = tid; e < m * m; e += nt) A[e] = B[sel[e / m] * m + (e % m)];
     __syncthreads();
-    if (!gauss_jordan(A, Ai, W, m, sbuf, &s_flag)) {
-        if (tid == 0) *status = kErrSingular;
-        return;
-    }
-    for (int e = tid; e < m * m; e += nt) {
-        Ai[e] *= D[e / m];
-        A[e] = Braw[(size_t)sel[e / m] * m + (e % m)];
-    }
-    __syncthreads();
-    if (tid == 0) {
-        *swaps_out = swaps;
-        *gmax_out = g;
+    // A^-1 = D (A D)^-1, computed from scratch, and the unscaled A (over the exchange's rows: after
+    // every block has read the last of them)
+    own(m, Rm);
+    if (!invert_rows(x, a, orig, g.Ai, g.status, load, [&](int row) { return D[row]; })) return;
+    if (!x.round(0.0, kNone)) return;
+    for (int e = tid; e < a.R * m; e += nt)
+        g.A[(size_t)a.first * m + e] = g.B[(size_t)sel[a.first + e / m] * m + e % m];
+    if (blockIdx.x == 0) {
+        for (int j = tid; j < m; j += nt) g.sel[j] = sel[j];
+        if (tid == 0) {
+            *g.swaps = swaps;
+            *g.gmax = gm;
+        }
     }
 }
 
@@ -305,27 +588,89 @@ __global__ void __launch_bounds__(256) k_grade(int n, int m, const T* __restrict
     }
 }
 
-__global__ void __launch_bounds__(kMvThreads) k_invert(int m, const double* A, double* Ai, double* W, int* status) {
-    __shared__ ArgMax sbuf[33];
-    __shared__ int s_flag;
-    if (!gauss_jordan(A, Ai, W, m, sbuf, &s_flag) && threadIdx.x == 0) *status = kErrSingular;
+struct InvertArgs {
+    int m, G;
+    bool rows_in, col_in;
+    const double* A;
+    double* Ai;
+    double* rows;             // [m][m] when the rows do not fit in shared memory
+    double* col;              // (col_in is always set for m rows)
+    double* slots;            // [2][G][m + 1]
+    unsigned long long* rec;  // [2][G][2], zero at the start
+    int* status;
+};
+
+__global__ void __launch_bounds__(kMvThreads) k_invert(const InvertArgs g) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int m = g.m, R = mv_rows(m, g.G);
+    Carve sh{smem};
+    Exchange x{g.rec, g.slots, g.G, m, 0u, g.status, nullptr, nullptr};
+    Rows a{};
+    int* orig;
+    carve_common(sh, x, a, &orig);
+    a.m = m;
+    a.first = min(m, (int)blockIdx.x * R);
+    a.R = min(m, a.first + R) - a.first;
+    a.col = sh.take<double>(R);
+    a.pos = sh.take<int>(2 * R);
+    a.w = g.rows_in ? sh.take<double>((size_t)R * m) : g.rows + (size_t)a.first * m;
+    __syncthreads();
+    invert_rows(x, a, orig, g.Ai, g.status, [&](int j, int c) { return g.A[(size_t)j * m + c]; },
+                [](int) { return 1.0; });
+}
+
+int mv_sm_count() {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 0 ? n : 1;
+}
+
+// Blocks of a cooperative kernel: as many as have rows to own and room for their exchange rows, one per
+// SM at most (the exchange costs the same for few and for many, the rows of a block set the step's FMAs).
+int mv_blocks(int m, size_t slot_doubles) {
+    const long by_slots = (long)(slot_doubles / (2 * (size_t)(m + 1)));
+    return (int)std::max(1l, std::min({(long)mv_sm_count(), (long)m / 2, by_slots}));
 }
 
 }  // namespace
 
 // The launchers return the number of kernels launched, or -1 if the launch itself failed (the
 // error is taken off cudaGetLastError, so the caller reports it instead of reading stale results).
+// W: 2 m^2 doubles.
 int launch_invert(int m, const double* A, double* Ai, double* W, int* status, cudaStream_t st) {
-    k_invert<<<1, kMvThreads, 0, st>>>(m, A, Ai, W, status);
-    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+    // W = [rows m^2 | records 4 G | slots 2 G (m + 1)]
+    const size_t mm = (size_t)m * m;
+    const int G = mv_blocks(m, mm > 4 * (size_t)(m / 2) ? mm - 4 * (size_t)(m / 2) : 0);
+    const Layout l = mv_layout(m, m, G, false);
+    InvertArgs g{m, G, l.rows_in, l.col_in, A, Ai, W, nullptr, W + mm + 4 * (size_t)G,
+                 reinterpret_cast<unsigned long long*>(W + mm), status};
+    if (!l.col_in || l.bytes > kMvSharedMost) return -1;  // not reachable for the widths of a model
+    if (G > 1 && cudaMemsetAsync(g.rec, 0, 32 * (size_t)G, st) != cudaSuccess) return -1;
+    if (cudaFuncSetAttribute(k_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMvSharedMost) != cudaSuccess)
+        return -1;
+    void* args[] = {&g};
+    return cudaLaunchCooperativeKernel((void*)k_invert, dim3(G), dim3(kMvThreads), args, l.bytes, st) == cudaSuccess
+               ? 1 : -1;
 }
 
-int launch_maxvol(int n, int m, const double* B, double* Bs, double* D, double* W, int* perm, int* sel, double* A,
-                  double* Ai, double* C, double tol, int max_iter, int* status, int* swaps, double* gmax,
-                  cudaStream_t st, int start_given) {
-    k_maxvol<<<1, kMvThreads, 0, st>>>(n, m, B, Bs, D, W, perm, sel, A, Ai, C, tol, max_iter, status, swaps, gmax,
-                                       start_given);
-    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+// W: max(n m, 2 m^2) + 2 m + n doubles, pos: n ints.
+int launch_maxvol(int n, int m, const double* B, double* W, int* pos, int* sel, double* A, double* Ai, double tol,
+                  int max_iter, int* status, int* swaps, double* gmax, cudaStream_t st, int start_given) {
+    const size_t nm = (size_t)n * m, mm = (size_t)m * m;
+    const int G = mv_blocks(m, mm);  // the exchange's rows lie in A until the end; records: 4 G <= 2 m doubles
+    const Layout l = mv_layout(n, m, G, true);
+    if (l.bytes > kMvSharedMost) return -1;  // not reachable for the widths of a model
+    double* tail = W + std::max(nm, 2 * mm);
+    MaxvolArgs g{n, m, G, l.br, l.rows_in, l.col_in, B, W, tail + 2 * (size_t)m, pos,
+                 reinterpret_cast<unsigned long long*>(tail), sel, A, Ai, tol, max_iter, start_given, status, swaps,
+                 gmax};
+    if (G > 1 && cudaMemsetAsync(g.rec, 0, 32 * (size_t)G, st) != cudaSuccess) return -1;
+    if (cudaFuncSetAttribute(k_maxvol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMvSharedMost) != cudaSuccess)
+        return -1;
+    void* args[] = {&g};
+    return cudaLaunchCooperativeKernel((void*)k_maxvol, dim3(G), dim3(kMvThreads), args, l.bytes, st) == cudaSuccess
+               ? 1 : -1;
 }
 
 __global__ void k_gather_columns(int rows, int w_in, const double* in, int w_out, const int* cols, double* out) {
@@ -405,8 +750,9 @@ extern "C" mtp_status mtp_select_active_set_noalloc(int n_rows, int m, const dou
                                                     double* a_inv, int* n_swaps, void* stream) {
     using namespace mtp;
     if (m < 1 || n_rows < m || !b_rows || !selected) return MTP_EINVAL;
-    // layout inside the fixed array (in doubles): Bs, C [n m]; W [max(n m, 2 m m) + 2 m + n];
-    // D [m]; A, A^-1 [m m]; then ints: perm [n], sel [m], status, swaps; then gmax.
+    // the documented limit (2 n m + m doubles of it are unused); layout inside the fixed array (in
+    // doubles): W [max(n m, 2 m m) + 2 m + n]; A, A^-1 [m m]; then ints: pos [n], sel [m], status,
+    // swaps; then gmax.
     const size_t nm = (size_t)n_rows * m, mm = (size_t)m * m;
     const size_t w = (nm > 2 * mm ? nm : 2 * mm) + 2 * (size_t)m + n_rows;
     const size_t ints = (size_t)n_rows + m + 2;
@@ -414,20 +760,17 @@ extern "C" mtp_status mtp_select_active_set_noalloc(int n_rows, int m, const dou
     if (need > kNoAllocScratchDoubles) return MTP_EINVAL;  // larger than the fixed scratch array
     double* base = nullptr;
     if (noalloc_scratch(&base) != cudaSuccess) return MTP_ECUDA;
-    double* Bs = base;
-    double* C = Bs + nm;
-    double* W = C + nm;
-    double* D = W + w;
-    double* A = D + m;
+    double* W = base;
+    double* A = W + w;
     double* Ai = A + mm;
-    int* perm = reinterpret_cast<int*>(Ai + mm);
-    int* sel = perm + n_rows;
+    int* pos = reinterpret_cast<int*>(Ai + mm);
+    int* sel = pos + n_rows;
     int* status = sel + m;
     int* swaps = status + 1;
     double* gmax = reinterpret_cast<double*>(base + (need - 1));
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaMemsetAsync(status, 0, 2 * sizeof(int), st) != cudaSuccess) return MTP_ECUDA;
-    if (launch_maxvol(n_rows, m, b_rows, Bs, D, W, perm, sel, A, Ai, C, 1e-3, 100 * m, status, swaps, gmax, st, 0) < 0)
+    if (launch_maxvol(n_rows, m, b_rows, W, pos, sel, A, Ai, 1e-3, 100 * m, status, swaps, gmax, st, 0) < 0)
         return MTP_ECUDA;
     int h[2] = {0, 0};
     if (cudaMemcpyAsync(h, status, sizeof h, cudaMemcpyDeviceToHost, st) != cudaSuccess) return MTP_ECUDA;
