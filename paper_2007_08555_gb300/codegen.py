@@ -780,9 +780,9 @@ def emit_slice_functions(prog: Program, slc, tag, slot_begin=None):
             out.append(f"    acc[{t}] += df[{mu}] * rdu * {mv} + f[{mu}] * ({g});")
         out.append("  }")
         # P_mu = sum adj mono and its tangent Pd_mu = sum adjt mono + adj (grad mono . u), with the
-        # adjoint values read from the tile layout (stride 32) starting at this slice
-        out.append("  template <class T> static __device__ __forceinline__ void pdot(const T x, const T y, const T z, "
-                   "const T* __restrict__ adjp, const T* __restrict__ adjtp, const T ux, const T uy, const T uz, "
+        # adjoint values of component t of this slice at [32 t] (a pointer, or an accessor)
+        out.append("  template <class T, class A, class B> static __device__ __forceinline__ void pdot(const T x, const T y, "
+                   "const T z, const A adjp, const B adjtp, const T ux, const T uy, const T uz, "
                    "T* __restrict__ P, T* __restrict__ Pd) {")
         out += ["    " + l for l in _mono_code(need, "T")]
         for t, ci in enumerate(comps):

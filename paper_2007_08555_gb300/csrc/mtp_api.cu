@@ -211,6 +211,9 @@ int choose_tpa(int n_atoms, int n_sm, int per_sm) {
     return 8;
 }
 
+// elements of an atom's row of dV/dM (whole 4-vectors of components)
+size_t adj_row(const mtp_model* M) { return (size_t)(M->C + 3) / 4 * 4; }
+
 template <class T>
 mtp_status fill_ctx(mtp_model* M, int K, int n, const int* cfg_off, const int* types, double* energy,
                     double* forces, double* virial, double* site, double* brows, double* batoms, cudaStream_t st,
@@ -222,7 +225,7 @@ mtp_status fill_ctx(mtp_model* M, int K, int n, const int* cfg_off, const int* t
     if (parts && (M->aslots.reserve(tiles * M->ops->contract_slots * 32 * sizeof(T) + 16) ||
                   M->epart.reserve(N * M->ops->contract_parts * sizeof(T) + 16)))
         return MTP_ENOMEM;
-    if (M->mom.reserve(tiles * M->C * 32 * sizeof(T)) || M->adjm.reserve(tiles * M->C * 32 * sizeof(T)) ||
+    if (M->mom.reserve(tiles * M->C * 32 * sizeof(T)) || M->adjm.reserve(tiles * 32 * adj_row(M) * sizeof(T)) ||
         M->gx.reserve(N * cap * sizeof(mtp::Vec4<T>)))
         return MTP_ENOMEM;
     if (n == 0) {  // otherwise the moments kernel clears them
@@ -631,7 +634,7 @@ mtp_status run_param_grad(mtp_model* M, int K, int n, const int* off, const int*
         M->g_virial.reserve(72 * (size_t)K + 8) || M->g_D.reserve(3 * N * sizeof(T) + 8) ||
         M->g_eps.reserve(9 * (size_t)K * sizeof(T) + 8) || M->g_ew.reserve(8 * (size_t)K + 8) ||
         M->g_momt.reserve(((N + 31) / 32) * M->C * 32 * sizeof(T)) ||
-        M->g_adjmt.reserve(((N + 31) / 32) * M->C * 32 * sizeof(T)))
+        M->g_adjmt.reserve(((N + 31) / 32) * 32 * adj_row(M) * sizeof(T)))
         return MTP_ENOMEM;
     const bool dual_parts = sizeof(T) == 4 && M->ops->contract_parts > 0;  // float tangent contraction in parts
     if (dual_parts && (M->g_dslots.reserve(2 * ((N + 31) / 32) * M->ops->dual_slots * 32 * sizeof(T) + 16) ||
@@ -745,7 +748,7 @@ mtp_status run_jacobian(mtp_model* M, int K, int n, const int* off, const int* t
     if (M->g_energy.reserve(8 * (size_t)K + 8) || M->g_D.reserve(3 * N * sizeof(T) + 8) ||
         M->g_eps.reserve(9 * (size_t)K * sizeof(T) + 8) || M->g_ew.reserve(8 * (size_t)K + 8) ||
         M->g_momt.reserve(((N + 31) / 32) * M->C * 32 * sizeof(T)) ||
-        M->g_adjmt.reserve(((N + 31) / 32) * M->C * 32 * sizeof(T)) ||
+        M->g_adjmt.reserve(((N + 31) / 32) * 32 * adj_row(M) * sizeof(T)) ||
         M->g_brows.reserve(sizeof(double) * (size_t)K * m + 8) || M->g_batoms.reserve(sizeof(double) * N * m + 8) ||
         M->j_rows.reserve(sizeof(double) * (size_t)K * nc + 8) || M->g_out.reserve(sizeof(double) * (1 + m + nc) + 64))
         return MTP_ENOMEM;

@@ -73,7 +73,7 @@ struct EvalCtx {
     int tpa;              // threads per atom in the pair-gradient, gather and loss-gradient kernels (1, 2, 4 or 8)
     int tpa_m;            // threads per atom in the moments kernel
     T* mom;               // [ceil(n/32)][C][32] moment components (tile layout)
-    T* adjm;              // [ceil(n/32)][C][32] dV/dM
+    T* adjm;              // [ceil(n/32)][C][32] dV/dM; in the loss gradient [n][C padded to a multiple of 4]
     T* aslots;            // [ceil(n/32)][NSLOT][32] dV/dM shares of the contraction parts (float path)
     T* epart;             // [NPART][n] site-energy shares of the contraction parts (float path)
     Vec4<T>* g;           // [cap][n] dV_i/dr_ij (x, y, z, unused): one vector load per pair
@@ -89,7 +89,7 @@ struct EvalCtx {
     const T* geps;        // [n_cfg][9] eps_k = 2 s_s w_s (W_k - W_k^ref)
     const double* gew;    // [n_cfg] e_k = 2 s_e w_e (E_k - E_k^ref)
     T* momt;              // tangent of the moments along u (tile layout)
-    T* adjmt;             // tangent of dV/dM (tile layout)
+    T* adjmt;             // [n][C padded] tangent of dV/dM
     double* dxi;          // [M] accumulated dL/dxi
     T* dslots;            // [2][ceil(n/32)][NDSLOT][32] dV/dM and its tangent, per tangent-contraction part
     double* dxt;          // [ceil(n/32)][M] per-tile shares of dL/dxi from the tangent contraction

@@ -1288,6 +1288,10 @@ __device__ __forceinline__ void run_program_dual(const unsigned long long* __res
     }
 }
 
+// Elements of an atom's row of dV/dM (and of its tangent) as the loss gradient's k_dc reads them: the
+// components of one atom side by side, padded to whole 4-vectors.
+constexpr int kAdjRow = (G::C_ + 3) / 4 * 4;
+
 #if MTPGEN_HAS_PARTS
 // Tangent contraction of the loss gradient (float), split into NDPART generated parts like the
 // forward contraction: warp w runs part w / n_tiles for the 32 atoms of tile w % n_tiles.  Each part
@@ -1310,25 +1314,38 @@ __global__ void __launch_bounds__(128) k_contract_tan_parts(const EvalCtx<float>
     }
 }
 
-// dV/dM and its tangent = sums of their dual slots (slot order), one warp per (tile, component)
+// dV/dM and its tangent = sums of their dual slots (slot order), one warp per (tile, eight components),
+// written atom by atom for k_dc (eight components: one whole sector of an atom's row)
 __global__ void __launch_bounds__(128) k_dual_sum(const EvalCtx<float> a) {
-    constexpr int C = G::C_;
+    constexpr int C = G::C_, CP = kAdjRow;
+    constexpr int NG = (C + 7) / 8;
     const int lane = threadIdx.x & 31;
     const int n_tiles = (a.n_atoms + 31) >> 5;
     const size_t half = (size_t)n_tiles * G::NDSLOT_ * 32;
     const int warps = (gridDim.x * blockDim.x) >> 5;
-    for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_tiles * C; w += warps) {
-        const int tile = w / C, c = w - tile * C;
+    for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_tiles * NG; w += warps) {
+        const int tile = w / NG, c0 = (w - tile * NG) * 8;
         const float* sl = a.dslots + (size_t)tile * G::NDSLOT_ * 32 + lane;
-        const int s0 = ::MTP_GEN_NS::dslot_begin[c], s1 = ::MTP_GEN_NS::dslot_begin[c + 1];
-        float va = 0.f, vt = 0.f;
-        for (int s = s0; s < s1; ++s) {
-            va += sl[s * 32];
-            vt += sl[half + s * 32];
+        float va[8], vt[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            va[q] = vt[q] = 0.f;
+            if (c0 + q < C) {
+                const int s0 = ::MTP_GEN_NS::dslot_begin[c0 + q], s1 = ::MTP_GEN_NS::dslot_begin[c0 + q + 1];
+                for (int s = s0; s < s1; ++s) {
+                    va[q] += sl[s * 32];
+                    vt[q] += sl[half + s * 32];
+                }
+            }
         }
-        const size_t q = ((size_t)tile * C + c) * 32 + lane;
-        a.adjm[q] = va;
-        a.adjmt[q] = vt;
+        if (tile * 32 + lane >= a.n_atoms) continue;
+        const size_t o = (size_t)(tile * 32 + lane) * CP + c0;
+#pragma unroll
+        for (int q = 0; q < 8; q += 4)
+            if (c0 + q < CP) {
+                *reinterpret_cast<Vec4<float>*>(a.adjm + o + q) = Vec4<float>{va[q], va[q + 1], va[q + 2], va[q + 3]};
+                *reinterpret_cast<Vec4<float>*>(a.adjmt + o + q) = Vec4<float>{vt[q], vt[q + 1], vt[q + 2], vt[q + 3]};
+            }
     }
 }
 
@@ -1392,8 +1409,8 @@ __global__ void __launch_bounds__(128) k_contract_tan(const EvalCtx<T> a) {
         __syncwarp();
         run_program_dual<T, true>(a.adj_ops, a.adj_layer_end, a.adj_layers, sw, val, tan, adj, adt, lane);
         for (int c = lane; c < C; c += 32) {
-            a.adjm[tb + (size_t)c * 32] = adj[c];
-            a.adjmt[tb + (size_t)c * 32] = adt[c];
+            a.adjm[(size_t)i * kAdjRow + c] = adj[c];
+            a.adjmt[(size_t)i * kAdjRow + c] = adt[c];
         }
         __syncwarp();
     }
@@ -1402,108 +1419,209 @@ __global__ void __launch_bounds__(128) k_contract_tan(const EvalCtx<T> a) {
         if (lane + 32 * t < M) atomicAdd(&a.dxi[lane + 32 * t], dx[t]);
 }
 
+// dV/dM or its tangent of one atom in shared memory (vectors of four components, kDcAtoms atoms side by
+// side), as the generated pdot reads it: component t of a slice that begins at OFF is at [32 t]
+constexpr int kDcLanes = 8, kDcAtoms = 32 / kDcLanes;
+template <class T, int OFF>
+struct DcAdj {
+    SharedAdj<T, kDcAtoms, OFF> v;
+    __device__ __forceinline__ T operator[](int t32) const { return v[t32 >> 5]; }
+};
+
 template <class T, int S, int NS>
-__device__ __forceinline__ void pdot_all(const T* adjp, const T* adjtp, T x, T y, T z, T ux, T uy, T uz, T* P,
-                                         T* Pd) {
+__device__ __forceinline__ void pdot_all(const Vec4<T>* adj, const Vec4<T>* adjt, T x, T y, T z, T ux, T uy, T uz,
+                                         T* P, T* Pd) {
     if constexpr (S < NS) {
         using SL = typename SliceSel<T, S>::type;
-        SL::template pdot<T>(x, y, z, adjp + (size_t)SL::BEGIN * 32, adjtp + (size_t)SL::BEGIN * 32, ux, uy, uz, P,
-                             Pd);
-        pdot_all<T, S + 1, NS>(adjp, adjtp, x, y, z, ux, uy, uz, P, Pd);
+        SL::template pdot<T>(x, y, z, DcAdj<T, SL::BEGIN>{{adj}}, DcAdj<T, SL::BEGIN>{{adjt}}, ux, uy, uz, P, Pd);
+        pdot_all<T, S + 1, NS>(adj, adjt, x, y, z, ux, uy, uz, P, Pd);
     }
 }
 
-// dL/dc: thread group per atom, one pass per neighbour species (register accumulators, when the
-// radial basis size NQC is a compile-time constant; 0 = any size), then shared-memory and global
-// double atomics
-template <class T, int TPA, int NQC>
-__global__ void __launch_bounds__(128) k_dc(const EvalCtx<T> a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int NMU = G::NMU_;
-    const int nc = a.S * a.S * NMU * a.NQ;
-    double* dcs = reinterpret_cast<double*>(smem_raw);
-    for (int k = threadIdx.x; k < nc; k += blockDim.x) dcs[k] = 0.0;
-    __syncthreads();
-    const size_t n = (size_t)a.n_atoms;
-    const int NQ = NQC ? NQC : a.NQ;
+// dL/dc.  A block is one warp: eight lanes per atom, four atoms at a time out of the block's `chunk` of
+// consecutive atoms, taken in order of their species.  dV/dM and its tangent of the four atoms lie in
+// shared memory (2 C reads per pair and lane, as broadcast vectors); every lane adds its pairs' terms to
+// sums of its own in shared memory, one set per neighbour species, so that the lanes of a warp work on
+// pairs of different species at once; the sums are combined over an atom's lanes and go to the block's
+// double sums when the central species changes and at least every kDcRounds rounds of four atoms (no
+// longer a float sum than one thread over one atom's neighbours has), and from there to global memory
+// by one atomic per entry and block.  Bound: FP32 (or FP64) issue, 3 C multiply-adds and the monomials'
+// tangents per pair.  NQC: the radial basis size when it is known at compile time, 0 = any.
+// Against one thread per atom, a pass per neighbour species, dV/dM from global memory for every pair and
+// a double atomic per entry and atom: the gradient of 67 cells at lev_max 12 in double 3.01 -> 1.20 ms
+// (this kernel 1.94 -> 0.196), of 2048 cells at lev_max 20 in float 12.8 -> 8.67 ms.
+constexpr int kDcRounds = 8, kDcChunkMax = 128;
+
+template <class T>
+__host__ __device__ inline size_t dc_bytes(int S, int NQ) {
+    const int E = G::NMU_ * NQ, SE8 = (S * E + 7) / 8 * 8;
+    return sizeof(double) * (size_t)S * S * E + sizeof(T) * (size_t)SE8 * 32 + sizeof(T) * 2 * (size_t)kAdjRow * kDcAtoms +
+           sizeof(short) * kDcChunkMax + 32;
+}
+
+template <class T, int NQC>
+__global__ void __launch_bounds__(32) k_dc(const EvalCtx<T> a, const int chunk) {
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    constexpr int NMU = G::NMU_, NV = kAdjRow / 4;
+    const int S = a.S, NQ = NQC ? NQC : a.NQ, E = NMU * NQ, SE = S * E, SE8 = (SE + 7) / 8 * 8;
     constexpr int NQM = NQC ? NQC : kMaxRadial;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.n_atoms * TPA; g += gridDim.x * blockDim.x) {
-        const int i = g / TPA, sub = g % TPA;
-        const int zi = clamp_species(a.types[i], a.S);
-        const int cnt = a.count[i];
-        const int k = a.cfg_of[i];
-        const T ek = (T)a.gew[k];
-        T Di[3], E[9];
-        for (int q = 0; q < 3; ++q) Di[q] = a.gD[3 * (size_t)i + q];
-        for (int q = 0; q < 9; ++q) E[q] = a.geps[9 * (size_t)k + q];
-        const size_t tb = (size_t)(i >> 5) * G::C_ * 32 + (i & 31);
-        for (int zp = 0; zp < a.S; ++zp) {
-            T acc[NMU][NQM];
+    const int nc = S * SE, lane = threadIdx.x, sub = lane % kDcLanes, slot = lane / kDcLanes;
+    Vec4<T>* adjs = reinterpret_cast<Vec4<T>*>(smem_raw);  // [2][NV][kDcAtoms]
+    T* acc = reinterpret_cast<T*>(adjs + 2 * NV * kDcAtoms);  // [SE8] sums of each lane
+    double* bins = reinterpret_cast<double*>(acc + (size_t)SE8 * 32);  // [S][S][NMU][NQ]
+    short* list = reinterpret_cast<short*>(bins + nc);
+    // the lanes' sums side by side: as vectors of four entries when the radial size is known
+    auto at = [&](int e) { return NQC ? (e >> 2) * 128 + lane * 4 + (e & 3) : e * 32 + lane; };
+    for (int e = 0; e < SE8; ++e) acc[at(e)] = T(0);
+    for (int q = lane; q < nc; q += 32) bins[q] = 0.0;
+    const size_t n = (size_t)a.n_atoms;
+    int rounds = 0, cz = -1, ck = -1;  // rounds in the sums, the slot's central species and configuration
+
+    // the sums over each slot's lanes: lane `sub` ends up with entry 8 t + sub
+    auto flush = [&]() {
+        for (int t = 0; t < SE8; t += 8) {
+            T v[8];
 #pragma unroll
-            for (int mu = 0; mu < NMU; ++mu)
+            for (int q = 0; q < 8; ++q) {
+                v[q] = acc[at(t + q)];
+                acc[at(t + q)] = T(0);
+            }
 #pragma unroll
-                for (int b = 0; b < NQM; ++b) acc[mu][b] = T(0);
-            bool any = false;
-            for (int p = sub; p < cnt; p += TPA) {
-                const size_t idx = (size_t)p * n + i;
-                const PairRec<T> pq = a.pr[idx];
-                if ((pq.jz >> 24) != zp) continue;
-                any = true;
-                const int j = pq.jz & 0xffffff;
+            for (int o = 4; o > 0; o >>= 1) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (q < o) {
+                        const T keep = (sub & o) ? v[o + q] : v[q], give = (sub & o) ? v[q] : v[o + q];
+                        v[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+                }
+            }
+            const double d = (double)v[0];
+            const bool mine = cz >= 0 && t + sub < SE;
+            if (a.dc_rows) {  // Jacobian rows: to the configuration's row
+                if (mine) atomicAdd(&a.dc_rows[(size_t)ck * nc + (size_t)cz * SE + t + sub], d);
+            } else {
+#pragma unroll
+                for (int s = 0; s < kDcAtoms; ++s) {  // slots of one species share their entries
+                    if (mine && slot == s) bins[(size_t)cz * SE + t + sub] += d;
+                    __syncwarp();
+                }
+            }
+        }
+        __syncwarp();
+        rounds = 0;
+        cz = ck = -1;
+    };
+
+    for (int base = blockIdx.x * chunk; base < a.n_atoms; base += gridDim.x * chunk) {
+        // the chunk's atoms by species
+        int have = 0;
+        for (int z = 0; z < S; ++z) {
+            for (int o = 0; o < chunk; o += 32) {
+                const int q = o + lane;
+                const bool in = q < chunk && base + q < a.n_atoms && clamp_species(a.types[base + q], S) == z;
+                const unsigned m = __ballot_sync(0xffffffffu, in);
+                if (in) list[have + __popc(m & ((1u << lane) - 1))] = (short)q;
+                have += __popc(m);
+            }
+        }
+        __syncwarp();
+        for (int r = 0; r < have; r += kDcAtoms) {
+            const bool active = r + slot < have;
+            const int i = base + list[active ? r + slot : r];
+            const int zi = clamp_species(a.types[i], S), k = a.cfg_of[i];
+            const bool other = active && cz >= 0 && (zi != cz || (a.dc_rows && k != ck));
+            if (__any_sync(0xffffffffu, other) || rounds == kDcRounds) flush();
+            if (active) {
+                cz = zi;
+                ck = k;
+            }
+            ++rounds;
+            __syncwarp();
+            for (int v = sub; v < NV; v += kDcLanes) {
+                adjs[v * kDcAtoms + slot] = reinterpret_cast<const Vec4<T>*>(a.adjm + (size_t)i * kAdjRow)[v];
+                adjs[(NV + v) * kDcAtoms + slot] = reinterpret_cast<const Vec4<T>*>(a.adjmt + (size_t)i * kAdjRow)[v];
+            }
+            __syncwarp();
+            const int cnt = active ? a.count[i] : 0;
+            const T ek = (T)a.gew[k];
+            T Di[3], X[9];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) Di[q] = a.gD[3 * (size_t)i + q];
+#pragma unroll
+            for (int q = 0; q < 9; ++q) X[q] = a.geps[9 * (size_t)k + q];
+            PairRec<T> nx{};
+            if (sub < cnt) nx = a.pr[(size_t)sub * n + i];
+#pragma unroll 1
+            for (int p = sub; p < cnt; p += kDcLanes) {
+                const PairRec<T> pq = nx;
+                if (p + kDcLanes < cnt) nx = a.pr[(size_t)(p + kDcLanes) * n + i];
                 const T x = pq.x, y = pq.y, z = pq.z;
-                const T r = my_sqrt(x * x + y * y + z * z);
+                const T rr = my_sqrt(x * x + y * y + z * z);
                 T ux, uy, uz;
-                pair_u(a, Di, E, j, x, y, z, ux, uy, uz);
-                const T rdu = (x * ux + y * uy + z * uz) / r;
+                pair_u(a, Di, X, pq.jz & 0xffffff, x, y, z, ux, uy, uz);
+                const T rdu = (x * ux + y * uy + z * uz) / rr;
                 T P[NMU], Pd[NMU];
 #pragma unroll
                 for (int mu = 0; mu < NMU; ++mu) P[mu] = Pd[mu] = T(0);
-                pdot_all<T, 0, NumSlices<T>::value>(a.adjm + tb, a.adjmt + tb, x, y, z, ux, uy, uz, P, Pd);
+                pdot_all<T, 0, NumSlices<T>::value>(adjs + slot, adjs + NV * kDcAtoms + slot, x, y, z, ux, uy, uz, P,
+                                                    Pd);
+                // the pair's share: Q_b (ek P - dP/dt) - Q'_b (r-hat . u) P
+#pragma unroll
+                for (int mu = 0; mu < NMU; ++mu) {
+                    Pd[mu] = ek * P[mu] - Pd[mu];
+                    P[mu] *= -rdu;
+                }
                 // Q_b = T_b(x) u^2 and dQ_b/dr (Eq. 4)
-                const T xx = (T(2) * r - a.rmin - a.rcut) * a.inv_span;
-                const T uu = r < a.rcut ? a.rcut - r : T(0);  // Q_b = 0 beyond the cutoff (Eq. 4)
-                T t0 = T(1), t1 = xx, d0 = T(0), d1 = T(1);
+                const T xx = (T(2) * rr - a.rmin - a.rcut) * a.inv_span;
+                const T uu = rr < a.rcut ? a.rcut - rr : T(0);  // Q_b = 0 beyond the cutoff (Eq. 4)
+                T t0 = T(1), t1 = xx, d0 = T(0), d1 = T(1), Q[NQM], dQ[NQM];
 #pragma unroll
                 for (int b = 0; b < NQM; ++b) {
                     if (!NQC && b >= NQ) break;
-                    T tb_, db_;
-                    if (b == 0) {
-                        tb_ = t0;
-                        db_ = d0;
-                    } else if (b == 1) {
-                        tb_ = t1;
-                        db_ = d1;
-                    } else {
+                    if (b > 1) {
                         const T t2 = T(2) * xx * t1 - t0, d2 = T(2) * t1 + T(2) * xx * d1 - d0;
                         t0 = t1;
                         t1 = t2;
                         d0 = d1;
                         d1 = d2;
-                        tb_ = t2;
-                        db_ = d2;
                     }
-                    const T Q = tb_ * uu * uu;
-                    const T dQ = db_ * (T(2) * a.inv_span) * uu * uu - T(2) * tb_ * uu;
+                    const T tb = b == 0 ? t0 : t1, db = b == 0 ? d0 : d1;
+                    Q[b] = tb * uu * uu;
+                    dQ[b] = db * (T(2) * a.inv_span) * uu * uu - T(2) * tb * uu;
+                }
+                const int e0 = (pq.jz >> 24) * E;
+                if constexpr (NQC % 4 == 0 && NQC > 0) {
+                    Vec4<T>* s4 = reinterpret_cast<Vec4<T>*>(acc) + (e0 >> 2) * 32 + lane;
 #pragma unroll
-                    for (int mu = 0; mu < NMU; ++mu) acc[mu][b] += ek * Q * P[mu] - dQ * rdu * P[mu] - Q * Pd[mu];
+                    for (int mu = 0; mu < NMU; ++mu) {
+#pragma unroll
+                        for (int b = 0; b < NQC; b += 4) {
+                            Vec4<T> s = s4[(mu * (NQC / 4) + b / 4) * 32];
+                            s.x += Q[b] * Pd[mu] + dQ[b] * P[mu];
+                            s.y += Q[b + 1] * Pd[mu] + dQ[b + 1] * P[mu];
+                            s.z += Q[b + 2] * Pd[mu] + dQ[b + 2] * P[mu];
+                            s.w += Q[b + 3] * Pd[mu] + dQ[b + 3] * P[mu];
+                            s4[(mu * (NQC / 4) + b / 4) * 32] = s;
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int b = 0; b < NQM; ++b) {
+                        if (b >= NQ) break;
+#pragma unroll
+                        for (int mu = 0; mu < NMU; ++mu)
+                            acc[(e0 + mu * NQ + b) * 32 + lane] += Q[b] * Pd[mu] + dQ[b] * P[mu];
+                    }
                 }
             }
-            if (any) {
-                // the loss gradient sums over the batch (shared memory first); Jacobian rows go to
-                // their configuration's row directly
-                double* dst = (a.dc_rows ? a.dc_rows + (size_t)k * nc : dcs) + (size_t)((zi * a.S + zp) * NMU) * NQ;
-#pragma unroll
-                for (int mu = 0; mu < NMU; ++mu)
-#pragma unroll
-                    for (int b = 0; b < NQM; ++b)
-                        if (NQC || b < NQ) atomicAdd(&dst[mu * NQ + b], (double)acc[mu][b]);
-            }
+            __syncwarp();
         }
+        if (rounds > 0) flush();
     }
-    __syncthreads();
     if (!a.dc_rows)
-        for (int q = threadIdx.x; q < nc; q += blockDim.x)
-            if (dcs[q] != 0.0) atomicAdd(&a.dc[q], dcs[q]);
+        for (int q = lane; q < nc; q += 32)
+            if (bins[q] != 0.0) atomicAdd(&a.dc[q], bins[q]);
 }
 
 template <class T, int TPA>
@@ -1545,7 +1663,7 @@ int grad_all(EvalCtx<T>& a, const LossArgs& L, cudaStream_t st, int n_sm) {
         const int n_tiles = (a.n_atoms + 31) / 32;
         const int blocks = (int)(((long)n_tiles * G::NDPART_ + 3) / 4);  // as for k_contract_parts
         k_contract_tan_parts<<<blocks, 128, 0, st>>>(a);
-        int sblocks = (int)(((long)n_tiles * G::C_ + 3) / 4);
+        int sblocks = (int)(((long)n_tiles * ((G::C_ + 7) / 8) + 3) / 4);
         if (sblocks > n_sm * 32) sblocks = n_sm * 32;
         k_dual_sum<<<sblocks, 128, 0, st>>>(a);
         k_dx_sum<<<G::M_, 128, 0, st>>>(a);
@@ -1569,14 +1687,20 @@ int grad_all(EvalCtx<T>& a, const LossArgs& L, cudaStream_t st, int n_sm) {
         ++launches;
     }
     {
-        const int threads = 128;
-        const size_t smem = sizeof(double) * (size_t)a.S * a.S * G::NMU_ * a.NQ;
-        int blocks = (a.n_atoms + threads - 1) / threads;
-        if (blocks > n_sm * 8) blocks = n_sm * 8;
+        // one warp per block; atoms per block: enough blocks for eight warps per SM, four atoms at least
+        const size_t smem = dc_bytes<T>(a.S, a.NQ);
+        const long per = ((long)a.n_atoms + n_sm * 8 - 1) / (n_sm * 8);
+        const int chunk = (int)(per < kDcAtoms ? kDcAtoms : per > kDcChunkMax ? kDcChunkMax : (per + 3) / 4 * 4);
+        const int blocks = (a.n_atoms + chunk - 1) / chunk;
+        auto go = [&](void (*k)(const EvalCtx<T>, int)) {
+            if (smem > 48 * 1024)
+                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            k<<<blocks, 32, smem, st>>>(a, chunk);
+        };
         if (a.NQ == 8)
-            k_dc<T, 1, 8><<<blocks, threads, smem, st>>>(a);
+            go(k_dc<T, 8>);
         else
-            k_dc<T, 1, 0><<<blocks, threads, smem, st>>>(a);
+            go(k_dc<T, 0>);
         ++launches;
     }
     return launches;
