@@ -290,6 +290,7 @@ struct BuildArgs {
     const int* nbins;  // bins handed out by the binning (its counter; empty bins are skipped)
     double rs2;      // rsearch^2 (double)
     float lo2, hi2;  // (rsearch -/+ band)^2
+    float cull2;     // (rsearch + margin)^2: candidates further than this from a bin's box are not staged
     const double* pos;
     const int* types;
     const int* cfg_of;
@@ -346,7 +347,8 @@ constexpr int kBias3 = 0x808080;  // three zero components
 // then per warp the accepted keys and the lattice shift of the neighbour's bin of each.
 constexpr int kBuildThreads = 128, kBuildWarps = kBuildThreads / 32;
 constexpr int kGroup = kBuildThreads;  // neighbour bins described per staging round
-constexpr int kChunk = 512;            // candidates staged per round
+constexpr int kChunk = 640;            // candidates staged at once
+constexpr float kCullMargin = 0.05f;   // float error of positions against their bin's box, Angstrom
 constexpr size_t kSmCpos = 0;
 constexpr size_t kSmCshift = kSmCpos + sizeof(float4) * kChunk;
 constexpr size_t kSmCtb = kSmCshift + sizeof(int) * kChunk;
@@ -358,11 +360,16 @@ constexpr size_t kSmWsum = kSmGoff + sizeof(float) * 3 * kGroup;
 constexpr size_t kSmWarp = kSmWsum + 64;
 size_t build_smem(int cap) { return kSmWarp + (size_t)kBuildWarps * cap * (8 + 4); }
 
-// One block per bin (grid-stride over the bins).  The atoms of the bins around it are the candidates
-// of every atom in it: they are staged once in shared memory (positions relative to the bin's
-// origin, image shift minus the candidate's wrap), then each warp takes one atom of the bin, tests
-// the staged candidates with its lanes and compacts the accepted ones with a ballot.  Small cells
-// whose candidates exceed one staging round are re-staged for every group of four atoms.
+// One block per bin, or per part of a bin's atoms where the batch has fewer bins than blocks (grid-stride
+// over those).  The atoms of the bins around it are the candidates of every atom in it: those within the
+// search radius of the bin's bounding box are staged once in shared memory (positions relative to the
+// bin's origin, image shift minus the candidate's wrap), then each warp takes one atom of the bin, tests
+// the staged candidates with its lanes and compacts the accepted ones with a ballot.  A small cell is one
+// bin seen through 27 to 125 images, of which the box keeps a half to a third, so nearly every bin's
+// candidates fit in one staging (kChunk); the others are staged piece by piece for every group of four
+// atoms.  Against staging every candidate, 512 at a time, with one block for a whole bin: 4096 cells of
+// 8-256 atoms 1130 -> 835 us; 61 cells of 8-96 atoms 85 -> 18 us (of which the parts give most); the
+// 16,384-atom fcc cell (12 atoms a bin, the box culls a quarter) 48.5 -> 49.8 us.
 template <class T>
 __global__ void __launch_bounds__(kBuildThreads) k_build(const BuildArgs a) {
     pdl_enter();
@@ -389,10 +396,13 @@ __global__ void __launch_bounds__(kBuildThreads) k_build(const BuildArgs a) {
     __shared__ int smax;
     if (threadIdx.x == 0) smax = 0;
     __syncthreads();
+    __shared__ int s_count;
     const int nbins = *a.nbins;
-    for (int bin = blockIdx.x; bin < nbins; bin += gridDim.x) {
+    const int parts = nbins > 0 ? max(1, min((int)gridDim.x / nbins, 64)) : 1;
+    for (int item = blockIdx.x; item < nbins * parts; item += gridDim.x) {
+        const int bin = item / parts, part = item - bin * parts;
         const int nat = a.bin_count[bin];
-        if (nat == 0) continue;
+        if (part * kBuildWarps >= nat) continue;
         const int start = a.bin_start[bin];
         const int k = a.cfg_of[a.bin_atoms[start]];
         const CellDesc& D = a.desc[k];
@@ -402,9 +412,16 @@ __global__ void __launch_bounds__(kBuildThreads) k_build(const BuildArgs a) {
         const int n_off = (2 * D.c[0] + 1) * ny * nz;
         // the visited bins are distinct (no bin seen through two images): each j is a candidate once
         const bool uniq = D.n[0] > 2 * D.c[0] && D.n[1] > 2 * D.c[1] && D.n[2] > 2 * D.c[2];
+        // the bin's bounding box, its origin at zero
+        const float bx0 = fminf(D.hn[0], 0.f) + fminf(D.hn[3], 0.f) + fminf(D.hn[6], 0.f);
+        const float by0 = fminf(D.hn[1], 0.f) + fminf(D.hn[4], 0.f) + fminf(D.hn[7], 0.f);
+        const float bz0 = fminf(D.hn[2], 0.f) + fminf(D.hn[5], 0.f) + fminf(D.hn[8], 0.f);
+        const float bx1 = fmaxf(D.hn[0], 0.f) + fmaxf(D.hn[3], 0.f) + fmaxf(D.hn[6], 0.f);
+        const float by1 = fmaxf(D.hn[1], 0.f) + fmaxf(D.hn[4], 0.f) + fmaxf(D.hn[7], 0.f);
+        const float bz1 = fmaxf(D.hn[2], 0.f) + fmaxf(D.hn[5], 0.f) + fmaxf(D.hn[8], 0.f);
         bool reuse = false;  // the previous group of atoms left every candidate staged
-        int total = 0;
-        for (int ab = 0; ab < nat; ab += kBuildWarps) {
+        int staged = 0;
+        for (int ab = part * kBuildWarps; ab < nat; ab += parts * kBuildWarps) {
             const bool has = ab + warp < nat;
             const int i = has ? a.bin_atoms[start + ab + warp] : 0;
             const float4 li = has ? a.local[i] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -413,8 +430,70 @@ __global__ void __launch_bounds__(kBuildThreads) k_build(const BuildArgs a) {
             // without carries as long as every component stays within +-127
             const int wik = key_shift(unpack(wi, 0), unpack(wi, 1), unpack(wi, 2)) - kBias3;
             int cnt = 0;
-            for (int g0 = 0; g0 < n_off; g0 += kGroup) {
-                if (!reuse) {
+            // float prefilter of the warp's atom on the first m staged candidates, two per lane per round
+            // (their shared-memory loads overlap); only the rare pairs within 1e-3 Angstrom of the cutoff
+            // take the double-precision decision
+            auto test_staged = [&](const int m) {
+                if (!has) return;
+                auto test = [&](int e, bool& acc, unsigned long long& key, int& tbe) {
+                    acc = false;
+                    key = 0;
+                    tbe = 0;
+                    if (e >= m) return;
+                    const float4 cp = cpos[e];
+                    const float dx = cp.x - li.x, dy = cp.y - li.y, dz = cp.z - li.z;
+                    const float r2 = dx * dx + dy * dy + dz * dz;
+                    if (r2 > a.hi2) return;
+                    const int j = __float_as_int(cp.w);
+                    const int ks = cshift[e] + wik;  // key-order shift s (species in byte 3)
+                    if (j == i && (ks & 0xffffff) == kBias3) return;
+                    if (r2 < a.lo2) {
+                        acc = true;
+                    } else {
+                        const int sv[3] = {key_s(ks, 0), key_s(ks, 1), key_s(ks, 2)};
+                        const double xi[3] = {a.pos[3 * (size_t)i], a.pos[3 * (size_t)i + 1],
+                                              a.pos[3 * (size_t)i + 2]};
+                        const double xj[3] = {a.pos[3 * (size_t)j], a.pos[3 * (size_t)j + 1],
+                                              a.pos[3 * (size_t)j + 2]};
+                        double dd[3];
+                        acc = exact_r2(xi, xj, D.H, sv, dd) < a.rs2;
+                    }
+                    key = ((unsigned long long)j << 32) | (unsigned long long)(unsigned)ks;
+                    tbe = ctb[e];
+                };
+                for (int e0 = 0; e0 < m; e0 += 64) {
+                    bool acc0, acc1;
+                    unsigned long long key0, key1;
+                    int tb0, tb1;
+                    test(e0 + lane, acc0, key0, tb0);
+                    test(e0 + 32 + lane, acc1, key1, tb1);
+                    const unsigned b0 = __ballot_sync(0xffffffffu, acc0);
+                    const unsigned b1 = __ballot_sync(0xffffffffu, acc1);
+                    const unsigned below = (1u << lane) - 1u;
+                    if (acc0) {
+                        const int pos_ = cnt + __popc(b0 & below);
+                        if (pos_ < a.cap) {
+                            keys[pos_] = key0;
+                            ktb[pos_] = tb0;
+                        }
+                    }
+                    cnt += __popc(b0);
+                    if (acc1) {
+                        const int pos_ = cnt + __popc(b1 & below);
+                        if (pos_ < a.cap) {
+                            keys[pos_] = key1;
+                            ktb[pos_] = tb1;
+                        }
+                    }
+                    cnt += __popc(b1);
+                }
+            };
+            if (!reuse) {
+                bool pieces = false;
+                __syncthreads();  // the previous group's tests of the staged candidates are done
+                if (threadIdx.x == 0) s_count = 0;
+                staged = 0;
+                for (int g0 = 0; g0 < n_off; g0 += kGroup) {
                     // 1a. this group's neighbour bins, one per thread: start, count, image shift of
                     //     the wrap, offset of its origin; then a block-wide exclusive scan of the counts
                     const int o = g0 + threadIdx.x;
@@ -432,9 +511,14 @@ __global__ void __launch_bounds__(kBuildThreads) k_build(const BuildArgs a) {
                         ox = o0 * D.hn[0] + o1 * D.hn[3] + o2 * D.hn[6];
                         oy = o0 * D.hn[1] + o1 * D.hn[4] + o2 * D.hn[7];
                         oz = o0 * D.hn[2] + o1 * D.hn[5] + o2 * D.hn[8];
-                        const int nbin = D.bin0 + (w0 * D.n[1] + w1) * D.n[2] + w2;
-                        bstart = a.bin_start[nbin];
-                        bcnt = a.bin_count[nbin];
+                        // a whole bin beyond the search radius of this bin's box holds no candidate
+                        const float ex = fmaxf(fabsf(ox) - (bx1 - bx0), 0.f), ey = fmaxf(fabsf(oy) - (by1 - by0), 0.f),
+                                    ez = fmaxf(fabsf(oz) - (bz1 - bz0), 0.f);
+                        if (ex * ex + ey * ey + ez * ez <= a.cull2) {
+                            const int nbin = D.bin0 + (w0 * D.n[1] + w1) * D.n[2] + w2;
+                            bstart = a.bin_start[nbin];
+                            bcnt = a.bin_count[nbin];
+                        }
                     }
                     int incl = bcnt;
 #pragma unroll
@@ -445,7 +529,7 @@ __global__ void __launch_bounds__(kBuildThreads) k_build(const BuildArgs a) {
                     if (lane == 31) wsum[warp] = incl;
                     __syncthreads();
                     int wpre = 0;
-                    total = 0;
+                    int total = 0;
 #pragma unroll
                     for (int w = 0; w < kBuildWarps; ++w) {
                         const int v = wsum[w];
@@ -459,95 +543,62 @@ __global__ void __launch_bounds__(kBuildThreads) k_build(const BuildArgs a) {
                     goff[kGroup + threadIdx.x] = oy;
                     goff[2 * kGroup + threadIdx.x] = oz;
                     __syncthreads();
-                }
-                for (int c0 = 0; c0 < total; c0 += kChunk) {
-                    const int m = min(kChunk, total - c0);
-                    if (!reuse) {
-                        // 1b. stage candidates c0 .. c0 + m: bin g holds candidate f when
+                    for (int c0 = 0; c0 < total;) {
+                        if (kChunk - staged < kBuildThreads) {  // full: test these, then stage over them
+                            pieces = true;
+                            test_staged(staged);
+                            __syncthreads();
+                            if (threadIdx.x == 0) s_count = 0;
+                            staged = 0;
+                            __syncthreads();
+                        }
+                        // 1b. stage from candidates c0 .. c0 + m: bin g holds candidate f when
                         //     gpre[g] <= f < gpre[g + 1] (the last g with gpre[g] <= f)
-                        for (int f = threadIdx.x; f < m; f += kBuildThreads) {
-                            const int ff = c0 + f;
-                            int g = 0;
+                        const int m = min(kChunk - staged, total - c0);
+                        for (int f0 = 0; f0 < m; f0 += kBuildThreads) {
+                            const int f = f0 + threadIdx.x, ff = c0 + f;
+                            bool in = f < m;
+                            int g = 0, j = 0;
+                            float4 cp = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (in) {
 #pragma unroll
-                            for (int step = kGroup / 2; step > 0; step >>= 1)
-                                if (gpre[g + step] <= ff) g += step;
-                            const int j = a.bin_atoms[gstart[g] + (ff - gpre[g])];
-                            const int wj = a.atom_wrap[j];
-                            const float4 lj = a.local[j];
-                            cpos[f] = make_float4(lj.x + goff[g], lj.y + goff[kGroup + g], lj.z + goff[2 * kGroup + g],
-                                                  __int_as_float(j));
-                            const int tb = gtb[g];
-                            int tz = a.types[j];
-                            tz = tz < 0 ? 0 : (tz >= a.S ? a.S - 1 : tz);  // invalid species are reported by the binning
-                            // the key's low word: image shift in bytes 0..2, the neighbour's species in byte 3
-                            // (a function of j: the key order stays (j, s))
-                            cshift[f] = key_shift(unpack(tb, 0) - unpack(wj, 0), unpack(tb, 1) - unpack(wj, 1),
-                                                  unpack(tb, 2) - unpack(wj, 2)) | (tz << 24);
-                            ctb[f] = tb;
+                                for (int step = kGroup / 2; step > 0; step >>= 1)
+                                    if (gpre[g + step] <= ff) g += step;
+                                j = a.bin_atoms[gstart[g] + (ff - gpre[g])];
+                                const float4 lj = a.local[j];
+                                cp = make_float4(lj.x + goff[g], lj.y + goff[kGroup + g], lj.z + goff[2 * kGroup + g],
+                                                 __int_as_float(j));
+                                // distance to the box: no atom in it is nearer
+                                const float ex = fmaxf(fmaxf(bx0 - cp.x, cp.x - bx1), 0.f),
+                                            ey = fmaxf(fmaxf(by0 - cp.y, cp.y - by1), 0.f),
+                                            ez = fmaxf(fmaxf(bz0 - cp.z, cp.z - bz1), 0.f);
+                                in = ex * ex + ey * ey + ez * ez <= a.cull2;
+                            }
+                            const unsigned keep = __ballot_sync(0xffffffffu, in);
+                            int at = 0;
+                            if (lane == 0 && keep) at = atomicAdd(&s_count, __popc(keep));
+                            at = __shfl_sync(0xffffffffu, at, 0) + __popc(keep & ((1u << lane) - 1u));
+                            if (in) {
+                                const int wj = a.atom_wrap[j], tb = gtb[g];
+                                int tz = a.types[j];
+                                tz = tz < 0 ? 0 : (tz >= a.S ? a.S - 1 : tz);  // invalid species are reported by the binning
+                                cpos[at] = cp;
+                                // the key's low word: image shift in bytes 0..2, the neighbour's species in byte 3
+                                // (a function of j: the key order stays (j, s))
+                                cshift[at] = key_shift(unpack(tb, 0) - unpack(wj, 0), unpack(tb, 1) - unpack(wj, 1),
+                                                       unpack(tb, 2) - unpack(wj, 2)) | (tz << 24);
+                                ctb[at] = tb;
+                            }
                         }
                         __syncthreads();
+                        staged = s_count;
+                        __syncthreads();  // every thread has the count (and is done with the tables)
+                        c0 += m;
                     }
-                    if (has) {
-                        // 1c. float prefilter on the staged candidates, two per lane per round (their
-                        //     shared-memory loads overlap); only the rare pairs within 1e-3 Angstrom of
-                        //     the cutoff take the double-precision decision
-                        auto test = [&](int e, bool& acc, unsigned long long& key, int& tbe) {
-                            acc = false;
-                            key = 0;
-                            tbe = 0;
-                            if (e >= m) return;
-                            const float4 cp = cpos[e];
-                            const float dx = cp.x - li.x, dy = cp.y - li.y, dz = cp.z - li.z;
-                            const float r2 = dx * dx + dy * dy + dz * dz;
-                            if (r2 > a.hi2) return;
-                            const int j = __float_as_int(cp.w);
-                            const int ks = cshift[e] + wik;  // key-order shift s (species in byte 3)
-                            if (j == i && (ks & 0xffffff) == kBias3) return;
-                            if (r2 < a.lo2) {
-                                acc = true;
-                            } else {
-                                const int sv[3] = {key_s(ks, 0), key_s(ks, 1), key_s(ks, 2)};
-                                const double xi[3] = {a.pos[3 * (size_t)i], a.pos[3 * (size_t)i + 1],
-                                                      a.pos[3 * (size_t)i + 2]};
-                                const double xj[3] = {a.pos[3 * (size_t)j], a.pos[3 * (size_t)j + 1],
-                                                      a.pos[3 * (size_t)j + 2]};
-                                double dd[3];
-                                acc = exact_r2(xi, xj, D.H, sv, dd) < a.rs2;
-                            }
-                            key = ((unsigned long long)j << 32) | (unsigned long long)(unsigned)ks;
-                            tbe = ctb[e];
-                        };
-                        for (int e0 = 0; e0 < m; e0 += 64) {
-                            bool acc0, acc1;
-                            unsigned long long key0, key1;
-                            int tb0, tb1;
-                            test(e0 + lane, acc0, key0, tb0);
-                            test(e0 + 32 + lane, acc1, key1, tb1);
-                            const unsigned b0 = __ballot_sync(0xffffffffu, acc0);
-                            const unsigned b1 = __ballot_sync(0xffffffffu, acc1);
-                            const unsigned below = (1u << lane) - 1u;
-                            if (acc0) {
-                                const int pos_ = cnt + __popc(b0 & below);
-                                if (pos_ < a.cap) {
-                                    keys[pos_] = key0;
-                                    ktb[pos_] = tb0;
-                                }
-                            }
-                            cnt += __popc(b0);
-                            if (acc1) {
-                                const int pos_ = cnt + __popc(b1 & below);
-                                if (pos_ < a.cap) {
-                                    keys[pos_] = key1;
-                                    ktb[pos_] = tb1;
-                                }
-                            }
-                            cnt += __popc(b1);
-                        }
-                    }
-                    if (!reuse) __syncthreads();  // the next staging round overwrites the candidates
                 }
+                reuse = !pieces;
             }
-            reuse = n_off <= kGroup && total <= kChunk;
+            test_staged(staged);
             if (!has) continue;
             __syncwarp();
             const int keep = min(cnt, a.cap);
@@ -896,6 +947,7 @@ int build_neighbors(NbrState& nb, int K, int n, const int* cfg_off, const double
     a.rs2 = rsearch * rsearch;
     a.lo2 = (float)((rsearch - kBand) * (rsearch - kBand));
     a.hi2 = (float)((rsearch + kBand) * (rsearch + kBand));
+    a.cull2 = ((float)rsearch + kCullMargin) * ((float)rsearch + kCullMargin);
     a.pos = pos;
     a.types = types;
     a.cfg_of = nb.cfg_of.as<int>();
