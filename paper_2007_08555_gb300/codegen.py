@@ -966,8 +966,8 @@ def emit_dual_parts(prog: Program, parts: int):
     """Straight-line tangent contraction split into parts, for the loss gradient (Sec. 2.2).  Part g
     reads moments M and their tangents T (directional derivatives along the force and stress
     residuals) for its sub-network, evaluates values v and tangents t (t_k = sum w (t_i v_j + v_i t_j)),
-    adds ek v - t of its basis functions over the warp's 32 atoms into dxt[alpha] (lane 0 writes),
-    then runs the adjoint a and its tangent at (seeds: xi, 0) and writes dV/dM and its tangent of
+    hands v and t of its basis functions to sink.put(index in the part, alpha, v, t), where the terms
+    ek v - t of dL/dxi are formed, then runs the adjoint a and its tangent at (seeds: xi, 0) and writes dV/dM and its tangent of
     its moments to dual slots (adj[slot * 32], adt[slot * 32]), numbered by component then part."""
     C = len(prog.comp_list)
     by_k = defaultdict(list)
@@ -991,9 +991,10 @@ def emit_dual_parts(prog: Program, parts: int):
 
     for g, (vals, alphas) in enumerate(groups):
         out.append(f"template <> struct DPart<{g}> {{")
-        out.append("  static __device__ __forceinline__ void run(const float* __restrict__ m, const float* __restrict__ mt, "
-                   "float* __restrict__ adj, float* __restrict__ adt, const float* __restrict__ xi, double ek, bool act, "
-                   "bool lane0, double* __restrict__ dxt) {")
+        out.append(f"  static constexpr int NALPHA = {len(alphas)};")
+        out.append("  template <class Sink> static __device__ __forceinline__ void run(const float* __restrict__ m, "
+                   "const float* __restrict__ mt, float* __restrict__ adj, float* __restrict__ adt, "
+                   "const float* __restrict__ xi, Sink& sink) {")
         comps = sorted(v for v in vals if v < C)
         for c in comps:
             out.append(f"    const float v{c} = m[{c * 32}], t{c} = mt[{c * 32}];")
@@ -1003,12 +1004,10 @@ def emit_dual_parts(prog: Program, parts: int):
             out.append(f"    const float t{k} = " + " + ".join(f"{lit(w)}(t{i} * v{j} + v{i} * t{j})"
                                                            for (i, j, w) in by_k[k]) + ";")
         seed = defaultdict(list)
-        for a in alphas:
+        for q, a in enumerate(alphas):
             v = prog.basis_value[a]
             seed[v].append(a)
-            out.append(f"    {{ double d = act ? ek * (double)v{v} - (double)t{v} : 0.0;")
-            out.append("      for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);")
-            out.append(f"      if (lane0) dxt[{a}] = d; }}")
+            out.append(f"    sink.put({q}, {a}, v{v}, t{v});")
         declared = set()
 
         def aref(v):
@@ -1030,12 +1029,29 @@ def emit_dual_parts(prog: Program, parts: int):
             out.append(f"    adj[{slot_of[(g, c)] * 32}] = {a_}; adt[{slot_of[(g, c)] * 32}] = {b_};")
         out.append("  }")
         out.append("};")
-    out.append("__device__ __forceinline__ void dual_part(int part, const float* m, const float* mt, float* adj, float* adt, "
-               "const float* xi, double ek, bool act, bool lane0, double* dxt) {")
+    out.append(f"constexpr int MAXDALPHA = {max(len(alphas) for _, alphas in groups)};")
+    out.append("template <class Sink>")
+    out.append("__device__ __forceinline__ int dual_part(int part, const float* m, const float* mt, float* adj, float* adt, "
+               "const float* xi, Sink& sink) {")
     out.append("  switch (part) {")
     for g in range(parts):
-        out.append(f"    case {g}: DPart<{g}>::run(m, mt, adj, adt, xi, ek, act, lane0, dxt); return;")
+        out.append(f"    case {g}: DPart<{g}>::run(m, mt, adj, adt, xi, sink); return DPart<{g}>::NALPHA;")
     out.append("  }")
+    out.append("  return 0;")
+    out.append("}")
+    # the same with ek v - t summed over the warp one basis function at a time
+    out.append("struct WarpSink {")
+    out.append("  double ek; bool act, lane0; double* dxt;")
+    out.append("  __device__ __forceinline__ void put(int, int alpha, float v, float t) {")
+    out.append("    double d = act ? ek * (double)v - (double)t : 0.0;")
+    out.append("    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);")
+    out.append("    if (lane0) dxt[alpha] = d;")
+    out.append("  }")
+    out.append("};")
+    out.append("__device__ __forceinline__ void dual_part(int part, const float* m, const float* mt, float* adj, float* adt, "
+               "const float* xi, double ek, bool act, bool lane0, double* dxt) {")
+    out.append("  WarpSink sink{ek, act, lane0, dxt};")
+    out.append("  dual_part(part, m, mt, adj, adt, xi, sink);")
     out.append("}")
     return out
 
