@@ -65,7 +65,7 @@ struct mtp_model {
     int cap = 128;
     double skin = 0.0;   // neighbour lists are built for R_cut + skin
     bool reused = false; // the last evaluation refreshed r_ij from the build-time list
-    DevBuf md_F, md_scalars, md_masses, md_flag;
+    DevBuf md_F, md_scalars, md_masses;
     int last_max = 0;
     int64_t launches = 0;
     // active set (Sec. 2.3): rows of the last selection, A and A^-1 in double precision
@@ -99,7 +99,7 @@ struct mtp_model {
     cudaGraphExec_t g_exec = nullptr;  // graph captured from a call with g_sig
     cudaStream_t cap_stream = nullptr; // private stream the graph is captured on
     int64_t g_launches = 0;            // kernels in the graph
-    int* h_flags = nullptr;            // pinned: error word and largest neighbour count of the last build
+    int* h_flags = nullptr;            // pinned: error word and largest neighbour count of the last build; MD scalars from byte 16
     int tpa_moments = 0, tpa_pairs = 0; // requested threads per atom (0 = chosen per call)
     // the reverse-pair search runs on a side stream, overlapping the evaluation kernels; the force
     // gather of the next evaluation waits for ev_join
@@ -315,14 +315,16 @@ void collect_profile(mtp_model* M) {
     M->prof_calls += 1;
 }
 
+bool reserve_host_flags(mtp_model* M) {
+    if (!M->h_flags && cudaHostAlloc((void**)&M->h_flags, 64, cudaHostAllocDefault) != cudaSuccess) M->h_flags = nullptr;
+    return M->h_flags == nullptr;
+}
+
 // Waits for the stream, then reports the errors the device recorded.  The two flag words come back
 // by stream-ordered copies into pinned memory before the one synchronisation, and the error word is
 // cleared by a stream-ordered memset, so a synchronous call costs a single wait.
 mtp_status finish(mtp_model* M, cudaStream_t st) {
-    if (!M->h_flags && cudaHostAlloc((void**)&M->h_flags, 2 * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
-        M->h_flags = nullptr;
-        return MTP_ENOMEM;
-    }
+    if (reserve_host_flags(M)) return MTP_ENOMEM;
     M->h_flags[0] = M->h_flags[1] = 0;
     if (M->rev_pending) cudaStreamWaitEvent(st, M->ev_join, 0);  // side-stream work of the last build
     if (M->nb.err.p) {
@@ -433,7 +435,7 @@ void mtp_destroy(mtp_model* M) {
                       &M->nb.bin_count, &M->nb.bin_start, &M->nb.atom_slot, &M->nb.bin_atoms, &M->nb.counters,
                       &M->nb.err, &M->g_energy, &M->g_forces, &M->g_virial, &M->g_D, &M->g_eps, &M->g_ew,
                       &M->g_momt, &M->g_adjmt, &M->g_out, &M->g_refs, &M->md_F, &M->md_scalars, &M->md_masses,
-                      &M->md_flag, &M->nb.x0, &M->nb.cpr, &M->d_A, &M->d_Ai, &M->mv_W, &M->mv_pos, &M->mv_sel,
+                      &M->nb.x0, &M->nb.disp, &M->nb.cpr, &M->d_A, &M->d_Ai, &M->mv_W, &M->mv_pos, &M->mv_sel,
                       &M->mv_status, &M->mv_swaps, &M->mv_gmax, &M->s_rows, &M->s_gamma, &M->g_brows,
                       &M->g_batoms};
     for (DevBuf* b : bufs) b->release();
@@ -608,13 +610,19 @@ static mtp_status prepare_neighbors(mtp_model* M, int K, int n, const int* off, 
     return MTP_OK;
 }
 
+static bool reserve_displacements(mtp_model* M, int n) {
+    return M->nb.disp.reserve((size_t)n * (is_fp64(M) ? sizeof(mtp::Vec4<double>) : sizeof(mtp::Vec4<float>))) !=
+           cudaSuccess;
+}
+
 // Refresh r_ij of the last list for new positions (same atoms); requires a build with a skin.
-static mtp_status refresh_neighbors(mtp_model* M, int K, int n, const double* pos, cudaStream_t st) {
+static mtp_status refresh_neighbors(mtp_model* M, int K, int n, const double* pos, cudaStream_t st,
+                                    bool have_u = false) {
     if (!M->nb.has_x0 || M->nb.n_atoms != n || M->nb.n_cfg != K) return MTP_EINVAL;
     const size_t bytes = (size_t)n * M->nb.cap * (is_fp64(M) ? sizeof(mtp::PairRec<double>) : sizeof(mtp::PairRec<float>));
-    if (M->nb.cpr.reserve(bytes)) return MTP_ENOMEM;
+    if (M->nb.cpr.reserve(bytes) || reserve_displacements(M, n)) return MTP_ENOMEM;
     if (M->profiling) mtp::record_mark(M->ev_nbr[0], st);
-    M->launches += mtp::launch_update_pairs(M->nb, pos, st, M->n_sm);
+    M->launches += mtp::launch_update_pairs(M->nb, pos, have_u, st, M->n_sm);
     if (M->profiling) mtp::record_mark(M->ev_nbr[1], st);
     M->reused = true;
     return cuda_status(cudaGetLastError());
@@ -1735,16 +1743,18 @@ mtp_status md_impl(mtp_model* M, int n, double* pos, double* vel, const int32_t*
     cudaStream_t st = (cudaStream_t)stream;
     const size_t N = (size_t)n;
     if (M->md_F.reserve(24 * N) || M->md_scalars.reserve(sizeof(double) * 4) ||
-        M->md_masses.reserve(sizeof(double) * M->S) || M->md_flag.reserve(16) || M->s_off.reserve(16))
+        M->md_masses.reserve(sizeof(double) * M->S) || M->s_off.reserve(16) || reserve_displacements(M, n) ||
+        reserve_host_flags(M))
         return MTP_ENOMEM;
+    const double* h_sc = reinterpret_cast<const double*>(M->h_flags + 4);
     if (cudaMemcpy(M->md_masses.p, masses, sizeof(double) * M->S, cudaMemcpyHostToDevice) != cudaSuccess)
         return MTP_ECUDA;
     int32_t off_h[2] = {0, n};
     cudaMemcpyAsync(M->s_off.p, off_h, sizeof off_h, cudaMemcpyHostToDevice, st);
     const int* off = M->s_off.as<int>();
     double* F = M->md_F.as<double>();
-    double* sc = M->md_scalars.as<double>();  // [0] E_pot, [1] E_kin, [2] grade
-    int* flag = M->md_flag.as<int>();
+    double* sc = M->md_scalars.as<double>();  // [0] E_pot, [1] E_kin, [2] grade, [3] the rebuild flag
+    int* flag = reinterpret_cast<int*>(sc + 3);
     const double* mass = M->md_masses.as<double>();
     const double lim2 = 0.25 * M->skin * M->skin;
     int rebuilds = 0;
@@ -1758,8 +1768,8 @@ mtp_status md_impl(mtp_model* M, int n, double* pos, double* vel, const int32_t*
         brow = M->g_brows.as<double>();
         batoms = M->g_batoms.as<double>();
     }
-    auto forces = [&](bool reuse) -> mtp_status {
-        mtp_status s2 = reuse ? refresh_neighbors(M, 1, n, pos, st)
+    auto forces = [&](bool reuse) -> mtp_status {  // (the drift has left the displacements)
+        mtp_status s2 = reuse ? refresh_neighbors(M, 1, n, pos, st, true)
                               : prepare_neighbors(M, 1, n, off, pos, types, cell, M->skin, st);
         if (s2) return s2;
         if (is_fp64(M))
@@ -1772,17 +1782,25 @@ mtp_status md_impl(mtp_model* M, int n, double* pos, double* vel, const int32_t*
         M->launches += l;
         return MTP_OK;
     };
-    bool stop = false;
+    bool stop = false, rebuild = false;
+    auto drift = [&]() {
+        M->launches += mtp::launch_kick_drift(M->nb, M->S, pos, vel, F, types, mass, dt, lim2, flag, st, M->n_sm);
+    };
+    auto scalars = [&]() { cudaMemcpyAsync(M->h_flags + 4, sc, 4 * sizeof(double), cudaMemcpyDeviceToHost, st); };
+    // Ends a step: the second half kick (not for step 0) and the energies, and the drift of the next step
+    // when nothing can stop the run here, so that one wait covers both.
     auto record = [&](int step) -> mtp_status {
         cudaMemsetAsync(sc + 1, 0, sizeof(double), st);
-        M->launches += mtp::launch_kinetic(n, M->S, vel, types, mass, sc + 1, st, M->n_sm);
-        double h[3] = {0.0, 0.0, 0.0};
-        cudaMemcpyAsync(h, sc, sizeof(double) * (sel ? 3 : 2), cudaMemcpyDeviceToHost, st);
+        M->launches += mtp::launch_kick_kinetic(n, M->S, vel, F, types, mass, 0.5 * dt, step > 0, sc + 1, flag, st,
+                                                M->n_sm);
+        if (!sel && step < n_steps) drift();
+        scalars();
         mtp_status s2 = finish(M, st);
-        ep[step] = h[0];
-        ek[step] = h[1];
+        ep[step] = h_sc[0];
+        ek[step] = h_sc[1];
+        rebuild = *reinterpret_cast<const int*>(h_sc + 3) != 0;
         if (!s2 && sel) {  // the two-threshold scheme on this configuration
-            const double g = h[2];
+            const double g = h_sc[2];
             if (sel->gammas) sel->gammas[step] = g;
             if (g > sel->g_select) {
                 if (sel->cap > 0) {
@@ -1807,16 +1825,15 @@ mtp_status md_impl(mtp_model* M, int n, double* pos, double* vel, const int32_t*
     if (!s) s = record(0);
     if (stop) done = 0;
     for (int step = 1; step <= n_steps && !s && !stop; ++step) {
-        M->launches += mtp::launch_kick(n, M->S, vel, F, types, mass, 0.5 * dt, st, M->n_sm);
-        cudaMemsetAsync(flag, 0, sizeof(int), st);
-        M->launches += mtp::launch_drift(n, pos, vel, M->nb.x0.as<double>(), dt, lim2, flag, st, M->n_sm);
-        int hf = 0;
-        cudaMemcpyAsync(&hf, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
-        if (cudaStreamSynchronize(st) != cudaSuccess) return MTP_ECUDA;
-        if (hf) ++rebuilds;
-        s = forces(hf == 0);
+        if (sel) {
+            drift();
+            scalars();
+            if (cudaStreamSynchronize(st) != cudaSuccess) return MTP_ECUDA;
+            rebuild = *reinterpret_cast<const int*>(h_sc + 3) != 0;
+        }
+        if (rebuild) ++rebuilds;
+        s = forces(!rebuild);
         if (s) break;
-        M->launches += mtp::launch_kick(n, M->S, vel, F, types, mass, 0.5 * dt, st, M->n_sm);
         s = record(step);
         if (stop) done = step;
     }

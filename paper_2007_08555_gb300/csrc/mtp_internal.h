@@ -48,9 +48,9 @@ struct NbrState {
     DevBuf count, pr, rev, keys_am;  // pr: [cap][n] PairRec (r_ij, neighbour | species << 24)
     DevBuf cfg_of, desc, atom_bin, atom_wrap, atom_local, atom_wp, bin_count, bin_start, atom_slot, bin_atoms, counters;
     DevBuf err;
-    // reuse with a skin: positions at the build and the pair records with r_ij refreshed for the
-    // current positions
-    DevBuf x0, cpr;
+    // reuse with a skin: positions at the build, displacements since then (a vector of the working
+    // precision per atom) and the pair records with r_ij refreshed for the current positions
+    DevBuf x0, disp, cpr;
     bool has_x0 = false;
 };
 
@@ -115,14 +115,13 @@ int launch_train_set(int P, int m, const double* theta, const double* d, double 
 int launch_lbfgs_pair(int P, const double* theta, const double* trial, const double* g, const double* g_new,
                       double* S, double* Y, int slot, double* scalars, cudaStream_t st);
 
-// Molecular dynamics helpers (mtp_md.cu).  The refreshed r_ij go to nb.cx/cy/cz.
-int launch_update_pairs(const NbrState& nb, const double* x, cudaStream_t st, int n_sm);
-int launch_kick(int n, int S, double* v, const double* F, const int* types, const double* masses, double half_dt,
-                cudaStream_t st, int n_sm);
-int launch_drift(int n, double* x, const double* v, const double* x0, double dt, double lim2, int* flag,
-                 cudaStream_t st, int n_sm);
-int launch_kinetic(int n, int S, const double* v, const int* types, const double* masses, double* out,
-                   cudaStream_t st, int n_sm);
+// Molecular dynamics helpers (mtp_md.cu).  The refreshed pairs go to nb.cpr, from the displacements in
+// nb.disp (have_u: already there from launch_kick_drift).
+int launch_update_pairs(const NbrState& nb, const double* x, bool have_u, cudaStream_t st, int n_sm);
+int launch_kick_kinetic(int n, int S, double* v, const double* F, const int* types, const double* masses,
+                        double half_dt, bool kick, double* e_kin, int* flag, cudaStream_t st, int n_sm);
+int launch_kick_drift(const NbrState& nb, int S, double* x, double* v, const double* F, const int* types,
+                      const double* masses, double dt, double lim2, int* flag, cudaStream_t st, int n_sm);
 
 // CSR export of the neighbour list with exact double-precision r_ij.
 int export_neighbors(const NbrState& nb, const double* pos, const int* offsets, int* nbr_j, int* nbr_s,
