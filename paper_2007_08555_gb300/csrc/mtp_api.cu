@@ -262,8 +262,13 @@ mtp_status fill_ctx(mtp_model* M, int K, int n, const int* cfg_off, const int* t
     a.n_weights = M->ops->n_weights;
     // explicit setting, else the autotuned choice of this size class, else the heuristic
     const std::pair<int, int> t = (M->tpa_pairs && M->tpa_moments) ? std::pair<int, int>{0, 0} : tuned(M, n);
-    a.tpa = M->tpa_pairs ? M->tpa_pairs : (t.second ? t.second : choose_tpa(n, M->n_sm, 512));
-    a.tpa_m = M->tpa_moments ? M->tpa_moments : (t.first ? t.first : choose_tpa(n, M->n_sm, 128));
+    // (float: two lanes for the pair kernels at any size -- they visit every pair once and read dV/dM from
+    // shared memory, one lane per atom costs 4-12% of an evaluation from 77k atoms on: 442k atoms 4.07 ms
+    // against 3.77 at lev_max 16, 7.3 against 6.6 at 20; and two for the moments up to lev_max 16, where a
+    // lane's running sums leave room for more warps: 0-5%, 55k atoms 0.468 against 0.446 ms)
+    const int least = sizeof(T) == 4 ? 2 : 1, least_m = sizeof(T) == 4 && M->L <= 16 ? 2 : 1;
+    a.tpa = M->tpa_pairs ? M->tpa_pairs : (t.second ? t.second : std::max(least, choose_tpa(n, M->n_sm, 512)));
+    a.tpa_m = M->tpa_moments ? M->tpa_moments : (t.first ? t.first : std::max(least_m, choose_tpa(n, M->n_sm, 128)));
     a.mom = M->mom.as<T>();
     a.adjm = M->adjm.as<T>();
     a.aslots = parts ? M->aslots.as<T>() : nullptr;
