@@ -59,9 +59,9 @@ def build(levels=codegen.SUPPORTED_LEVELS, jobs=None, verbose=False) -> str:
     for name in ("mtp_api.cu", "mtp_nbr.cu", "mtp_maxvol.cu", "mtp_md.cu", "mtp_peak.cu", "mtp_grade_tc.cu", "mtp_relax.cu", "mtp_train.cu"):
         units.append((os.path.join(CSRC, name), os.path.join(OUT, name.replace(".cu", ".o")), common, verbose))
     for L in levels:
-        src = os.path.join(GEN, f"mtp_level_L{L}.cu")
-        units.append((src, os.path.join(OUT, f"mtp_level_L{L}.o"), common + [os.path.join(GEN, f"mtp_gen_L{L}.h")],
-                      verbose))
+        for suffix in ("", "_f64"):
+            units.append((os.path.join(GEN, f"mtp_level_L{L}{suffix}.cu"), os.path.join(OUT, f"mtp_level_L{L}{suffix}.o"),
+                          common + [os.path.join(GEN, f"mtp_gen_L{L}.h")], verbose))
     jobs = jobs or min(len(units), max(2, os.cpu_count() or 2))
     # biggest units first so they overlap with the rest
     units.sort(key=lambda u: -os.path.getsize(u[2][-1]) if u[0].endswith(".cu") and "level" in u[0] else 0)

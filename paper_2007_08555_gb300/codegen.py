@@ -685,12 +685,12 @@ def emit_slice_functions(prog: Program, slc, tag, slot_begin=None):
        mom(x,y,z,f,acc):   acc[t] += f[mu] * x^a y^b z^c                    (moments, Sec. 2.1)
        grad(x,y,z,f,df,adj,s,gx,gy,gz):
              s += sum adj * df[mu] * mono;  g += sum adj * f[mu] * grad(mono)   (adjoint)"""
-    name = {"f": "SliceF", "d": "SliceD", "mf": "SliceMF"}[tag]
+    name = {"f": "SliceF", "d": "SliceD", "mf": "SliceMF", "md": "SliceMD"}[tag]
     out = [f"template <int S> struct {name};"]
     for si, (monos, comps) in enumerate(slc):
         out.append(f"template <> struct {name}<{si}> {{")
         out.append(f"  static constexpr int BEGIN = {min(comps)}, SIZE = {len(comps)};")
-        if tag == "mf":  # the moments kernel's slices: the accumulation alone
+        if tag in ("mf", "md"):  # the moments kernels' slices: the accumulation alone
             out += _mom_function(prog, monos, comps)
             out.append("};")
             continue
@@ -810,6 +810,7 @@ def emit_slice_functions(prog: Program, slc, tag, slot_begin=None):
 # ---------------------------------------------------------------------------------------------
 SLICE_F32 = int(os.environ.get("MTP_SLICE_F32", "136"))
 SLICE_F64 = 64
+SLICE_M64 = 56  # the double moments kernel: two registers per running sum
 
 
 def flop_counts(prog: Program):
@@ -836,6 +837,9 @@ def flop_counts(prog: Program):
 # file (~900 bytes of spills); at 18-20 ptxas keeps most values in local memory, which is still 5.8x
 # faster than the warp-cooperative program at lev_max 20 (measured on a 1M-atom cell).
 UNROLLED_MAX_LEVEL = int(os.environ.get("MTP_UNROLLED_MAX_LEVEL", "20"))
+# The same in double up to this level (two registers per value: beyond it ptxas gives up on allocating
+# registers for the parts); higher levels keep the warp-cooperative program in double.
+UNROLLED_MAX_LEVEL_F64 = 16
 
 
 # The float contraction is split by basis functions into CONTRACT_PARTS[L] programs; each part evaluates the sub-network its basis functions need (shared
@@ -880,7 +884,7 @@ def partition_program(prog: Program, parts: int, balance: float = PART_BALANCE):
 
 
 def emit_parts(prog: Program, parts: int):
-    """Straight-line float contraction split into parts (see CONTRACT_PARTS).  Part g reads the
+    """Straight-line contraction split into parts (see CONTRACT_PARTS), in the precision T of its arrays.  Part g reads the
     moments it needs from the tile layout (src[c * 32]), computes its values in creation order, its
     share of the site energy and of b, then the adjoint of its sub-network seeded by its own basis
     functions, and writes dV/dM of its moments to adjoint slots (dst[slot * 32]).  Slots are
@@ -904,20 +908,20 @@ def emit_parts(prog: Program, parts: int):
            "template <int PART> struct Part;"]
 
     def lit(w):
-        return "" if w == 1.0 else f"{w!r}f * "
+        return "" if w == 1.0 else f"T({w!r}) * "
 
     for g, (vals, alphas) in enumerate(groups):
         out.append(f"template <> struct Part<{g}> {{")
-        out.append("  template <bool WANT_B> static __device__ __forceinline__ float run(const float* __restrict__ src, "
-                   "float* __restrict__ dst, const float* __restrict__ xi, double* __restrict__ bout) {")
+        out.append("  template <bool WANT_B, class T> static __device__ __forceinline__ T run(const T* __restrict__ src, "
+                   "T* __restrict__ dst, const T* __restrict__ xi, double* __restrict__ bout) {")
         comps = sorted(v for v in vals if v < C)
         for c in comps:
-            out.append(f"    const float v{c} = src[{c * 32}];")
+            out.append(f"    const T v{c} = src[{c * 32}];")
         inner = sorted(v for v in vals if v >= C)
         for k in inner:
             terms = [f"{lit(w)}v{i} * v{j}" for (i, j, w) in by_k[k]]
-            out.append(f"    const float v{k} = " + " + ".join(terms) + ";")
-        out.append("    float e = 0.f;")
+            out.append(f"    const T v{k} = " + " + ".join(terms) + ";")
+        out.append("    T e = T(0);")
         seed = defaultdict(list)
         for a in alphas:
             v = prog.basis_value[a]
@@ -929,8 +933,8 @@ def emit_parts(prog: Program, parts: int):
         def aref(v):
             if v not in declared:
                 declared.add(v)
-                init = " + ".join(f"xi[{a}]" for a in seed.get(v, [])) or "0.f"
-                out.append(f"    float a{v} = {init};")
+                init = " + ".join(f"xi[{a}]" for a in seed.get(v, [])) or "T(0)"
+                out.append(f"    T a{v} = {init};")
             return f"a{v}"
 
         for k in reversed(inner):
@@ -945,14 +949,14 @@ def emit_parts(prog: Program, parts: int):
         out.append("    return e;")
         out.append("  }")
         out.append("};")
-    out.append("template <bool WANT_B>")
-    out.append("__device__ __forceinline__ float contract_part(int part, const float* __restrict__ src, "
-               "float* __restrict__ dst, const float* __restrict__ xi, double* __restrict__ bout) {")
+    out.append("template <bool WANT_B, class T>")
+    out.append("__device__ __forceinline__ T contract_part(int part, const T* __restrict__ src, "
+               "T* __restrict__ dst, const T* __restrict__ xi, double* __restrict__ bout) {")
     out.append("  switch (part) {")
     for g in range(parts):
         out.append(f"    case {g}: return Part<{g}>::template run<WANT_B>(src, dst, xi, bout);")
     out.append("  }")
-    out.append("  return 0.f;")
+    out.append("  return T(0);")
     out.append("}")
     return out
 
@@ -987,21 +991,21 @@ def emit_dual_parts(prog: Program, parts: int):
            "template <int PART> struct DPart;"]
 
     def lit(w):
-        return "" if w == 1.0 else f"{w!r}f * "
+        return "" if w == 1.0 else f"T({w!r}) * "
 
     for g, (vals, alphas) in enumerate(groups):
         out.append(f"template <> struct DPart<{g}> {{")
         out.append(f"  static constexpr int NALPHA = {len(alphas)};")
-        out.append("  template <class Sink> static __device__ __forceinline__ void run(const float* __restrict__ m, "
-                   "const float* __restrict__ mt, float* __restrict__ adj, float* __restrict__ adt, "
-                   "const float* __restrict__ xi, Sink& sink) {")
+        out.append("  template <class Sink, class T> static __device__ __forceinline__ void run(const T* __restrict__ m, "
+                   "const T* __restrict__ mt, T* __restrict__ adj, T* __restrict__ adt, "
+                   "const T* __restrict__ xi, Sink& sink) {")
         comps = sorted(v for v in vals if v < C)
         for c in comps:
-            out.append(f"    const float v{c} = m[{c * 32}], t{c} = mt[{c * 32}];")
+            out.append(f"    const T v{c} = m[{c * 32}], t{c} = mt[{c * 32}];")
         inner = sorted(v for v in vals if v >= C)
         for k in inner:
-            out.append(f"    const float v{k} = " + " + ".join(f"{lit(w)}v{i} * v{j}" for (i, j, w) in by_k[k]) + ";")
-            out.append(f"    const float t{k} = " + " + ".join(f"{lit(w)}(t{i} * v{j} + v{i} * t{j})"
+            out.append(f"    const T v{k} = " + " + ".join(f"{lit(w)}v{i} * v{j}" for (i, j, w) in by_k[k]) + ";")
+            out.append(f"    const T t{k} = " + " + ".join(f"{lit(w)}(t{i} * v{j} + v{i} * t{j})"
                                                            for (i, j, w) in by_k[k]) + ";")
         seed = defaultdict(list)
         for q, a in enumerate(alphas):
@@ -1013,8 +1017,8 @@ def emit_dual_parts(prog: Program, parts: int):
         def aref(v):
             if v not in declared:
                 declared.add(v)
-                init = " + ".join(f"xi[{a}]" for a in seed.get(v, [])) or "0.f"
-                out.append(f"    float a{v} = {init}, b{v} = 0.f;")
+                init = " + ".join(f"xi[{a}]" for a in seed.get(v, [])) or "T(0)"
+                out.append(f"    T a{v} = {init}, b{v} = T(0);")
             return f"a{v}", f"b{v}"
 
         for k in reversed(inner):
@@ -1030,26 +1034,27 @@ def emit_dual_parts(prog: Program, parts: int):
         out.append("  }")
         out.append("};")
     out.append(f"constexpr int MAXDALPHA = {max(len(alphas) for _, alphas in groups)};")
-    out.append("template <class Sink>")
-    out.append("__device__ __forceinline__ int dual_part(int part, const float* m, const float* mt, float* adj, float* adt, "
-               "const float* xi, Sink& sink) {")
+    out.append("template <class Sink, class T>")
+    out.append("__device__ __forceinline__ int dual_part(int part, const T* m, const T* mt, T* adj, T* adt, "
+               "const T* xi, Sink& sink) {")
     out.append("  switch (part) {")
     for g in range(parts):
-        out.append(f"    case {g}: DPart<{g}>::run(m, mt, adj, adt, xi, sink); return DPart<{g}>::NALPHA;")
+        out.append(f"    case {g}: DPart<{g}>::template run<Sink, T>(m, mt, adj, adt, xi, sink); return DPart<{g}>::NALPHA;")
     out.append("  }")
     out.append("  return 0;")
     out.append("}")
     # the same with ek v - t summed over the warp one basis function at a time
     out.append("struct WarpSink {")
     out.append("  double ek; bool act, lane0; double* dxt;")
-    out.append("  __device__ __forceinline__ void put(int, int alpha, float v, float t) {")
+    out.append("  template <class T> __device__ __forceinline__ void put(int, int alpha, T v, T t) {")
     out.append("    double d = act ? ek * (double)v - (double)t : 0.0;")
     out.append("    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);")
     out.append("    if (lane0) dxt[alpha] = d;")
     out.append("  }")
     out.append("};")
-    out.append("__device__ __forceinline__ void dual_part(int part, const float* m, const float* mt, float* adj, float* adt, "
-               "const float* xi, double ek, bool act, bool lane0, double* dxt) {")
+    out.append("template <class T>")
+    out.append("__device__ __forceinline__ void dual_part(int part, const T* m, const T* mt, T* adj, T* adt, "
+               "const T* xi, double ek, bool act, bool lane0, double* dxt) {")
     out.append("  WarpSink sink{ek, act, lane0, dxt};")
     out.append("  dual_part(part, m, mt, adj, adt, xi, sink);")
     out.append("}")
@@ -1067,6 +1072,7 @@ def emit_level(L, outdir):
     s32 = slices(prog, SLICE_F32)
     sm32 = moment_slices(prog, SLICE_F32)
     s64 = slices(prog, SLICE_F64)
+    sm64 = moment_slices(prog, SLICE_M64)
     fl = flop_counts(prog)
     tag = f"L{L}"
     lines = [f"// Generated by paper_2007_08555_gb300/codegen.py for lev_max = {L}. Do not edit.",
@@ -1074,7 +1080,7 @@ def emit_level(L, outdir):
     lines.append(f"constexpr int L = {L}, C = {C}, V = {V}, M = {prog.basis.m}, NMU = {prog.n_mu}, "
                  f"NUMAX = {prog.numax};")
     lines.append(f"constexpr int NS32 = {len(s32)}, NS64 = {len(s64)}, MAXS32 = {max(len(c) for _, c in s32)}, "
-                 f"NSM32 = {len(sm32)};")
+                 f"MAXS64 = {max(len(c) for _, c in s64)}, NSM32 = {len(sm32)}, NSM64 = {len(sm64)};")
     lines.append(f"constexpr int FWD_ROWS = {len(fwd_rows)}, ADJ_ROWS = {len(adj_rows)};")
     lines.append(f"constexpr int FWD_LAYERS = {len(fwd_layers)}, ADJ_LAYERS = {len(adj_layers)};")
     lines.append(f"constexpr int PROGRAM_OPS = {len(prog.ops)};")
@@ -1127,18 +1133,21 @@ def emit_level(L, outdir):
         lines += dual_lines
     else:
         lines.append("#define MTPGEN_HAS_PARTS 0")
+    lines.append(f"#define MTPGEN_HAS_PARTS64 {int(has_parts and L <= UNROLLED_MAX_LEVEL_F64)}")
     lines += emit_slice_functions(prog, s32, "f", slot_begin if has_parts else None)
-    lines += emit_slice_functions(prog, s64, "d")
+    lines += emit_slice_functions(prog, s64, "d", slot_begin if has_parts and L <= UNROLLED_MAX_LEVEL_F64 else None)
     lines += emit_slice_functions(prog, sm32, "mf")
+    lines += emit_slice_functions(prog, sm64, "md")
     lines.append("struct Traits {")
     lines.append("  static constexpr int L_ = L, C_ = C, V_ = V, M_ = M, NMU_ = NMU, NUMAX_ = NUMAX, NS32_ = NS32, NS64_ = NS64, "
-                 "MAXS32_ = MAXS32, NSM32_ = NSM32;")
+                 "MAXS32_ = MAXS32, MAXS64_ = MAXS64, NSM32_ = NSM32, NSM64_ = NSM64;")
     lines.append(f"  static constexpr int NPART_ = {nparts}, NSLOT_ = {max(nslots, 1)};")
     lines.append(f"  static constexpr bool HAS_PARTS_ = {'true' if has_parts else 'false'};")
     lines.append(f"  static constexpr int NDPART_ = {ndparts}, NDSLOT_ = {max(ndslots, 1)};")
     lines.append("  template <int S> using F32 = SliceF<S>;")
     lines.append("  template <int S> using F64 = SliceD<S>;")
     lines.append("  template <int S> using MF32 = SliceMF<S>;")
+    lines.append("  template <int S> using MF64 = SliceMD<S>;")
     lines.append("};")
     lines.append(f"}}  // namespace mtpgen_{tag}")
     path = os.path.join(outdir, f"mtp_gen_{tag}.h")
@@ -1151,17 +1160,18 @@ def emit_level(L, outdir):
 
 
 def emit_tu(L, outdir):
-    """One translation unit per level: instantiates the kernels of mtp_level_impl.cuh."""
-    text = (f"// Generated by paper_2007_08555_gb300/codegen.py for lev_max = {L}. Do not edit.\n"
-            f"#include \"mtp_gen_L{L}.h\"\n"
-            f"#define MTP_GEN_NS mtpgen_L{L}\n"
-            f"#define MTP_LEVEL_FN mtp_level_ops_L{L}\n"
-            f"#include \"mtp_level_impl.cuh\"\n")
-    path = os.path.join(outdir, f"mtp_level_L{L}.cu")
-    if not os.path.exists(path) or open(path).read() != text:
-        with open(path, "w") as fh:
-            fh.write(text)
-    return path
+    """Two translation units per level, compiled side by side: mtp_level_L<L>.cu instantiates the float
+    kernels of mtp_level_impl.cuh and holds the registry, mtp_level_L<L>_f64.cu the double ones."""
+    for suffix, extra in (("", ""), ("_f64", "#define MTP_LEVEL_DOUBLE 1\n")):
+        text = (f"// Generated by paper_2007_08555_gb300/codegen.py for lev_max = {L}. Do not edit.\n"
+                f"#include \"mtp_gen_L{L}.h\"\n"
+                f"#define MTP_GEN_NS mtpgen_L{L}\n"
+                f"#define MTP_LEVEL_FN mtp_level_ops_L{L}\n{extra}"
+                f"#include \"mtp_level_impl.cuh\"\n")
+        path = os.path.join(outdir, f"mtp_level_L{L}{suffix}.cu")
+        if not os.path.exists(path) or open(path).read() != text:
+            with open(path, "w") as fh:
+                fh.write(text)
 
 
 def emit_all(outdir, levels=SUPPORTED_LEVELS):

@@ -221,7 +221,7 @@ mtp_status fill_ctx(mtp_model* M, int K, int n, const int* cfg_off, const int* t
     const size_t N = (size_t)n;
     const size_t tiles = (N + 31) / 32;
     const int cap = M->nb.cap;
-    const bool parts = sizeof(T) == 4;  // the float path splits its contraction into parts
+    const bool parts = sizeof(T) == 4 || M->ops->parts_f64;  // the contraction runs in parts
     if (parts && (M->aslots.reserve(tiles * M->ops->contract_slots * 32 * sizeof(T) + 16) ||
                   M->epart.reserve(N * M->ops->contract_parts * sizeof(T) + 16)))
         return MTP_ENOMEM;
@@ -266,7 +266,8 @@ mtp_status fill_ctx(mtp_model* M, int K, int n, const int* cfg_off, const int* t
     // shared memory, one lane per atom costs 4-12% of an evaluation from 77k atoms on: 442k atoms 4.07 ms
     // against 3.77 at lev_max 16, 7.3 against 6.6 at 20; and two for the moments up to lev_max 16, where a
     // lane's running sums leave room for more warps: 0-5%, 55k atoms 0.468 against 0.446 ms)
-    const int least = sizeof(T) == 4 ? 2 : 1, least_m = sizeof(T) == 4 && M->L <= 16 ? 2 : 1;
+    // double: four lanes, from which on every pair is visited once
+    const int least = sizeof(T) == 4 ? 2 : 4, least_m = sizeof(T) == 4 && M->L <= 16 ? 2 : 1;
     a.tpa = M->tpa_pairs ? M->tpa_pairs : (t.second ? t.second : std::max(least, choose_tpa(n, M->n_sm, 512)));
     a.tpa_m = M->tpa_moments ? M->tpa_moments : (t.first ? t.first : std::max(least_m, choose_tpa(n, M->n_sm, 128)));
     a.mom = M->mom.as<T>();
@@ -649,7 +650,7 @@ mtp_status run_param_grad(mtp_model* M, int K, int n, const int* off, const int*
         M->g_momt.reserve(((N + 31) / 32) * M->C * 32 * sizeof(T)) ||
         M->g_adjmt.reserve(((N + 31) / 32) * 32 * adj_row(M) * sizeof(T)))
         return MTP_ENOMEM;
-    const bool dual_parts = sizeof(T) == 4 && M->ops->contract_parts > 0;  // float tangent contraction in parts
+    const bool dual_parts = sizeof(T) == 4 || M->ops->parts_f64;  // tangent contraction in parts
     if (dual_parts && (M->g_dslots.reserve(2 * ((N + 31) / 32) * M->ops->dual_slots * 32 * sizeof(T) + 16) ||
                        M->g_dxt.reserve(((N + 31) / 32) * M->m * sizeof(double) + 16)))
         return MTP_ENOMEM;
@@ -765,7 +766,7 @@ mtp_status run_jacobian(mtp_model* M, int K, int n, const int* off, const int* t
         M->g_brows.reserve(sizeof(double) * (size_t)K * m + 8) || M->g_batoms.reserve(sizeof(double) * N * m + 8) ||
         M->j_rows.reserve(sizeof(double) * (size_t)K * nc + 8) || M->g_out.reserve(sizeof(double) * (1 + m + nc) + 64))
         return MTP_ENOMEM;
-    const bool dual_parts = sizeof(T) == 4 && M->ops->contract_parts > 0;
+    const bool dual_parts = sizeof(T) == 4 || M->ops->parts_f64;
     if (dual_parts && (M->g_dslots.reserve(2 * ((N + 31) / 32) * M->ops->dual_slots * 32 * sizeof(T) + 16) ||
                        M->g_dxt.reserve(((N + 31) / 32) * m * sizeof(double) + 16)))
         return MTP_ENOMEM;

@@ -20,7 +20,8 @@ struct LevelOps {
     int n_weights;
     int program_ops;
     int flop_pair_moments, flop_pair_adjoint, flop_atom_program;
-    int contract_parts, contract_slots;  // float contraction parts and their dV/dM slots per atom
+    int parts_f64;                       // 1: the double path runs the parts too
+    int contract_parts, contract_slots;  // contraction parts and their dV/dM slots per atom
     int dual_parts, dual_slots;          // the same for the tangent contraction of the loss gradient
     // launchers (stream-ordered, no synchronisation); return the number of kernels launched
     // gather_after (or NULL): an event the force gather waits for (the reverse-pair slots)

@@ -1,5 +1,6 @@
-// Kernels of one lev_max, instantiated by a generated translation unit that first includes the
-// generated header and defines MTP_GEN_NS (its namespace) and MTP_LEVEL_FN (registry function).
+// Kernels of one lev_max, instantiated by two generated translation units that first include the
+// generated header and define MTP_GEN_NS (its namespace) and MTP_LEVEL_FN (registry function): one for
+// the float kernels and the registry, one (MTP_LEVEL_DOUBLE) for the double kernels.
 //
 // One evaluation (Sec. 2.1, Eqs. 1-4) runs four kernels:
 //   k_moments   thread group per atom: radial functions f_mu (Eq. 3 with the Chebyshev basis of
@@ -14,6 +15,8 @@
 //   k_gather    thread group per atom: F_i = sum_p (g_ip - g_{j_p, reverse}) and the virial
 //               W = -sum g_ij (x) r_ij, summed per warp and added per configuration in double.
 // The kernels of one evaluation are chained by programmatic dependent launch (launch_pdl).
+#include <algorithm>
+#include <type_traits>
 #include "mtp_common.cuh"
 #include "mtp_level.h"
 
@@ -42,8 +45,8 @@ template <>
 struct NumSlices<double> {
     static constexpr int value = G::NS64_;
 };
-// slices of the moments kernel: in float as many as above with balanced sizes (the largest slice
-// sets the running sums a thread holds), in double the same as above
+// slices of the moments kernels, of balanced sizes (the largest slice sets the running sums a thread
+// holds)
 template <class T, int S>
 struct MomSliceSel;
 template <int S>
@@ -52,7 +55,7 @@ struct MomSliceSel<float, S> {
 };
 template <int S>
 struct MomSliceSel<double, S> {
-    using type = typename G::template F64<S>;
+    using type = typename G::template MF64<S>;
 };
 template <class T>
 struct NumMomSlices;
@@ -62,12 +65,35 @@ struct NumMomSlices<float> {
 };
 template <>
 struct NumMomSlices<double> {
-    static constexpr int value = G::NS64_;
+    static constexpr int value = G::NSM64_;
+};
+template <class T>
+constexpr int max_slice() { return sizeof(T) == 4 ? G::MAXS32_ : G::MAXS64_; }
+
+// whether the contraction runs as generated straight-line parts
+template <class T>
+struct HasParts {
+    static constexpr bool value = sizeof(T) == 4 ? MTPGEN_HAS_PARTS : MTPGEN_HAS_PARTS64;
 };
 
 __device__ __forceinline__ int clamp_species(int z, int S) { return z < 0 ? 0 : (z >= S ? S - 1 : z); }
 __device__ __forceinline__ float my_sqrt(float x) { return sqrtf(x); }
 __device__ __forceinline__ double my_sqrt(double x) { return sqrt(x); }
+
+// |r| and x / |r| of a pair: in double from one reciprocal square root (a square root and a division take
+// some thirty more instructions of the slow double-precision pipe)
+struct Length {
+    double r, inv;
+    __device__ __forceinline__ explicit Length(double r2) : inv(rsqrt(r2)) { r = r2 * inv; }
+    __device__ __forceinline__ double over(double x) const { return x * inv; }
+};
+struct LengthF {
+    float r;
+    __device__ __forceinline__ explicit LengthF(float r2) : r(sqrtf(r2)) {}
+    __device__ __forceinline__ float over(float x) const { return x / r; }
+};
+template <class T>
+using LengthOf = std::conditional_t<sizeof(T) == 4, LengthF, Length>;
 
 // Double-float numbers (hi + lo, |lo| <= ulp(hi) / 2): Knuth's TwoSum and the FMA form of Dekker's
 // TwoProduct give the exact rounding errors, so sums and products keep ~44 significant bits on the
@@ -333,23 +359,26 @@ __device__ __forceinline__ void moments_all(const EvalCtx<T>& a, int i, int sub,
     }
 }
 
-template <class T, int TPA>
-__global__ void __launch_bounds__(128) k_moments(const EvalCtx<T> a) {
-    pdl_enter();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* cs = reinterpret_cast<T*>(smem_raw);
-    load_c(a, cs);
-    const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int stride = gridDim.x * blockDim.x;
-    // the first evaluation kernel clears the per-configuration sums (energy, virial) that later
-    // kernels accumulate
-    for (int t = gtid; t < 10 * a.n_cfg; t += stride) {
+// the first evaluation kernel clears the per-configuration sums (energy, virial) that later kernels
+// accumulate
+template <class T>
+__device__ __forceinline__ void clear_sums(const EvalCtx<T>& a) {
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < 10 * a.n_cfg; t += gridDim.x * blockDim.x) {
         if (t < a.n_cfg) {
             if (a.energy) a.energy[t] = 0.0;
         } else if (a.virial) {
             a.virial[t - a.n_cfg] = 0.0;
         }
     }
+}
+
+template <class T, int TPA>
+__global__ void __launch_bounds__(128) k_moments(const EvalCtx<T> a) {
+    pdl_enter();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* cs = reinterpret_cast<T*>(smem_raw);
+    load_c(a, cs);
+    clear_sums(a);
     // packed-atom work queue: every warp takes the next 32 (atom, lane) units of the batch (atoms of
     // all configurations in one sequence) until none are left; whole warps stay converged
     const int total = ((a.n_atoms + 31) / 32) * 32 * TPA;
@@ -369,6 +398,94 @@ __global__ void __launch_bounds__(128) k_moments(const EvalCtx<T> a) {
         }
         moments_all<T, 0, NumMomSlices<T>::value, TPA>(a, i, sub, active, zi, cnt, cs);
     }
+}
+
+// The double path's moments: a warp per slice of components, all warps of a block on the same 32 (atom,
+// lane) units.  Warp w evaluates the radial functions of every NS-th pair and leaves (r, f) in shared
+// memory for all slices, so that no radial function is evaluated twice: the double-precision pipe is the
+// bound (16 clocks of the SM per warp instruction), and every slice evaluating its own took a third of
+// the kernel.  M64_FIGURES
+template <int S, int NS, int TPA>
+__device__ void moments_split(const EvalCtx<double>& a, const double* cs, double* buf) {
+    if constexpr (S < NS) {
+        if ((int)(threadIdx.x >> 5) != S) {
+            moments_split<S + 1, NS, TPA>(a, cs, buf);
+            return;
+        }
+        using SL = typename MomSliceSel<double, S>::type;
+        constexpr int W = 3 + G::NMU_;
+        const size_t n = (size_t)a.n_atoms;
+        const int lane = threadIdx.x & 31, csz = coef_row(a);
+        const int items = ((a.n_atoms + 31) / 32) * TPA;
+        int half = 0;
+        for (int item = blockIdx.x; item < items; item += gridDim.x) {
+            const int g = item * 32 + lane, i = g / TPA, sub = g % TPA;
+            const bool active = i < a.n_atoms;
+            const int zi = active ? clamp_species(a.types[i], a.S) : 0;
+            const int cnt = active ? a.count[i] : 0;
+            const int trips = cnt > sub ? (cnt - sub + TPA - 1) / TPA : 0;
+            const int rounds = (__reduce_max_sync(0xffffffffu, trips) + NS - 1) / NS;  // equal in every warp
+            double acc[SL::SIZE];
+#pragma unroll
+            for (int t = 0; t < SL::SIZE; ++t) acc[t] = 0.0;
+            PairIn<double> nx{};
+            if (S < trips) nx = load_pair(a, (size_t)(sub + TPA * S) * n + i);
+            for (int rd = 0; rd < rounds; ++rd) {
+                const int t = rd * NS + S;
+                const PairIn<double> cur = nx;
+                if (t + NS < trips) nx = load_pair(a, (size_t)(sub + TPA * (t + NS)) * n + i);
+                double* mine = buf + (size_t)(half * NS + S) * W * 32 + lane;
+                double f[G::NMU_];
+                if (t < trips) {
+                    const Length len(cur.x * cur.x + cur.y * cur.y + cur.z * cur.z);
+                    radial<double, false>(len.r, cs + (zi * a.S + cur.zj) * csz, a.NQ, a.rmin, a.rcut, a.inv_span, f,
+                                          nullptr);
+                    mine[0] = cur.x;
+                    mine[32] = cur.y;
+                    mine[64] = cur.z;
+#pragma unroll
+                    for (int mu = 0; mu < G::NMU_; ++mu) mine[32 * (3 + mu)] = f[mu];
+                } else {  // adds zeros
+#pragma unroll
+                    for (int q = 0; q < W; ++q) mine[32 * q] = 0.0;
+                }
+                // (the other half is written next: its readers passed this barrier)
+                asm volatile("barrier.sync 1, %0;" ::"n"(32 * NS) : "memory");
+#pragma unroll 1
+                for (int q = 0; q < NS; ++q) {
+                    const double* from = buf + (size_t)(half * NS + q) * W * 32 + lane;
+#pragma unroll
+                    for (int mu = 0; mu < G::NMU_; ++mu) f[mu] = from[32 * (3 + mu)];
+                    SL::template mom<double>(from[0], from[32], from[64], f, acc);
+                }
+                half ^= 1;
+            }
+            if (TPA > 1) {
+#pragma unroll
+                for (int t = 0; t < SL::SIZE; ++t) {
+#pragma unroll
+                    for (int o = 1; o < TPA; o <<= 1) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], o);
+                }
+            }
+            if (active) {
+                double* dst = a.mom + (size_t)(i >> 5) * G::C_ * 32 + (i & 31);
+#pragma unroll
+                for (int t = 0; t < SL::SIZE; ++t)
+                    if (t % TPA == sub) dst[(size_t)(SL::BEGIN + t) * 32] = acc[t];
+            }
+        }
+    }
+}
+
+template <int TPA>
+__global__ void __launch_bounds__(32 * NumMomSlices<double>::value) k_moments_split(const EvalCtx<double> a) {
+    pdl_enter();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double* cs = reinterpret_cast<double*>(smem_raw);
+    load_c(a, cs);
+    clear_sums(a);
+    moments_split<0, NumMomSlices<double>::value, TPA>(
+        a, cs, reinterpret_cast<double*>(smem_raw + ((coef_bytes(a) + 15) & ~(size_t)15)));
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -529,12 +646,13 @@ __global__ void __launch_bounds__(256) k_contract(const EvalCtx<T> a) {
 }
 
 #if MTPGEN_HAS_PARTS
-// Float contraction, split into NPART generated parts (basis functions grouped so that one part's
-// values fit in registers): warp w runs part w / n_tiles for the 32 atoms of tile w % n_tiles, so
+// Contraction split into NPART generated parts (basis functions grouped so that one float part's values
+// fit in registers; a double part spills, but the double-precision pipe is its bound): warp w runs part w / n_tiles for the 32 atoms of tile w % n_tiles, so
 // that the warps on an SM mostly run the same code.  Each part writes its site-energy share and
 // dV/dM of its moments to slots; the pair-gradient kernel adds the slots of each component and the
 // gather the energy shares, in a fixed order.
-__global__ void __launch_bounds__(128) k_contract_parts(const EvalCtx<float> a) {
+template <class T>
+__global__ void __launch_bounds__(128) k_contract_parts(const EvalCtx<T> a) {
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int n_tiles = (a.n_atoms + 31) >> 5;
@@ -543,11 +661,11 @@ __global__ void __launch_bounds__(128) k_contract_parts(const EvalCtx<float> a) 
         const int part = w / n_tiles, tile = w - part * n_tiles;
         const int i = tile * 32 + lane;
         if (i >= a.n_atoms) continue;
-        const float* src = a.mom + (size_t)tile * G::C_ * 32 + lane;
-        float* dst = a.aslots + (size_t)tile * G::NSLOT_ * 32 + lane;
+        const T* src = a.mom + (size_t)tile * G::C_ * 32 + lane;
+        T* dst = a.aslots + (size_t)tile * G::NSLOT_ * 32 + lane;
         double* bout = a.b_atoms ? a.b_atoms + (size_t)i * G::M_ : nullptr;
-        const float e = bout ? ::MTP_GEN_NS::contract_part<true>(part, src, dst, a.xi, bout)
-                             : ::MTP_GEN_NS::contract_part<false>(part, src, dst, a.xi, nullptr);
+        const T e = bout ? ::MTP_GEN_NS::contract_part<true, T>(part, src, dst, a.xi, bout)
+                         : ::MTP_GEN_NS::contract_part<false, T>(part, src, dst, a.xi, nullptr);
         a.epart[(size_t)part * a.n_atoms + i] = e;
     }
 }
@@ -583,31 +701,33 @@ struct SharedAdj {
     }
 };
 
-// the float path keeps dV/dM in shared memory, shared by the TPA lanes of an atom, which leaves
-// the registers to the per-pair arithmetic (more resident warps); the double path keeps them in
-// registers
+// dV/dM of an atom lies in shared memory, shared by its TPA lanes, which leaves the registers to the
+// per-pair arithmetic (more resident warps)
 template <class T>
 struct PairgradShared {
-#if MTPGEN_HAS_PARTS
-    static constexpr bool value = sizeof(T) == 4;
-#else
-    static constexpr bool value = false;
-#endif
+    static constexpr bool value = MTPGEN_HAS_PARTS;
 };
 
-// With two or more lanes per atom (PairgradMerged) dV/dM of every slice of an atom sits in shared
+// dV/dM of components [BEGIN, BEGIN + SIZE) of one atom from the contraction's tile layout into its
+// shared vectors (the packed program; the parts' slots are summed by the generated adj_to_shared)
+template <class T, int TPA, int NSA, int OFF>
+__device__ __forceinline__ void adj_tile_to_shared(const T* src, int size, T* mine, int sub) {
+    for (int t = sub; t < size; t += TPA) mine[((t + OFF) / 4) * 4 * NSA + (t + OFF) % 4] = src[(size_t)t * 32];
+}
+
+// With two (float) or four (double) lanes per atom or more (PairgradMerged) dV/dM of every slice of an atom sits in shared
 // memory at once and each pair is visited once: its record, radial functions and gradient store are
-// not repeated per slice.  With one lane per atom a block holds 128 atoms and that array would not
+// not repeated per slice.  With fewer lanes a block holds more atoms and that array would not
 // fit beside the coefficients at the largest sizes, so the slices take turns.
 template <class T, int TPA>
 struct PairgradMerged {
-    static constexpr bool value = PairgradShared<T>::value && TPA >= 2 && NumSlices<T>::value > 1;
+    static constexpr bool value = PairgradShared<T>::value && TPA >= (sizeof(T) == 4 ? 2 : 4) && NumSlices<T>::value > 1;
 };
 
 template <class T, int TPA>
 constexpr size_t pairgrad_adj_bytes() {
     return !PairgradShared<T>::value ? 0
-           : sizeof(T) * (size_t)(((PairgradMerged<T, TPA>::value ? G::C_ : G::MAXS32_) + 3) / 4 * 4) * (128 / TPA);
+           : sizeof(T) * (size_t)(((PairgradMerged<T, TPA>::value ? G::C_ : max_slice<T>()) + 3) / 4 * 4) * (128 / TPA);
 }
 
 template <class T, int S, int TPA, class A>
@@ -624,12 +744,13 @@ __device__ __forceinline__ void pairgrad_pairs(const EvalCtx<T>& a, int i, int s
         const PairIn<T> cur = nx;
         if (p + TPA < cnt) nx = load_pair(a, (size_t)(p + TPA) * n + i);
         const T x = cur.x, y = cur.y, z = cur.z;
-        const T r = my_sqrt(x * x + y * y + z * z);
+        const LengthOf<T> len(x * x + y * y + z * z);
+        const T r = len.r;
         T f[G::NMU_], df[G::NMU_];
         radial<T, true>(r, cs + (zi * a.S + cur.zj) * csz, a.NQ, a.rmin, a.rcut, a.inv_span, f, df);
         T s = T(0), gx = T(0), gy = T(0), gz = T(0);
         SliceSel<T, S>::type::template grad<T>(x, y, z, f, df, adj, s, gx, gy, gz);
-        const T sr = s / r;
+        const T sr = len.over(s);
         gx += sr * x;
         gy += sr * y;
         gz += sr * z;
@@ -653,8 +774,14 @@ __device__ __forceinline__ void pairgrad_slice(const EvalCtx<T>& a, int i, int s
         constexpr int NSA = 128 / TPA;
         T* mine = sadj + 4 * (threadIdx.x / TPA);
         __syncwarp();  // the atom's lanes are done with the previous slice or atom
-        if (active) SL::template adj_to_shared<T, TPA, NSA>(a.aslots + (size_t)(i >> 5) * G::NSLOT_ * 32 + (i & 31),
-                                                            mine, sub);
+        if (active) {
+            if constexpr (HasParts<T>::value)
+                SL::template adj_to_shared<T, TPA, NSA>(a.aslots + (size_t)(i >> 5) * G::NSLOT_ * 32 + (i & 31), mine,
+                                                        sub);
+            else
+                adj_tile_to_shared<T, TPA, NSA, 0>(
+                    a.adjm + ((size_t)(i >> 5) * G::C_ + SL::BEGIN) * 32 + (i & 31), SL::SIZE, mine, sub);
+        }
         __syncwarp();
         pairgrad_pairs<T, S, TPA>(a, i, sub, zi, cnt, cs,
                                   SharedAdj<T, NSA>{reinterpret_cast<const Vec4<T>*>(mine)});
@@ -698,8 +825,12 @@ __device__ __forceinline__ void pairgrad_merged(const EvalCtx<T>& a, int i, int 
     constexpr int NSA = 128 / TPA;
     T* mine = sadj + 4 * (threadIdx.x / TPA);
     __syncwarp();  // the atom's lanes are done with the previous atom
-    if (active)
-        adj_all_to_shared<T, 0, TPA, NSA>(a.aslots + (size_t)(i >> 5) * G::NSLOT_ * 32 + (i & 31), mine, sub);
+    if (active) {
+        if constexpr (HasParts<T>::value)
+            adj_all_to_shared<T, 0, TPA, NSA>(a.aslots + (size_t)(i >> 5) * G::NSLOT_ * 32 + (i & 31), mine, sub);
+        else
+            adj_tile_to_shared<T, TPA, NSA, 0>(a.adjm + (size_t)(i >> 5) * G::C_ * 32 + (i & 31), G::C_, mine, sub);
+    }
     __syncwarp();
     const Vec4<T>* q = reinterpret_cast<const Vec4<T>*>(mine);
     const size_t n = (size_t)a.n_atoms;
@@ -712,12 +843,13 @@ __device__ __forceinline__ void pairgrad_merged(const EvalCtx<T>& a, int i, int 
         const PairIn<T> cur = nx;
         if (p + TPA < cnt) nx = load_pair(a, (size_t)(p + TPA) * n + i);
         const T x = cur.x, y = cur.y, z = cur.z;
-        const T r = my_sqrt(x * x + y * y + z * z);
+        const LengthOf<T> len(x * x + y * y + z * z);
+        const T r = len.r;
         T f[G::NMU_], df[G::NMU_];
         radial<T, true>(r, cs + (zi * a.S + cur.zj) * csz, a.NQ, a.rmin, a.rcut, a.inv_span, f, df);
         T s = T(0), gx = T(0), gy = T(0), gz = T(0);
         grad_all_slices<T, 0, NSA>(x, y, z, f, df, q, s, gx, gy, gz);
-        const T sr = s / r;
+        const T sr = len.over(s);
         a.g[idx] = Vec4<T>{gx + sr * x, gy + sr * y, gz + sr * z, T(0)};
     }
 }
@@ -781,6 +913,19 @@ __device__ __forceinline__ void flush_run(const EvalCtx<T>& a, int cfg, const T*
     if (want_e) atomicAdd(&a.energy[cfg], erun);
 }
 
+__device__ __forceinline__ Df run_add(Df a, Df b) { return df_add(a, b); }
+__device__ __forceinline__ double run_add(double a, double b) { return a + b; }
+__device__ __forceinline__ void run_zero(Df& a) { a = {0.f, 0.f}; }
+__device__ __forceinline__ void run_zero(double& a) { a = 0.0; }
+__device__ __forceinline__ Df run_of(float e) { return {e, 0.f}; }
+__device__ __forceinline__ double run_of(double e) { return e; }
+__device__ __forceinline__ double run_value(Df a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double run_value(double a) { return a; }
+__device__ __forceinline__ Df run_shfl(Df a, int o) {
+    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ double run_shfl(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+
 template <class T>
 struct GatherIn {
     Vec4<T> g;
@@ -791,12 +936,7 @@ struct GatherIn {
 template <class T, int TPA>
 __global__ void __launch_bounds__(128, TPA >= 4 ? 8 : 1) k_gather(const EvalCtx<T> a) {
     pdl_enter();
-    // float path with contraction parts: the site energies are the sums of the parts' shares
-#if MTPGEN_HAS_PARTS
-    constexpr bool kE = sizeof(T) == 4;
-#else
-    constexpr bool kE = false;
-#endif
+    constexpr bool kE = HasParts<T>::value;  // the site energies are the sums of the contraction parts' shares
     const bool want_e = kE && a.energy != nullptr;
     constexpr int kWarps = 4;  // blockDim.x == 128
     __shared__ int s_cfg[kWarps];
@@ -806,7 +946,8 @@ __global__ void __launch_bounds__(128, TPA >= 4 ? 8 : 1) k_gather(const EvalCtx<
     const int stride = gridDim.x * blockDim.x;
     const int n_groups = ((a.n_atoms + 31) / 32) * 32;  // whole warps stay converged for the shuffles
     T Wrun[9];
-    Df Erun = {0.f, 0.f};  // energy: an unevaluated float pair (error-free sums, no FP64 work)
+    std::conditional_t<sizeof(T) == 4, Df, double> Erun;  // energy: on the float path an unevaluated float pair
+    run_zero(Erun);
 #pragma unroll
     for (int k = 0; k < 9; ++k) Wrun[k] = T(0);
     int wcfg = -1;
@@ -902,10 +1043,10 @@ __global__ void __launch_bounds__(128, TPA >= 4 ? 8 : 1) k_gather(const EvalCtx<
             a.forces[3 * (size_t)i + 1] = (double)F[1];
             a.forces[3 * (size_t)i + 2] = (double)F[2];
         }
-        float e_i = 0.f;
+        T e_i = T(0);
         if constexpr (kE) {
             if (active && sub == 0) {
-                float e = 0.f;
+                T e = T(0);
 #pragma unroll
                 for (int p = 0; p < G::NPART_; ++p) e += a.epart[(size_t)p * n + i];
                 if (a.site) a.site[i] = (double)e;
@@ -914,15 +1055,15 @@ __global__ void __launch_bounds__(128, TPA >= 4 ? 8 : 1) k_gather(const EvalCtx<
         }
         if (active && (a.virial || want_e)) {
             if (cfg != wcfg) {
-                if (wcfg >= 0) flush_run(a, wcfg, Wrun, (double)Erun.hi + (double)Erun.lo, want_e);
+                if (wcfg >= 0) flush_run(a, wcfg, Wrun, run_value(Erun), want_e);
 #pragma unroll
                 for (int k = 0; k < 9; ++k) Wrun[k] = T(0);
-                Erun = {0.f, 0.f};
+                run_zero(Erun);
                 wcfg = cfg;
             }
 #pragma unroll
             for (int k = 0; k < 9; ++k) Wrun[k] += W[k];
-            if (want_e) Erun = df_add(Erun, {e_i, 0.f});
+            if (want_e) Erun = run_add(Erun, run_of(e_i));
         }
     }
     if (!a.virial && !want_e) return;
@@ -942,10 +1083,7 @@ __global__ void __launch_bounds__(128, TPA >= 4 ? 8 : 1) k_gather(const EvalCtx<
         }
         if (want_e) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const Df other = {__shfl_xor_sync(0xffffffffu, Erun.hi, o), __shfl_xor_sync(0xffffffffu, Erun.lo, o)};
-                Erun = df_add(Erun, other);
-            }
+            for (int o = 16; o > 0; o >>= 1) Erun = run_add(Erun, run_shfl(Erun, o));
         }
         if (lane < 9) {
             T v = Wrun[0];
@@ -953,9 +1091,9 @@ __global__ void __launch_bounds__(128, TPA >= 4 ? 8 : 1) k_gather(const EvalCtx<
             for (int k = 1; k < 9; ++k) v = lane == k ? Wrun[k] : v;
             s_w[warp][lane] = v;
         }
-        if (lane == 9) s_e[warp] = (double)Erun.hi + (double)Erun.lo;
+        if (lane == 9) s_e[warp] = run_value(Erun);
     } else if (wcfg >= 0) {
-        flush_run(a, wcfg, Wrun, (double)Erun.hi + (double)Erun.lo, want_e);
+        flush_run(a, wcfg, Wrun, run_value(Erun), want_e);
     }
     if (lane == 0) s_cfg[warp] = wuni ? cmax : -1;  // -1: nothing left to add
     __syncthreads();
@@ -991,14 +1129,26 @@ int launch_pairs(const EvalCtx<T>& a, cudaStream_t st, int n_sm, bool moments) {
     const int max_blocks = n_sm * 16;
     if (blocks > max_blocks) blocks = max_blocks;
     if (blocks < 1) blocks = 1;
-    if (moments) {
+    if constexpr (sizeof(T) == 8) {
+        if (moments) {
+            constexpr int NS = NumMomSlices<double>::value;
+            const size_t smem = ((cbytes + 15) & ~(size_t)15) + sizeof(double) * 2 * NS * (3 + G::NMU_) * 32;
+            if (smem > 48 * 1024)
+                cudaFuncSetAttribute(k_moments_split<TPA>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+            const long items = (long)((a.n_atoms + 31) / 32) * TPA;
+            launch_pdl(k_moments_split<TPA>, (int)std::min(items, (long)n_sm * 16), 32 * NS, smem, st, a);
+            return 1;
+        }
+    } else if (moments) {
         static bool attr_m = false;
         if (!attr_m && cbytes > 48 * 1024) {  // 8 species with 16 radial functions in double
             cudaFuncSetAttribute(k_moments<T, TPA>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
             attr_m = true;
         }
         launch_pdl(k_moments<T, TPA>, blocks, threads, cbytes, st, a);
-    } else {
+        return 1;
+    }
+    {
         const size_t smem = ((cbytes + 15) & ~(size_t)15) + pairgrad_adj_bytes<T, TPA>();
         static bool attr_set = false;
         if (!attr_set && smem > 48 * 1024) {
@@ -1029,23 +1179,22 @@ int eval_all(const EvalCtx<T>& a, cudaStream_t st, int n_sm, cudaEvent_t* marks,
     if (marks) record_mark(marks[kPhaseMoments], st);
     launches += launch_pairs_tpa<T>(a, st, n_sm, true);
     if (marks) record_mark(marks[kPhaseContract], st);
+    if constexpr (HasParts<T>::value) {
 #if MTPGEN_HAS_PARTS
-    if constexpr (sizeof(T) == 4) {
         const int threads = 128;
         // one warp per (part, tile) item and no grid-stride: the blocks resident at any time are a
         // window of consecutive part-major items, so an SM mostly runs one part's code (the parts are
         // long straight-line programs and their instruction fetch bounds the kernel otherwise)
         const long warps = (long)((a.n_atoms + 31) / 32) * G::NPART_;
         const int blocks = (int)((warps + 3) / 4);
-        launch_pdl(k_contract_parts, blocks, threads, 0, st, a);
+        launch_pdl(k_contract_parts<T>, blocks, threads, 0, st, a);
         ++launches;
         if (a.b_rows) {  // the caller provides per-atom rows whenever b rows are requested
             launch_pdl(k_brows<T>, a.n_cfg, 128, 0, st, a, a.cfg_off);
             ++launches;
         }
-    } else
 #endif
-    {
+    } else {
         // atoms per warp: amortise each program word over several atoms while the per-warp working
         // set (2 A V values) stays small enough for at least two blocks per SM
         constexpr int A = (sizeof(T) * G::V_ * 2 * 4 * 8 <= 100 * 1024) ? 4
@@ -1095,12 +1244,16 @@ int eval_all(const EvalCtx<T>& a, cudaStream_t st, int n_sm, cudaEvent_t* marks,
     return launches;
 }
 
+int eval_f64(const EvalCtx<double>& a, cudaStream_t st, int n_sm, cudaEvent_t* marks, cudaEvent_t gather_after);
+#ifndef MTP_LEVEL_DOUBLE
 int eval_f32(const EvalCtx<float>& a, cudaStream_t st, int n_sm, cudaEvent_t* marks, cudaEvent_t gather_after) {
     return eval_all<float>(a, st, n_sm, marks, gather_after);
 }
+#else
 int eval_f64(const EvalCtx<double>& a, cudaStream_t st, int n_sm, cudaEvent_t* marks, cudaEvent_t gather_after) {
     return eval_all<double>(a, st, n_sm, marks, gather_after);
 }
+#endif
 
 
 // ----------------------------------------------------------------------------------------------
@@ -1293,14 +1446,18 @@ __device__ __forceinline__ void run_program_dual(const unsigned long long* __res
 constexpr int kAdjRow = (G::C_ + 3) / 4 * 4;
 
 #if MTPGEN_HAS_PARTS
-// Tangent contraction of the loss gradient (float), split into NDPART generated parts like the
+// Tangent contraction of the loss gradient, split into NDPART generated parts like the
 // forward contraction: warp w runs part w / n_tiles for the 32 atoms of tile w % n_tiles.  Each part
 // writes dV/dM and its tangent for its moments to dual slots and its basis functions' shares of
 // dL/dxi (summed over the tile's atoms) to dxt[tile].  Every lane forms its atom's ek B - dB/dt as a
 // double-float pair in shared memory, then a lane per basis function sums the 32 atoms in double-float
 // arithmetic: warp sums in double cost ten instructions of the double-precision pipe per basis function,
 // 16 clocks of the SM each (2048 cells, lev_max 20: 3.79 ms, with these sums 2.98).
-struct TanSink {
+template <class T>
+struct TanSink;
+template <>
+struct TanSink<float> {
+    using Pair = float2;
     float eh, el;  // ek as a float pair; zero for a lane without an atom
     float keep;    // 1, or 0 for a lane without an atom
     float2* s;     // [MAXDALPHA][33]
@@ -1312,14 +1469,44 @@ struct TanSink {
         s[q * 33 + lane] = make_float2(d.hi, d.lo);
         if (lane == 0) alpha[q] = al;
     }
+    __device__ __forceinline__ double sum(int q) const {
+        Df d = {0.f, 0.f};
+#pragma unroll 4
+        for (int l = 0; l < 32; ++l) d = df_add(d, {s[q * 33 + l].x, s[q * 33 + l].y});
+        return (double)d.hi + (double)d.lo;
+    }
+    __device__ __forceinline__ TanSink(double ek, bool act, Pair* st, int* al, int ln)
+        : eh((float)ek), el((float)(ek - (double)(float)ek)), keep(act ? 1.f : 0.f), s(st), alpha(al), lane(ln) {}
+};
+template <>
+struct TanSink<double> {
+    using Pair = double;
+    double ek, keep;
+    double* s;
+    int* alpha;
+    int lane;
+    __device__ __forceinline__ void put(int q, int al, double v, double t) {
+        s[q * 33 + lane] = ek * v - keep * t;
+        if (lane == 0) alpha[q] = al;
+    }
+    __device__ __forceinline__ double sum(int q) const {
+        double d = 0.0;
+#pragma unroll 4
+        for (int l = 0; l < 32; ++l) d += s[q * 33 + l];
+        return d;
+    }
+    __device__ __forceinline__ TanSink(double e, bool act, Pair* st, int* al, int ln)
+        : ek(e), keep(act ? 1.0 : 0.0), s(st), alpha(al), lane(ln) {}
 };
 constexpr int kTanWarps = 4;
-constexpr size_t kTanWarpBytes = (size_t)::MTP_GEN_NS::MAXDALPHA * (33 * sizeof(float2) + 8);
+constexpr size_t kTanWarpBytes = (size_t)::MTP_GEN_NS::MAXDALPHA * (33 * 8 + 8);
 
-__global__ void __launch_bounds__(32 * kTanWarps) k_contract_tan_parts(const EvalCtx<float> a) {
+template <class T>
+__global__ void __launch_bounds__(32 * kTanWarps) k_contract_tan_parts(const EvalCtx<T> a) {
+    using Pair = typename TanSink<T>::Pair;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
-    float2* stage = reinterpret_cast<float2*>(smem_raw + (threadIdx.x >> 5) * kTanWarpBytes);
+    Pair* stage = reinterpret_cast<Pair*>(smem_raw + (threadIdx.x >> 5) * kTanWarpBytes);
     int* alpha = reinterpret_cast<int*>(stage + ::MTP_GEN_NS::MAXDALPHA * 33);
     const int n_tiles = (a.n_atoms + 31) >> 5;
     const int total = n_tiles * G::NDPART_;
@@ -1329,29 +1516,21 @@ __global__ void __launch_bounds__(32 * kTanWarps) k_contract_tan_parts(const Eva
         const int i = tile * 32 + lane;
         const bool act = i < a.n_atoms;
         const double ek = act ? a.gew[a.cfg_of[i]] : 0.0;
-        const float eh = (float)ek;
-        TanSink sink{eh, (float)(ek - (double)eh), act ? 1.f : 0.f, stage, alpha, lane};
+        TanSink<T> sink(ek, act, stage, alpha, lane);
         const size_t mo = (size_t)tile * G::C_ * 32 + lane;
         const size_t so = (size_t)tile * G::NDSLOT_ * 32 + lane;
         const int na = ::MTP_GEN_NS::dual_part(part, a.mom + mo, a.momt + mo, a.dslots + so, a.dslots + half + so, a.xi,
                                                sink);
         __syncwarp();
-        for (int q = lane; q < na; q += 32) {
-            Df d = {0.f, 0.f};
-#pragma unroll 4
-            for (int l = 0; l < 32; ++l) {
-                const float2 x = stage[q * 33 + l];
-                d = df_add(d, {x.x, x.y});
-            }
-            a.dxt[(size_t)tile * G::M_ + alpha[q]] = (double)d.hi + (double)d.lo;
-        }
+        for (int q = lane; q < na; q += 32) a.dxt[(size_t)tile * G::M_ + alpha[q]] = sink.sum(q);
         __syncwarp();
     }
 }
 
 // dV/dM and its tangent = sums of their dual slots (slot order), one warp per (tile, eight components),
 // written atom by atom for k_dc (eight components: one whole sector of an atom's row)
-__global__ void __launch_bounds__(128) k_dual_sum(const EvalCtx<float> a) {
+template <class T>
+__global__ void __launch_bounds__(128) k_dual_sum(const EvalCtx<T> a) {
     constexpr int C = G::C_, CP = kAdjRow;
     constexpr int NG = (C + 7) / 8;
     const int lane = threadIdx.x & 31;
@@ -1360,11 +1539,11 @@ __global__ void __launch_bounds__(128) k_dual_sum(const EvalCtx<float> a) {
     const int warps = (gridDim.x * blockDim.x) >> 5;
     for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_tiles * NG; w += warps) {
         const int tile = w / NG, c0 = (w - tile * NG) * 8;
-        const float* sl = a.dslots + (size_t)tile * G::NDSLOT_ * 32 + lane;
-        float va[8], vt[8];
+        const T* sl = a.dslots + (size_t)tile * G::NDSLOT_ * 32 + lane;
+        T va[8], vt[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            va[q] = vt[q] = 0.f;
+            va[q] = vt[q] = T(0);
             if (c0 + q < C) {
                 const int s0 = ::MTP_GEN_NS::dslot_begin[c0 + q], s1 = ::MTP_GEN_NS::dslot_begin[c0 + q + 1];
                 for (int s = s0; s < s1; ++s) {
@@ -1378,14 +1557,15 @@ __global__ void __launch_bounds__(128) k_dual_sum(const EvalCtx<float> a) {
 #pragma unroll
         for (int q = 0; q < 8; q += 4)
             if (c0 + q < CP) {
-                *reinterpret_cast<Vec4<float>*>(a.adjm + o + q) = Vec4<float>{va[q], va[q + 1], va[q + 2], va[q + 3]};
-                *reinterpret_cast<Vec4<float>*>(a.adjmt + o + q) = Vec4<float>{vt[q], vt[q + 1], vt[q + 2], vt[q + 3]};
+                *reinterpret_cast<Vec4<T>*>(a.adjm + o + q) = Vec4<T>{va[q], va[q + 1], va[q + 2], va[q + 3]};
+                *reinterpret_cast<Vec4<T>*>(a.adjmt + o + q) = Vec4<T>{vt[q], vt[q + 1], vt[q + 2], vt[q + 3]};
             }
     }
 }
 
 // dL/dxi += sum over tiles of dxt (one block per basis function, fixed reduction order)
-__global__ void __launch_bounds__(128) k_dx_sum(const EvalCtx<float> a) {
+template <class T>
+__global__ void __launch_bounds__(128) k_dx_sum(const EvalCtx<T> a) {
     __shared__ double s[128];
     const int alpha = blockIdx.x;
     const int n_tiles = (a.n_atoms + 31) >> 5;
@@ -1693,22 +1873,21 @@ int grad_all(EvalCtx<T>& a, const LossArgs& L, cudaStream_t st, int n_sm) {
         case 2: launches += launch_grad_pairs<T, 2>(a, st, n_sm); break;
         default: launches += launch_grad_pairs<T, 1>(a, st, n_sm); break;
     }
+    if constexpr (HasParts<T>::value) {
 #if MTPGEN_HAS_PARTS
-    if constexpr (sizeof(T) == 4) {
         const int n_tiles = (a.n_atoms + 31) / 32;
         const int blocks = (int)(((long)n_tiles * G::NDPART_ + 3) / 4);  // as for k_contract_parts
         if (kTanWarps * kTanWarpBytes > 48 * 1024)
-            cudaFuncSetAttribute(k_contract_tan_parts, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(k_contract_tan_parts<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(kTanWarps * kTanWarpBytes));
-        k_contract_tan_parts<<<blocks, 32 * kTanWarps, kTanWarps * kTanWarpBytes, st>>>(a);
+        k_contract_tan_parts<T><<<blocks, 32 * kTanWarps, kTanWarps * kTanWarpBytes, st>>>(a);
         int sblocks = (int)(((long)n_tiles * ((G::C_ + 7) / 8) + 3) / 4);
         if (sblocks > n_sm * 32) sblocks = n_sm * 32;
-        k_dual_sum<<<sblocks, 128, 0, st>>>(a);
-        k_dx_sum<<<G::M_, 128, 0, st>>>(a);
+        k_dual_sum<T><<<sblocks, 128, 0, st>>>(a);
+        k_dx_sum<T><<<G::M_, 128, 0, st>>>(a);
         launches += 3;
-    } else
 #endif
-    {
+    } else {
         const int threads = 128, wpb = 4;
         const size_t smem = sizeof(T) * (size_t)G::V_ * (1 + 4 * wpb) + sizeof(float) * (a.n_weights + 4) + 64;
         if (smem > 200 * 1024) return -1000;
@@ -1744,11 +1923,16 @@ int grad_all(EvalCtx<T>& a, const LossArgs& L, cudaStream_t st, int n_sm) {
     return launches;
 }
 
+int grad_f64(EvalCtx<double>& a, const LossArgs& L, cudaStream_t st, int n_sm);
+#ifndef MTP_LEVEL_DOUBLE
 int grad_f32(EvalCtx<float>& a, const LossArgs& L, cudaStream_t st, int n_sm) { return grad_all<float>(a, L, st, n_sm); }
+#else
 int grad_f64(EvalCtx<double>& a, const LossArgs& L, cudaStream_t st, int n_sm) { return grad_all<double>(a, L, st, n_sm); }
+#endif
 
 }  // namespace MTP_GEN_NS
 
+#ifndef MTP_LEVEL_DOUBLE
 const LevelOps* MTP_LEVEL_FN() {
     namespace g = ::MTP_GEN_NS;
     static const LevelOps ops = {
@@ -1757,9 +1941,11 @@ const LevelOps* MTP_LEVEL_FN() {
         g::fwd_ops, g::fwd_layer_rows, g::FWD_ROWS, g::FWD_LAYERS,
         g::adj_ops, g::adj_layer_rows, g::ADJ_ROWS, g::ADJ_LAYERS, g::weights, g::NWEIGHTS,
         g::PROGRAM_OPS, g::FLOP_PAIR_MOMENTS, g::FLOP_PAIR_ADJOINT, g::FLOP_ATOM_PROGRAM,
-        g::Traits::NPART_, g::Traits::NSLOT_, g::Traits::NDPART_, g::Traits::NDSLOT_,
+        MTPGEN_HAS_PARTS64, g::Traits::NPART_, g::Traits::NSLOT_, g::Traits::NDPART_, g::Traits::NDSLOT_,
         &MTP_GEN_NS::eval_f32, &MTP_GEN_NS::eval_f64, &MTP_GEN_NS::grad_f32, &MTP_GEN_NS::grad_f64};
     return &ops;
 }
+
+#endif
 
 }  // namespace mtp
