@@ -21,9 +21,10 @@
 // pivot eliminates is replaced by the column of the inverse that it creates).  Pivots, factors and
 // inverse are the same operations in the same order as elimination by one block with explicit
 // interchanges, so the selection does not depend on the number of blocks.
-// Bound: one exchange per step (a release, a poll and a row read through L2) and the step's FMAs on the
-// double-precision pipe (~2 per clock and SM).  Measured with all grades of the rows: 232 x 116 in
-// 2.81 ms, 920 x 460 in 13.7 ms; one block with every matrix in global memory took 11.3 and 482 ms.
+// Bound: one exchange per step (a trip to the L2 for the records and one for the winner's row) and the
+// step's FMAs on the double-precision pipe (~2 per clock and SM).  Measured with all grades of the rows:
+// 232 x 116 in 1.61 ms, 920 x 460 in 7.9 ms; with flags and fences instead of tagged words 2.81 and 13.7;
+// one block with every matrix in global memory 11.3 and 482 ms.
 // k_grade: gamma_r = max_j |(b_r A^-1)_j| for many rows; 64x64 output tiles through shared memory,
 //   the row maxima are combined with an atomic max on the bit pattern (gamma >= 0); a NaN in a row
 //   of b A^-1 gives gamma = +inf, so a broken configuration reads as extrapolating.
@@ -41,149 +42,205 @@ namespace {
 constexpr int kMvThreads = 512;
 
 // One round of all blocks: each publishes a candidate (a non-negative value and a 32-bit payload, ties
-// to the smaller payload) and a row of numbers; everyone gets the winner.  A record is two words that
-// carry their own round (a parity in the sign bit of the value, the round's number beside the payload),
-// in two alternating sets: a block publishes round t + 1 only after it has read every record of round t,
-// so nobody can still be reading what it overwrites.
+// to the smaller payload) and its row; everyone gets the winner.  Every word that another block reads
+// travels with the round's number in one 128-bit store, and a reader polls until the number is there, so
+// that neither the record nor the row waits for a fence: a round costs one trip to the L2 for the records
+// and one for the winner's row.  Two alternating sets of records and rows: a block publishes round t + 1
+// only after it has read all that it needs of round t, and nobody publishes t + 2 before that, so nobody
+// can still be reading what is overwritten.
 constexpr unsigned kNone = 0xffffffffu;
+constexpr long kMvSpins = 4l << 20;  // a poll takes the better part of a microsecond: gives up after seconds
 
-// The exchange's rows: in global memory, or in shared memory when there is one block, so these are
-// generic accesses (volatile: never from the L1 cache).
-__device__ __forceinline__ void put_row(double* p, double v) { *(volatile double*)p = v; }
-__device__ __forceinline__ double get_row(const double* p) { return *(const volatile double*)p; }
+// (generic addresses: the exchange lies in shared memory when there is one block)
+__device__ __forceinline__ void put_tagged(void* p, unsigned long long v, unsigned long long tag) {
+    asm volatile("{ .reg .b128 q; mov.b128 q, {%1, %2}; st.relaxed.gpu.b128 [%0], q; }" ::"l"(p), "l"(v), "l"(tag)
+                 : "memory");
+}
+__device__ __forceinline__ unsigned long long get_tagged(const void* p, unsigned long long* tag) {
+    unsigned long long v;
+    asm volatile("{ .reg .b128 q; ld.relaxed.gpu.b128 q, [%2]; mov.b128 {%0, %1}, q; }"
+                 : "=l"(v), "=l"(*tag)
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
 
-struct Exchange {
-    unsigned long long* rec;  // [2][G][2]
-    double* slots;            // [2][G][m + 1] the candidates' rows, and the row's number
-    int G, m;
-    unsigned t;
-    int* err;
-    unsigned long long* s_key;  // shared [G]
-    unsigned* s_pay;            // shared [G]
-
-    __device__ double* mine() const { return slots + ((size_t)((t + 1) & 1) * G + blockIdx.x) * (m + 1); }
-    __device__ const double* slot(int q) const { return slots + ((size_t)(t & 1) * G + q) * (m + 1); }
-
-    // Publishes (value, payload; kNone: no candidate) after the block's writes to mine(), and waits for
-    // the others' records.  False if a wait gave up.
-    __device__ bool round(double value, unsigned payload) {
-        __syncthreads();
-        ++t;
-        unsigned long long* r = rec + (size_t)(t & 1) * G * 2;
-        const unsigned long long par = (unsigned long long)(((t + 1) >> 1) & 1u) << 63;
-        bool bad = false;
-        if (threadIdx.x == 0) {
-            volatile unsigned long long* w = r + 2 * blockIdx.x;
-            __threadfence();
-            w[0] = ((unsigned long long)__double_as_longlong(value) & 0x7fffffffffffffffull) | par;
-            w[1] = ((unsigned long long)t << 32) | payload;
-        }
-        if (threadIdx.x < G) {
-            volatile unsigned long long* w = r + 2 * threadIdx.x;
-            unsigned long long v = 0, p = 0;
-            long spins = 0;
-            do {  // a poll takes the better part of a microsecond: this gives up after some seconds
-                p = w[1];
-                v = w[0];
-            } while (((unsigned)(p >> 32) != t || (v & 0x8000000000000000ull) != par) && ++spins < (4l << 20));
-            bad = spins >= (4l << 20);
-            __threadfence();
-            s_key[threadIdx.x] = v & 0x7fffffffffffffffull;
-            s_pay[threadIdx.x] = (unsigned)p;
-        }
-        bad = __syncthreads_or(bad);
-        if (bad && threadIdx.x == 0) atomicOr(err, kErrTimeout);
-        return !bad;
-    }
-
-    // The winner of the round (every warp finds it for itself): its block, or -1 if there is none.
-    __device__ int winner(double* value, unsigned* payload) const {
-        unsigned long long bv = 0;
-        unsigned bp = kNone;
-        int bq = -1;
-        for (int q = threadIdx.x & 31; q < G; q += 32) {
-            const unsigned long long v = s_key[q];
-            const unsigned p = s_pay[q];
-            if (p != kNone && (bq < 0 || v > bv || (v == bv && p < bp))) {
-                bv = v;
-                bp = p;
-                bq = q;
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long v = __shfl_xor_sync(0xffffffffu, bv, o);
-            const unsigned p = __shfl_xor_sync(0xffffffffu, bp, o);
-            const int q = __shfl_xor_sync(0xffffffffu, bq, o);
-            if (q >= 0 && (bq < 0 || v > bv || (v == bv && p < bp))) {
-                bv = v;
-                bp = p;
-                bq = q;
-            }
-        }
-        *value = __longlong_as_double((long long)bv);
-        *payload = bp;
-        return bq;
-    }
-};
+// The warp's best (value bits, payload): the largest value, ties to the smaller payload, kNone loses to
+// everything.  Every lane gets it, and the lane that holds it (payloads are distinct).
+__device__ __forceinline__ int warp_best(unsigned long long& v, unsigned& p) {
+    const unsigned hi = p == kNone ? 0u : (unsigned)(v >> 32), lo = p == kNone ? 0u : (unsigned)v;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    const bool top = hi == mh && lo == ml;
+    const unsigned mp = __reduce_min_sync(0xffffffffu, top ? p : kNone);
+    v = ((unsigned long long)mh << 32) | ml;
+    const unsigned who = __ballot_sync(0xffffffffu, top && p == mp);
+    p = mp;
+    return __ffs(who) - 1;
+}
 
 // A block's own rows: w [R][m], their positions, and R numbers for a column of them.
 struct Rows {
     double* w;
     int* pos;
     double* col;
-    int first, R, m;  // rows first .. first + R - 1 of the matrix
-    double* prow;     // shared [m]: the winner's row
+    int first, R, m;          // rows first .. first + R - 1 of the matrix
+    double* prow;             // shared [m]: the winner's row
     unsigned long long* s_v;  // shared [32]: candidates of the warps
     unsigned* s_p;
     int* s_r;
 };
 
-// The block's candidate of a pivot step: largest |w[r][k]| among its rows at positions >= k (ties to
-// the smaller position; NaN is no candidate).  Threads take rows, then the warps' winners are combined.
-// Returns the local row, or -1.
-__device__ int pivot_candidate(const Rows& a, int k, double* value, unsigned* payload) {
+struct Exchange {
+    unsigned long long* rec;    // [2][G][2]: (value bits, round | payload)
+    unsigned long long* slots;  // [2][G][m + 2][2]: the candidates' rows, the row's number, 1 / pivot
+    int G, m;
+    unsigned t;
+    int* err;
+    unsigned long long* s_win;  // shared [3]: the winner's value, payload, block (-1: none, -2: gave up)
+
+    __device__ unsigned long long* slot(int q) const {
+        return slots + ((size_t)(t & 1) * G + q) * (m + 2) * 2;
+    }
+    __device__ void send(int c, double v) const {
+        put_tagged(slot(blockIdx.x) + 2 * c, (unsigned long long)__double_as_longlong(v), t);
+    }
+    // entry c of block q's row; *bad if it never comes
+    __device__ double receive(int q, int c, bool* bad) const {
+        unsigned long long tag, v;
+        long spins = 0;
+        do {
+            v = get_tagged(slot(q) + 2 * c, &tag);
+        } while (tag != t && ++spins < kMvSpins);
+        if (tag != t) *bad = true;
+        return __longlong_as_double((long long)v);
+    }
+    // the same, or a negative number if it is not there yet
+    __device__ double peek(int q, int c) const {
+        unsigned long long tag;
+        const unsigned long long v = get_tagged(slot(q) + 2 * c, &tag);
+        return tag == t ? __longlong_as_double((long long)v) : -1.0;
+    }
+    // (one thread) this block's record of the round
+    __device__ void publish(unsigned long long v, unsigned payload) const {
+        put_tagged(rec + ((size_t)(t & 1) * G + blockIdx.x) * 2, v, ((unsigned long long)t << 32) | payload);
+    }
+    // (one warp) all blocks' records: the winner into s_win
+    __device__ void poll() const {
+        unsigned long long bv = 0;
+        unsigned bp = kNone;
+        int bq = -1;
+        bool bad = false;
+        constexpr int kEach = 8;  // records a lane polls at once (256 blocks; more take turns)
+        for (int q0 = threadIdx.x & 31; q0 < G; q0 += 32 * kEach) {
+            unsigned long long v[kEach], w[kEach];
+            long spins = 0;
+            bool missing;
+            do {  // all loads are on their way before the first is looked at
+                missing = false;
+#pragma unroll
+                for (int u = 0; u < kEach; ++u)
+                    if (q0 + 32 * u < G) v[u] = get_tagged(rec + ((size_t)(t & 1) * G + q0 + 32 * u) * 2, &w[u]);
+#pragma unroll
+                for (int u = 0; u < kEach; ++u)
+                    if (q0 + 32 * u < G) missing = missing || (unsigned)(w[u] >> 32) != t;
+            } while (missing && ++spins < kMvSpins);
+            bad = bad || missing;
+#pragma unroll
+            for (int u = 0; u < kEach; ++u) {
+                const unsigned p = (unsigned)w[u];
+                if (q0 + 32 * u < G && p != kNone && (bq < 0 || v[u] > bv || (v[u] == bv && p < bp))) {
+                    bv = v[u];
+                    bp = p;
+                    bq = q0 + 32 * u;
+                }
+            }
+        }
+        bad = __any_sync(0xffffffffu, bad);
+        const int who = warp_best(bv, bp);
+        bq = __shfl_sync(0xffffffffu, bq, who);
+        if ((threadIdx.x & 31) == 0) {
+            s_win[0] = bv;
+            s_win[1] = bp;
+            s_win[2] = (unsigned long long)(long long)(bad ? -2 : bq);
+            if (bad) atomicOr(err, kErrTimeout);
+        }
+    }
+    // The round's end for the block, after warp 0 published: the winner's block, or -1, or -2.
+    __device__ int winner(double* value, unsigned* payload) const {
+        if ((threadIdx.x >> 5) == 1) poll();
+        __syncthreads();
+        *value = __longlong_as_double((long long)s_win[0]);
+        *payload = (unsigned)s_win[1];
+        return (int)(long long)s_win[2];
+    }
+    // Waits until every block has come here; what the blocks wrote before is visible after.
+    __device__ bool barrier() {
+        ++t;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            publish(0, kNone);
+        }
+        double v;
+        unsigned p;
+        const int q = winner(&v, &p);
+        __threadfence();
+        __syncthreads();
+        return q != -2;
+    }
+};
+
+// The candidate of a pivot step: largest |w[r][k]| among the block's rows at positions >= k (ties to the
+// smaller position; NaN is no candidate).  Warp 0 publishes it with its row from column c0 on and, while
+// the record travels, the reciprocal of the pivot.  The block is in step before and after is not.
+__device__ void publish_pivot(Exchange& x, const Rows& a, int k, int c0) {
+    ++x.t;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     unsigned long long bv = 0;
     unsigned bp = kNone;
     int br = -1;
-    auto take = [&](unsigned long long v, unsigned p, int r) {
-        if (r >= 0 && (br < 0 || v > bv || (v == bv && p < bp))) {
-            bv = v;
-            bp = p;
-            br = r;
-        }
-    };
-    auto across = [&]() {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long v = __shfl_xor_sync(0xffffffffu, bv, o);
-            const unsigned p = __shfl_xor_sync(0xffffffffu, bp, o);
-            const int r = __shfl_xor_sync(0xffffffffu, br, o);
-            take(v, p, r);
-        }
-    };
-    const int warps = (a.R + 31) >> 5 < (int)(blockDim.x >> 5) ? (a.R + 31) >> 5 : (int)(blockDim.x >> 5);
-    if ((int)(threadIdx.x >> 5) < warps) {
-        for (int r = threadIdx.x; r < a.R; r += warps * 32) {
+    auto scan = [&](int from, int step) {
+        for (int r = from; r < a.R; r += step) {
             const int p = a.pos[r];
             const unsigned long long v =
                 (unsigned long long)__double_as_longlong(a.w[(size_t)r * a.m + k]) & 0x7fffffffffffffffull;
-            if (p >= k && v <= 0x7ff0000000000000ull) take(v, (unsigned)p, r);
+            if (p >= k && v <= 0x7ff0000000000000ull && (br < 0 || v > bv || (v == bv && (unsigned)p < bp))) {
+                bv = v;
+                bp = (unsigned)p;
+                br = r;
+            }
         }
-        across();
-        if ((threadIdx.x & 31) == 0) {
-            a.s_v[threadIdx.x >> 5] = bv;
-            a.s_p[threadIdx.x >> 5] = bp;
-            a.s_r[threadIdx.x >> 5] = br;
+    };
+    if (a.R > 64) {  // many rows: every warp takes a share first
+        scan(threadIdx.x, blockDim.x);
+        const int who = warp_best(bv, bp);
+        br = __shfl_sync(0xffffffffu, br, who);
+        if (lane == 0) {
+            a.s_v[warp] = bv;
+            a.s_p[warp] = bp;
+            a.s_r[warp] = br;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            bv = lane < nw ? a.s_v[lane] : 0;
+            bp = lane < nw ? a.s_p[lane] : kNone;
+            br = lane < nw ? a.s_r[lane] : -1;
+        }
+    } else if (warp == 0) {
+        scan(lane, 32);
+    }
+    if (warp == 0) {
+        const int who = warp_best(bv, bp);
+        br = __shfl_sync(0xffffffffu, br, who);
+        if (lane == 0) x.publish(bv, bp);
+        if (bp != kNone) {
+            const double* row = a.w + (size_t)br * a.m;
+            for (int c = c0 + lane; c < a.m; c += 32) x.send(c, row[c]);
+            if (lane == 0) x.send(a.m, (double)(a.first + br));
+            if (lane == 1) x.send(a.m + 1, 1.0 / row[k]);
         }
     }
-    __syncthreads();
-    br = -1;
-    bp = kNone;
-    for (int q = 0; q < warps; ++q) take(a.s_v[q], a.s_p[q], a.s_r[q]);
-    *value = __longlong_as_double((long long)bv);
-    *payload = br < 0 ? kNone : bp;
-    return br;
 }
 
 // w[r][c] <- w[r][c] - col[r] prow[c] for the block's rows that keep(r) takes and columns c0 <= c < m;
@@ -236,24 +293,18 @@ __device__ bool invert_rows(Exchange& x, Rows& a, int* orig, double* Ai, int* st
     for (int r = tid; r < a.R; r += nt) a.pos[r] = a.first + r;
     __syncthreads();
     for (int k = 0; k < m; ++k) {
+        publish_pivot(x, a, k, 0);
         double v;
         unsigned p;
-        const int br = pivot_candidate(a, k, &v, &p);
-        if (br >= 0) {
-            double* out = x.mine();
-            for (int c = tid; c < m; c += nt) put_row(out + c, a.w[(size_t)br * m + c]);
-            if (tid == 0) put_row(out + m, (double)(a.first + br));
-        }
-        if (!x.round(v, p)) return false;
         const int q = x.winner(&v, &p);
         if (q < 0 || v == 0.0) {
-            if (tid == 0 && blockIdx.x == 0) atomicOr(status, kErrSingular);
+            if (q != -2 && tid == 0 && blockIdx.x == 0) atomicOr(status, kErrSingular);
             return false;
         }
-        const double* in = x.slot(q);
-        const double inv = 1.0 / get_row(in + k);
-        for (int c = tid; c < m; c += nt) a.prow[c] = c == k ? inv : get_row(in + c) * inv;
-        if (tid == 0) orig[k] = (int)get_row(in + m);
+        bool bad = false;
+        const double inv = x.receive(q, m + 1, &bad);
+        for (int c = tid; c < m; c += nt) a.prow[c] = c == k ? inv : x.receive(q, c, &bad) * inv;
+        if (tid == nt - 1) orig[k] = (int)x.receive(q, m, &bad);
         for (int r = tid; r < a.R; r += nt) {
             if (a.pos[r] == (int)p)
                 a.pos[r] = k;
@@ -262,10 +313,15 @@ __device__ bool invert_rows(Exchange& x, Rows& a, int* orig, double* Ai, int* st
             a.col[r] = a.w[(size_t)r * m + k];
             a.w[(size_t)r * m + k] = 0.0;  // the eliminated column; the new column of the inverse grows here
         }
-        __syncthreads();
+        if (__syncthreads_or(bad)) {
+            if (bad) atomicOr(x.err, kErrTimeout);
+            return false;
+        }
         rank_one(a, 0, [&](int r) { return a.pos[r] != k; }, [](double, int, int) {});
         if (q == (int)blockIdx.x)
-            for (int c = tid; c < m; c += nt) a.w[(size_t)br * m + c] = a.prow[c];
+            for (int r = 0; r < a.R; ++r)
+                if (a.pos[r] == k)
+                    for (int c = tid; c < m; c += nt) a.w[(size_t)r * m + c] = a.prow[c];
         __syncthreads();
     }
     for (int e = tid; e < a.R * m; e += nt) {
@@ -275,8 +331,8 @@ __device__ bool invert_rows(Exchange& x, Rows& a, int* orig, double* Ai, int* st
     return true;
 }
 
-// Shared memory of the cooperative kernels, in order: exchange keys and payloads [G], warps' candidates,
-// (G == 1: records and slots), prow [m], orig [m], then for k_maxvol D [m], sel [m] and a chunk of B, and
+// Shared memory of the cooperative kernels, in order: the winner, the warps' candidates,
+// (G == 1: records and rows of the exchange), prow [m], orig [m], then for k_maxvol D [m], sel [m] and a chunk of B, and
 // the block's rows with their positions and column when those fit.
 struct Layout {
     int G, R, br;          // blocks, rows of a block at most, rows of B in a chunk
@@ -292,7 +348,7 @@ inline Layout mv_layout(int n, int m, int G, bool full) {
     l.G = G;
     l.R = mv_rows(n > m ? n : m, G);
     l.br = full ? (m <= 1024 ? 8 : 1) : 0;
-    size_t b = 16 * (size_t)((G + 1) / 2 * 2) + 32 * 16 + (G == 1 ? 8 * (size_t)(4 + 2 * (m + 1)) : 0);
+    size_t b = 32 + 32 * 16 + (G == 1 ? 32 + 32 * (size_t)(m + 2) : 0);
     b += 8 * (size_t)m + 8 * (size_t)m;                                     // prow, orig (8-byte slots)
     if (full) b += 8 * (size_t)m + 8 * (size_t)m + 8 * (size_t)m * l.br;    // D, sel, chunk
     l.col_in = b + 16 * (size_t)l.R <= kMvSharedMost;
@@ -314,15 +370,14 @@ struct Carve {
 };
 
 __device__ void carve_common(Carve& s, Exchange& x, Rows& a, int** orig) {
-    x.s_key = s.take<unsigned long long>(x.G);
-    x.s_pay = s.take<unsigned>(x.G);
+    x.s_win = s.take<unsigned long long>(4);
     a.s_v = s.take<unsigned long long>(32);
     a.s_p = s.take<unsigned>(32);
     a.s_r = s.take<int>(32);
-    if (x.G == 1) {
+    if (x.G == 1) {  // (16-byte aligned: everything before is a multiple of 32 bytes)
         x.rec = s.take<unsigned long long>(4);
-        x.slots = s.take<double>(2 * (x.m + 1));
-        if (threadIdx.x < 4) x.rec[threadIdx.x] = 0;
+        x.slots = s.take<unsigned long long>(4 * (size_t)(x.m + 2));
+        for (int e = threadIdx.x; e < 4 + 4 * (x.m + 2); e += blockDim.x) x.rec[e] = 0;
     }
     a.prow = s.take<double>(x.m);
     *orig = s.take<int>(2 * x.m);
@@ -336,8 +391,9 @@ struct MaxvolArgs {
     double* col;               // [max(n, m)], likewise
     int* pos;                  // [n], likewise
     unsigned long long* rec;   // [2][G][2], zero at the start (G > 1)
+    unsigned long long* slots; // [2][G][m + 2][2], zero at the start (G > 1); may lie in A
     int* sel;                  // [m]
-    double* A;                 // [m][m]; holds the exchange's rows until the end
+    double* A;                 // [m][m]
     double* Ai;                // [m][m]
     double tol;
     int max_iter, start_given;
@@ -349,7 +405,7 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x, nt = blockDim.x, n = g.n, m = g.m;
     Carve sh{smem};
-    Exchange x{g.rec, g.A, g.G, m, 0u, g.status, nullptr, nullptr};
+    Exchange x{g.rec, g.slots, g.G, m, 0u, g.status, nullptr};
     Rows a{};
     int* orig;
     carve_common(sh, x, a, &orig);
@@ -371,19 +427,35 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
     own(n, Rn);
     __syncthreads();
     // 0. column equilibration: the largest |column| of the block's rows, then of all blocks'
+    ++x.t;
     for (int c = tid; c < m; c += nt) {
         double mx = 0.0;
         for (int r = 0; r < a.R; ++r) mx = fmax(mx, fabs(g.B[(size_t)(a.first + r) * m + c]));
-        put_row(x.mine() + c, mx);
+        x.send(c, mx);
     }
-    if (!x.round(0.0, kNone)) return;
-    bool zero = false;
+    if (tid == 0) x.publish(0, kNone);
+    {
+        double v;
+        unsigned p;
+        if (x.winner(&v, &p) == -2) return;
+    }
+    bool zero = false, late = false;
     for (int c = tid; c < m; c += nt) {
         double mx = 0.0;
-#pragma unroll 8
-        for (int q = 0; q < g.G; ++q) mx = fmax(mx, get_row(x.slot(q) + c));
+        for (int q0 = 0; q0 < g.G; q0 += 8) {  // eight on their way at once
+            double each[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) each[u] = x.peek(min(q0 + u, g.G - 1), c);
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                mx = fmax(mx, each[u] >= 0.0 ? each[u] : x.receive(min(q0 + u, g.G - 1), c, &late));
+        }
         D[c] = mx > 0.0 ? 1.0 / mx : 0.0;
         zero = zero || D[c] == 0.0;
+    }
+    if (__syncthreads_or(late)) {
+        if (late) atomicOr(g.status, kErrTimeout);
+        return;
     }
     if (__syncthreads_or(zero)) {
         if (tid == 0 && blockIdx.x == 0) atomicOr(g.status, kErrSingular);
@@ -397,32 +469,29 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
         for (int r = tid; r < a.R; r += nt) a.pos[r] = a.first + r;
         __syncthreads();
         for (int k = 0; k < m; ++k) {
+            publish_pivot(x, a, k, k + 1);
             double v;
             unsigned p;
-            const int br = pivot_candidate(a, k, &v, &p);
-            if (br >= 0) {
-                double* out = x.mine();
-                for (int c = k + tid; c < m; c += nt) put_row(out + c, a.w[(size_t)br * m + c]);
-                if (tid == 0) put_row(out + m, (double)(a.first + br));
-            }
-            if (!x.round(v, p)) return;
             const int q = x.winner(&v, &p);
             if (q < 0 || v == 0.0) {
-                if (tid == 0 && blockIdx.x == 0) atomicOr(g.status, kErrSingular);
+                if (q != -2 && tid == 0 && blockIdx.x == 0) atomicOr(g.status, kErrSingular);
                 return;
             }
-            const double* in = x.slot(q);
-            const double piv = get_row(in + k);
-            for (int c = k + 1 + tid; c < m; c += nt) a.prow[c] = get_row(in + c);
-            if (tid == 0) sel[k] = (int)get_row(in + m);
+            bool bad = false;
+            for (int c = k + 1 + tid; c < m; c += nt) a.prow[c] = x.receive(q, c, &bad);
+            if (tid == nt - 1) sel[k] = (int)x.receive(q, m, &bad);
+            const double inv = tid < a.R ? x.receive(q, m + 1, &bad) : 0.0;
             for (int r = tid; r < a.R; r += nt) {
                 if (a.pos[r] == (int)p)
                     a.pos[r] = k;
                 else if (a.pos[r] == k)
                     a.pos[r] = (int)p;
-                a.col[r] = a.w[(size_t)r * m + k] / piv;
+                a.col[r] = a.w[(size_t)r * m + k] * inv;
             }
-            __syncthreads();
+            if (__syncthreads_or(bad)) {
+                if (bad) atomicOr(g.status, kErrTimeout);
+                return;
+            }
             rank_one(a, k + 1, [&](int r) { return a.pos[r] > k; }, [](double, int, int) {});
             __syncthreads();
         }
@@ -432,7 +501,7 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
     const auto load = [&](int j, int c) { return g.B[(size_t)sel[j] * m + c] * D[c]; };
     own(m, Rm);
     if (!invert_rows(x, a, orig, g.Ai, g.status, load, [](int) { return 1.0; })) return;
-    if (!x.round(0.0, kNone)) return;  // every block's rows of A^-1 are written
+    if (!x.barrier()) return;  // every block's rows of A^-1 are written
     // 3. C = B A^-1 for the block's rows, a few rows at a time (a thread per column)
     own(n, Rn);
     double best = -1.0;
@@ -468,37 +537,32 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
     int swaps = 0;
     double gm = -1.0;
     for (int it = 0; it <= g.max_iter; ++it) {
-        // the block's largest |C| (ties: the smallest element)
-        for (int o = 16; o > 0; o >>= 1) {
-            const double v = __shfl_xor_sync(0xffffffffu, best, o);
-            const int e = __shfl_xor_sync(0xffffffffu, at, o);
-            if (v > best || (v == best && e < at)) {
-                best = v;
-                at = e;
+        // the block's largest |C| (ties: the smallest element), with its row
+        {
+            unsigned long long bv = best >= 0.0 ? (unsigned long long)__double_as_longlong(best) : 0;
+            unsigned bp = best >= 0.0 ? (unsigned)at : kNone;
+            warp_best(bv, bp);
+            ++x.t;
+            if ((tid & 31) == 0) {
+                a.s_v[tid >> 5] = bv;
+                a.s_p[tid >> 5] = bp;
+            }
+            __syncthreads();  // (and the rows are up to date)
+            if (tid < 32) {
+                bv = tid < nt >> 5 ? a.s_v[tid] : 0;
+                bp = tid < nt >> 5 ? a.s_p[tid] : kNone;
+                warp_best(bv, bp);
+                if (tid == 0) x.publish(bv, bp);
+                if (bp != kNone) {
+                    const double* row = a.w + (size_t)((int)bp / m - a.first) * m;
+                    for (int c = tid; c < m; c += 32) x.send(c, row[c]);
+                }
             }
         }
-        __syncthreads();
-        if ((tid & 31) == 0) {
-            a.s_v[tid >> 5] = (unsigned long long)__double_as_longlong(best);
-            a.s_r[tid >> 5] = at;
-        }
-        __syncthreads();
-        for (int q = 0; q < nt >> 5; ++q) {
-            const double v = __longlong_as_double((long long)a.s_v[q]);
-            if (v > best || (v == best && a.s_r[q] < at)) {
-                best = v;
-                at = a.s_r[q];
-            }
-        }
-        if (best >= 0.0) {
-            double* out = x.mine();
-            const double* row = a.w + (size_t)(at / m - a.first) * m;
-            for (int c = tid; c < m; c += nt) put_row(out + c, row[c]);
-        }
-        if (!x.round(best, best >= 0.0 ? (unsigned)at : kNone)) return;
         unsigned e;
         double v;
         const int q = x.winner(&v, &e);
+        if (q == -2) return;
         gm = q < 0 ? -1.0 : v;
         if (gm <= 1.0 + g.tol) break;
         if (it == g.max_iter) {
@@ -506,23 +570,26 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
             break;
         }
         const int j = (int)e % m;
-        const double* in = x.slot(q);
-        const double ckj = get_row(in + j);
-        for (int c = tid; c < m; c += nt) a.prow[c] = get_row(in + c) - (c == j ? 1.0 : 0.0);
+        bool bad = false;
+        const double ckj = x.receive(q, j, &bad);
+        for (int c = tid; c < m; c += nt) a.prow[c] = x.receive(q, c, &bad) - (c == j ? 1.0 : 0.0);
         for (int r = tid; r < a.R; r += nt) a.col[r] = a.w[(size_t)r * m + j] / ckj;
         if (tid == 0) sel[j] = (int)e / m;
-        __syncthreads();
+        if (__syncthreads_or(bad)) {
+            if (bad) atomicOr(g.status, kErrTimeout);
+            return;
+        }
         best = -1.0;
         at = 0;
         rank_one(a, 0, [](int) { return true; }, [&](double v, int r, int c) { track(v, (a.first + r) * m + c); });
         ++swaps;
     }
     __syncthreads();
-    // A^-1 = D (A D)^-1, computed from scratch, and the unscaled A (over the exchange's rows: after
-    // every block has read the last of them)
+    // A^-1 = D (A D)^-1, computed from scratch, and the unscaled A (possibly over the exchange's rows:
+    // after every block has read the last of them)
     own(m, Rm);
     if (!invert_rows(x, a, orig, g.Ai, g.status, load, [&](int row) { return D[row]; })) return;
-    if (!x.round(0.0, kNone)) return;
+    if (!x.barrier()) return;
     for (int e = tid; e < a.R * m; e += nt)
         g.A[(size_t)a.first * m + e] = g.B[(size_t)sel[a.first + e / m] * m + e % m];
     if (blockIdx.x == 0) {
@@ -595,7 +662,7 @@ struct InvertArgs {
     double* Ai;
     double* rows;             // [m][m] when the rows do not fit in shared memory
     double* col;              // (col_in is always set for m rows)
-    double* slots;            // [2][G][m + 1]
+    unsigned long long* slots;  // [2][G][m + 2][2], zero at the start
     unsigned long long* rec;  // [2][G][2], zero at the start
     int* status;
 };
@@ -604,7 +671,7 @@ __global__ void __launch_bounds__(kMvThreads) k_invert(const InvertArgs g) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int m = g.m, R = mv_rows(m, g.G);
     Carve sh{smem};
-    Exchange x{g.rec, g.slots, g.G, m, 0u, g.status, nullptr, nullptr};
+    Exchange x{g.rec, g.slots, g.G, m, 0u, g.status, nullptr};
     Rows a{};
     int* orig;
     carve_common(sh, x, a, &orig);
@@ -626,51 +693,70 @@ int mv_sm_count() {
     return n > 0 ? n : 1;
 }
 
-// Blocks of a cooperative kernel: as many as have rows to own and room for their exchange rows, one per
-// SM at most (the exchange costs the same for few and for many, the rows of a block set the step's FMAs).
+// Blocks of a cooperative kernel: as many as have two rows of A each and room for their exchange rows, one
+// per SM at most (the exchange costs the same for few and for many, the rows of a block set the step's
+// FMAs).
 int mv_blocks(int m, size_t slot_doubles) {
-    const long by_slots = (long)(slot_doubles / (2 * (size_t)(m + 1)));
+    const long by_slots = (long)(slot_doubles / (4 * (size_t)(m + 2)));
     return (int)std::max(1l, std::min({(long)mv_sm_count(), (long)m / 2, by_slots}));
+}
+size_t mv_slot_bytes(int m, int G) { return 32 * (size_t)G * (m + 2); }
+
+template <class K, class Args>
+int mv_launch(K kernel, Args& g, int G, size_t smem, cudaStream_t st) {
+    if (G > 1 && (cudaMemsetAsync(g.rec, 0, 32 * (size_t)G, st) != cudaSuccess ||
+                  cudaMemsetAsync(g.slots, 0, mv_slot_bytes(g.m, G), st) != cudaSuccess))
+        return -1;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMvSharedMost) != cudaSuccess)
+        return -1;
+    void* args[] = {&g};
+    return cudaLaunchCooperativeKernel((void*)kernel, dim3(G), dim3(kMvThreads), args, smem, st) == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace
 
 // The launchers return the number of kernels launched, or -1 if the launch itself failed (the
 // error is taken off cudaGetLastError, so the caller reports it instead of reading stale results).
-// W: 2 m^2 doubles.
+// W: 2 m^2 + 4 doubles, 16-byte aligned.
 int launch_invert(int m, const double* A, double* Ai, double* W, int* status, cudaStream_t st) {
-    // W = [rows m^2 | records 4 G | slots 2 G (m + 1)]
-    const size_t mm = (size_t)m * m;
-    const int G = mv_blocks(m, mm > 4 * (size_t)(m / 2) ? mm - 4 * (size_t)(m / 2) : 0);
-    const Layout l = mv_layout(m, m, G, false);
-    InvertArgs g{m, G, l.rows_in, l.col_in, A, Ai, W, nullptr, W + mm + 4 * (size_t)G,
-                 reinterpret_cast<unsigned long long*>(W + mm), status};
+    // W = [records 4 G | slots 4 G (m + 2) | rows m^2 if they do not fit in shared memory]
+    const size_t mm = (size_t)m * m, per = 4 + 4 * (size_t)(m + 2);
+    auto blocks = [&](size_t room) {
+        return (int)std::max(1l, std::min({(long)mv_sm_count(), (long)m / 2, (long)(room / per)}));
+    };
+    int G = blocks(2 * mm);
+    Layout l = mv_layout(m, m, G, false);
+    if (!l.rows_in) {
+        G = blocks(mm);
+        l = mv_layout(m, m, G, false);
+    }
     if (!l.col_in || l.bytes > kMvSharedMost) return -1;  // not reachable for the widths of a model
-    if (G > 1 && cudaMemsetAsync(g.rec, 0, 32 * (size_t)G, st) != cudaSuccess) return -1;
-    if (cudaFuncSetAttribute(k_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMvSharedMost) != cudaSuccess)
-        return -1;
-    void* args[] = {&g};
-    return cudaLaunchCooperativeKernel((void*)k_invert, dim3(G), dim3(kMvThreads), args, l.bytes, st) == cudaSuccess
-               ? 1 : -1;
+    auto* rec = reinterpret_cast<unsigned long long*>(W);
+    InvertArgs g{m, G, l.rows_in, l.col_in, A, Ai, W + mm, nullptr, rec + 4 * (size_t)G, rec, status};
+    return mv_launch(k_invert, g, G, l.bytes, st);
 }
 
-// W: max(n m, 2 m^2) + 2 m + n doubles, pos: n ints.
+// W: max(n m, 2 m^2) + 2 m + n doubles, 16-byte aligned, pos: n ints.
 int launch_maxvol(int n, int m, const double* B, double* W, int* pos, int* sel, double* A, double* Ai, double tol,
                   int max_iter, int* status, int* swaps, double* gmax, cudaStream_t st, int start_given) {
     const size_t nm = (size_t)n * m, mm = (size_t)m * m;
-    const int G = mv_blocks(m, mm);  // the exchange's rows lie in A until the end; records: 4 G <= 2 m doubles
-    const Layout l = mv_layout(n, m, G, true);
+    // records at the start of W (4 G <= 2 m doubles); then the exchange's rows, where the matrix's rows
+    // are in shared memory, else the matrix's rows and column, with the exchange's rows in A
+    int G = mv_blocks(m, std::max(nm, 2 * mm));
+    Layout l = mv_layout(n, m, G, true);
+    const bool in = l.rows_in && l.col_in;
+    if (!in) {
+        G = mv_blocks(m, mm - 1);  // (A need not be 16-byte aligned)
+        l = mv_layout(n, m, G, true);
+    }
     if (l.bytes > kMvSharedMost) return -1;  // not reachable for the widths of a model
-    double* tail = W + std::max(nm, 2 * mm);
-    MaxvolArgs g{n, m, G, l.br, l.rows_in, l.col_in, B, W, tail + 2 * (size_t)m, pos,
-                 reinterpret_cast<unsigned long long*>(tail), sel, A, Ai, tol, max_iter, start_given, status, swaps,
-                 gmax};
-    if (G > 1 && cudaMemsetAsync(g.rec, 0, 32 * (size_t)G, st) != cudaSuccess) return -1;
-    if (cudaFuncSetAttribute(k_maxvol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMvSharedMost) != cudaSuccess)
-        return -1;
-    void* args[] = {&g};
-    return cudaLaunchCooperativeKernel((void*)k_maxvol, dim3(G), dim3(kMvThreads), args, l.bytes, st) == cudaSuccess
-               ? 1 : -1;
+    auto* rec = reinterpret_cast<unsigned long long*>(W);
+    double* rest = W + 2 * (size_t)m;
+    auto* in_A = reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(A) + 15) & ~(uintptr_t)15);
+    MaxvolArgs g{n, m, G, l.br, l.rows_in, l.col_in, B, rest, rest + std::max(nm, 2 * mm), pos, rec,
+                 in ? reinterpret_cast<unsigned long long*>(rest) : in_A, sel, A, Ai, tol, max_iter, start_given, status,
+                 swaps, gmax};
+    return mv_launch(k_maxvol, g, G, l.bytes, st);
 }
 
 __global__ void k_gather_columns(int rows, int w_in, const double* in, int w_out, const int* cols, double* out) {
