@@ -602,7 +602,9 @@ def _closure(monos):
 # channel (_grad_terms_folded): measured on GB300 at lev_max 20, 10% fewer instructions and 7% less
 # time in the pair-gradient kernel (126 registers either way).  At lev_max 16 the extra partial sums
 # cost registers (124 instead of 72 per thread with eight lanes per atom) and the time was unchanged
-# within the run-to-run spread, so lower levels keep one multiplication per term.
+# within the run-to-run spread, so lower levels keep one multiplication per term.  The double adjoints
+# are folded at every level: the double-precision pipe is their bound, and 509 cells at lev_max 16 went
+# from 3.99 to 3.66 ms.
 FOLD_GRAD_MIN_LEVEL = 18
 
 
@@ -739,7 +741,7 @@ def emit_slice_functions(prog: Program, slc, tag, slot_begin=None):
         for mu in mus:
             out.append(f"    const T P{mu} = " + " + ".join(p_terms[mu]) + ";")
         out.append("    s += " + " + ".join(f"df[{mu}] * P{mu}" for mu in mus) + ";")
-        if tag == "f" and prog.L >= FOLD_GRAD_MIN_LEVEL:
+        if tag == "d" or prog.L >= FOLD_GRAD_MIN_LEVEL:  # (in double every multiplication counts)
             out += ["    " + l for l in _grad_terms_folded(monos, by_m)]
         else:
             for m in monos:
