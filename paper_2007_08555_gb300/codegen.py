@@ -668,6 +668,79 @@ def _grad_terms_folded(monos, by_m):
     return decl + body + fin
 
 
+def horner_order(prog: Program):
+    """Components in the order the nested Horner scheme takes them (z, then y, then x exponents, each from
+    the highest down; the radial channels of a monomial side by side): a permutation of range(C)."""
+    return sorted(range(len(prog.comp_list)), key=lambda t: (-prog.comp_list[t][1][2], -prog.comp_list[t][1][1],
+                                                            -prog.comp_list[t][1][0], prog.comp_list[t][0]))
+
+
+def emit_horner(prog: Program, slot_begin):
+    """struct HornerF: the adjoint of one pair over every component, by nested Horner schemes.  With
+    alpha_m = sum_mu f_mu adj[mu, m] and beta_m = sum_mu df_mu adj[mu, m] the pair's terms are the gradient
+    of the polynomial sum alpha_m m and the value of sum beta_m m in (x, y, z); Horner's scheme in x inside
+    y inside z needs no monomials (a handful of running values instead of up to 165 registers of
+    monomials: 72 registers a thread instead of 254 at lev_max 20), and reads dV/dM in the one order in
+    which adj_to_shared lays it down.  The force-gradient phase, slices of components against this: lev_max
+    20, 1,048,576 atoms 4.12 against 3.84 ms, 16,384 atoms 104 against 85 us; lev_max 16, 393,000 atoms 447
+    against 404 us; lev_max 12, 104,000 atoms 60.6 against 57.5 us; lev_max 10 equal."""
+    order = horner_order(prog)
+    pos = {t: q for q, t in enumerate(order)}
+    out = ["struct HornerF {"]
+    out.append("  template <class T, int TPA, int NS> static __device__ __forceinline__ void adj_to_shared("
+               "const T* __restrict__ sl, T* __restrict__ dst, const int sub) {")
+    for t in range(len(order)):  # slots in memory order, a component by the lane with t % TPA == sub
+        terms = [f"sl[{s * 32}]" for s in range(slot_begin[t], slot_begin[t + 1])] or ["T(0)"]
+        q = pos[t]
+        out.append(f"    if ({t} % TPA == sub) dst[{q // 4} * 4 * NS + {q % 4}] = " + " + ".join(terms) + ";")
+        out.append(f'    if ({t + 1} % (16 * TPA) == 0) asm volatile("" ::: "memory");')
+    out.append("  }")
+    out.append("  template <class T, class A> static __device__ __forceinline__ void grad(const T x, const T y, const T z, "
+               "const T* __restrict__ f, const T* __restrict__ df, const A adj, T& s, T& gx, T& gy, T& gz) {")
+    by = defaultdict(list)
+    for t in order:
+        mu, m = prog.comp_list[t]
+        by[m].append((pos[t], mu))
+    L = out.append
+
+    def step(name, var, terms, first):
+        """name <- name * var + terms (terms: a list of products)"""
+        if first:
+            return f"{name} = " + " + ".join(terms) + ";"
+        return f"{name} = " + " + ".join([f"{name} * {var}"] + terms) + ";"
+
+    zs = sorted({m[2] for m in by}, reverse=True)
+    L("    T V = T(0), Vx = T(0), Vy = T(0), Vz = T(0), B = T(0);")
+    for iz, c in enumerate(zs):
+        assert c == zs[0] - iz
+        ys = sorted({m[1] for m in by if m[2] == c}, reverse=True)
+        L("    { T U = T(0), Ux = T(0), Uy = T(0), W = T(0);")
+        for iy, b in enumerate(ys):
+            assert b == ys[0] - iy
+            xs = sorted({m[0] for m in by if m[2] == c and m[1] == b}, reverse=True)
+            L("      { T u = T(0), ux = T(0), w = T(0);")
+            for ix, a in enumerate(xs):
+                assert a == xs[0] - ix
+                terms = by[(a, b, c)]
+                if ix > 0:
+                    L("        ux = " + ("ux * x + u;" if ix > 1 else "u;"))
+                L("        { " + " ".join(f"const T a{q} = adj[{q}];" for q, _ in terms))
+                L("          " + step("u", "x", [f"f[{mu}] * a{q}" for q, mu in terms], ix == 0))
+                L("          " + step("w", "x", [f"df[{mu}] * a{q}" for q, mu in terms], ix == 0) + " }")
+            if iy > 0:
+                L("        Uy = " + ("Uy * y + U;" if iy > 1 else "U;"))
+            L("        U = " + ("u;" if iy == 0 else "U * y + u;") + " Ux = " + ("ux;" if iy == 0 else "Ux * y + ux;")
+              + " W = " + ("w;" if iy == 0 else "W * y + w;") + " }")
+        if iz > 0:
+            L("      Vz = " + ("Vz * z + V;" if iz > 1 else "V;"))
+        L("      V = " + ("U;" if iz == 0 else "V * z + U;") + " Vx = " + ("Ux;" if iz == 0 else "Vx * z + Ux;") + " Vy = "
+          + ("Uy;" if iz == 0 else "Vy * z + Uy;") + " B = " + ("W;" if iz == 0 else "B * z + W;") + " }")
+    L("    s += B; gx += Vx; gy += Vy; gz += Vz;")
+    L("  }")
+    out.append("};")
+    return out
+
+
 def _mom_function(prog: Program, monos, comps):
     """mom(x, y, z, f, acc) of one slice: acc[t] += f[mu] x^a y^b z^c for its components (Eq. 5 for
     one neighbour)."""
@@ -1135,8 +1208,11 @@ def emit_level(L, outdir):
         lines += dual_lines
     else:
         lines.append("#define MTPGEN_HAS_PARTS 0")
+    lines.append(f"#define MTPGEN_HORNER {int(has_parts)}")
     lines.append(f"#define MTPGEN_HAS_PARTS64 {int(has_parts and L <= UNROLLED_MAX_LEVEL_F64)}")
     lines += emit_slice_functions(prog, s32, "f", slot_begin if has_parts else None)
+    if has_parts:
+        lines += emit_horner(prog, slot_begin)
     lines += emit_slice_functions(prog, s64, "d", slot_begin if has_parts and L <= UNROLLED_MAX_LEVEL_F64 else None)
     lines += emit_slice_functions(prog, sm32, "mf")
     lines += emit_slice_functions(prog, sm64, "md")

@@ -725,7 +725,9 @@ __device__ __forceinline__ void adj_tile_to_shared(const T* src, int size, T* mi
 // fit beside the coefficients at the largest sizes, so the slices take turns.
 template <class T, int TPA>
 struct PairgradMerged {
-    static constexpr bool value = PairgradShared<T>::value && TPA >= (sizeof(T) == 4 ? 2 : 4) && NumSlices<T>::value > 1;
+    static constexpr bool horner = MTPGEN_HORNER && sizeof(T) == 4 && TPA >= 2;  // (emit_horner in codegen.py)
+    static constexpr bool value =
+        horner || (PairgradShared<T>::value && TPA >= (sizeof(T) == 4 ? 2 : 4) && NumSlices<T>::value > 1);
 };
 
 template <class T, int TPA>
@@ -829,8 +831,12 @@ __device__ __forceinline__ void pairgrad_merged(const EvalCtx<T>& a, int i, int 
     constexpr int NSA = 128 / TPA;
     T* mine = sadj + 4 * (threadIdx.x / TPA);
     __syncwarp();  // the atom's lanes are done with the previous atom
+    constexpr bool kHorner = PairgradMerged<T, TPA>::horner;
     if (active) {
-        if constexpr (HasParts<T>::value)
+        if constexpr (kHorner)
+            ::MTP_GEN_NS::HornerF::adj_to_shared<T, TPA, NSA>(
+                a.aslots + (size_t)(i >> 5) * G::NSLOT_ * 32 + (i & 31), mine, sub);
+        else if constexpr (HasParts<T>::value)
             adj_all_to_shared<T, 0, TPA, NSA>(a.aslots + (size_t)(i >> 5) * G::NSLOT_ * 32 + (i & 31), mine, sub);
         else
             adj_tile_to_shared<T, TPA, NSA, 0>(a.adjm + (size_t)(i >> 5) * G::C_ * 32 + (i & 31), G::C_, mine, sub);
@@ -852,7 +858,10 @@ __device__ __forceinline__ void pairgrad_merged(const EvalCtx<T>& a, int i, int 
         T f[G::NMU_], df[G::NMU_];
         radial<T, true>(r, cs + (zi * a.S + cur.zj) * csz, a.NQ, a.rmin, a.rcut, a.inv_span, f, df);
         T s = T(0), gx = T(0), gy = T(0), gz = T(0);
-        grad_all_slices<T, 0, NSA>(x, y, z, f, df, q, s, gx, gy, gz);
+        if constexpr (kHorner)
+            ::MTP_GEN_NS::HornerF::grad<T>(x, y, z, f, df, SharedAdj<T, NSA>{q}, s, gx, gy, gz);
+        else
+            grad_all_slices<T, 0, NSA>(x, y, z, f, df, q, s, gx, gy, gz);
         const T sr = len.over(s);
         a.g[idx] = Vec4<T>{gx + sr * x, gy + sr * y, gz + sr * z, T(0)};
     }
