@@ -265,9 +265,10 @@ mtp_status fill_ctx(mtp_model* M, int K, int n, const int* cfg_off, const int* t
     // (float: two lanes for the pair kernels at any size -- they visit every pair once and read dV/dM from
     // shared memory, one lane per atom costs 4-12% of an evaluation from 77k atoms on: 442k atoms 4.07 ms
     // against 3.77 at lev_max 16, 7.3 against 6.6 at 20; and two for the moments up to lev_max 16, where a
-    // lane's running sums leave room for more warps: 0-5%, 55k atoms 0.468 against 0.446 ms)
+    // lane's running sums leave room for more warps: 0-5%, 55k atoms 0.468 against 0.446 ms, and below
+    // 100k atoms at any level: 70k at lev_max 18 150 against 129 us of the moments)
     // double: four lanes, from which on every pair is visited once
-    const int least = sizeof(T) == 4 ? 2 : 4, least_m = sizeof(T) == 4 && M->L <= 16 ? 2 : 1;
+    const int least = sizeof(T) == 4 ? 2 : 4, least_m = sizeof(T) == 4 && (M->L <= 16 || n < 100000) ? 2 : 1;
     a.tpa = M->tpa_pairs ? M->tpa_pairs : (t.second ? t.second : std::max(least, choose_tpa(n, M->n_sm, 512)));
     a.tpa_m = M->tpa_moments ? M->tpa_moments : (t.first ? t.first : std::max(least_m, choose_tpa(n, M->n_sm, 128)));
     a.mom = M->mom.as<T>();
