@@ -693,12 +693,13 @@ int mv_sm_count() {
     return n > 0 ? n : 1;
 }
 
-// Blocks of a cooperative kernel: as many as have two rows of A each and room for their exchange rows, one
-// per SM at most (the exchange costs the same for few and for many, the rows of a block set the step's
-// FMAs).
+// Blocks of a cooperative kernel: as many as have two rows of A each and room for their exchange rows, two
+// for three SMs at most: fewer blocks take longer over their rows, more of them over the exchange (920 x 460:
+// 10.2 ms with 32 blocks, 7.5 with 64, 6.8 with 100, 7.6 with 128, 8.7 with 152; 232 x 116: 1.73 ms with 8,
+// 1.37 with 32, 1.31 with 58).
 int mv_blocks(int m, size_t slot_doubles) {
     const long by_slots = (long)(slot_doubles / (4 * (size_t)(m + 2)));
-    return (int)std::max(1l, std::min({(long)mv_sm_count(), (long)m / 2, by_slots}));
+    return (int)std::max(1l, std::min({(long)mv_sm_count() * 2 / 3, (long)m / 2, by_slots}));
 }
 size_t mv_slot_bytes(int m, int G) { return 32 * (size_t)G * (m + 2); }
 
@@ -722,7 +723,7 @@ int launch_invert(int m, const double* A, double* Ai, double* W, int* status, cu
     // W = [records 4 G | slots 4 G (m + 2) | rows m^2 if they do not fit in shared memory]
     const size_t mm = (size_t)m * m, per = 4 + 4 * (size_t)(m + 2);
     auto blocks = [&](size_t room) {
-        return (int)std::max(1l, std::min({(long)mv_sm_count(), (long)m / 2, (long)(room / per)}));
+        return (int)std::max(1l, std::min({(long)mv_sm_count() * 2 / 3, (long)m / 2, (long)(room / per)}));
     };
     int G = blocks(2 * mm);
     Layout l = mv_layout(m, m, G, false);
