@@ -696,7 +696,8 @@ int mv_sm_count() {
 // Blocks of a cooperative kernel: as many as have two rows of A each and room for their exchange rows, two
 // for three SMs at most: fewer blocks take longer over their rows, more of them over the exchange (920 x 460:
 // 10.2 ms with 32 blocks, 7.5 with 64, 6.8 with 100, 7.6 with 128, 8.7 with 152; 232 x 116: 1.73 ms with 8,
-// 1.37 with 32, 1.31 with 58).
+// 1.37 with 32, 1.31 with 58).  Where the exchange rows lie in memory matters too: of eight allocations seven
+// gave 6.7 against 8.5 ms, one 7.4 ms with either number of blocks.
 int mv_blocks(int m, size_t slot_doubles) {
     const long by_slots = (long)(slot_doubles / (4 * (size_t)(m + 2)));
     return (int)std::max(1l, std::min({(long)mv_sm_count() * 2 / 3, (long)m / 2, by_slots}));

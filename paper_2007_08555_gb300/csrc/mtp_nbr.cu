@@ -347,6 +347,7 @@ constexpr int kBias3 = 0x808080;  // three zero components
 // then per warp the accepted keys and the lattice shift of the neighbour's bin of each.
 constexpr int kBuildThreads = 128, kBuildWarps = kBuildThreads / 32;
 constexpr int kGroup = kBuildThreads;  // neighbour bins described per staging round
+constexpr int kStageEach = 4;          // candidates a thread stages at once
 constexpr int kChunk = 640;            // candidates staged at once
 constexpr float kCullMargin = 0.05f;   // float error of positions against their bin's box, Angstrom
 constexpr size_t kSmCpos = 0;
@@ -374,7 +375,8 @@ size_t build_smem(int cap) { return kSmWarp + (size_t)kBuildWarps * cap * (8 + 4
 // 16,384-atom fcc cell (12 atoms a bin, the box culls a quarter) 48.5 -> 49.8 us.  The distance test runs
 // alone and what passes it (a tenth to a fifth) is settled 32 at a time, instead of every lane carrying the
 // key of its candidate along: the neighbour phase of the 4096 cells 913 -> 895 us, of 1,048,576 atoms 2.26
-// -> 2.21 ms, of the 16,384 atoms 67.0 -> 64.5 us.
+// -> 2.21 ms, of the 16,384 atoms 67.0 -> 64.5 us; with four candidates staged at once by a thread 866 us,
+// 2.16 ms and 63.9 us.
 template <class T>
 __global__ void __launch_bounds__(kBuildThreads) k_build(const BuildArgs a) {
     pdl_enter();
@@ -574,39 +576,58 @@ __global__ void __launch_bounds__(kBuildThreads) k_build(const BuildArgs a) {
                         // 1b. stage from candidates c0 .. c0 + m: bin g holds candidate f when
                         //     gpre[g] <= f < gpre[g + 1] (the last g with gpre[g] <= f)
                         const int m = min(kChunk - staged, total - c0);
-                        for (int f0 = 0; f0 < m; f0 += kBuildThreads) {
-                            const int f = f0 + threadIdx.x, ff = c0 + f;
-                            bool in = f < m;
-                            int g = 0, j = 0;
-                            float4 cp = make_float4(0.f, 0.f, 0.f, 0.f);
-                            if (in) {
+                        // (several candidates per thread at once: a candidate is a chain of a search and two
+                        // dependent loads, and their latency is what staging costs)
+                        for (int f0 = 0; f0 < m; f0 += kStageEach * kBuildThreads) {
+                            int g[kStageEach], j[kStageEach];
+                            float4 cp[kStageEach];
+                            unsigned keep[kStageEach];
 #pragma unroll
-                                for (int step = kGroup / 2; step > 0; step >>= 1)
-                                    if (gpre[g + step] <= ff) g += step;
-                                j = a.bin_atoms[gstart[g] + (ff - gpre[g])];
-                                const float4 lj = a.local[j];
-                                cp = make_float4(lj.x + goff[g], lj.y + goff[kGroup + g], lj.z + goff[2 * kGroup + g],
-                                                 __int_as_float(j));
-                                // distance to the box: no atom in it is nearer
-                                const float ex = fmaxf(fmaxf(bx0 - cp.x, cp.x - bx1), 0.f),
-                                            ey = fmaxf(fmaxf(by0 - cp.y, cp.y - by1), 0.f),
-                                            ez = fmaxf(fmaxf(bz0 - cp.z, cp.z - bz1), 0.f);
-                                in = ex * ex + ey * ey + ez * ez <= a.cull2;
+                            for (int u = 0; u < kStageEach; ++u) {
+                                const int f = f0 + u * kBuildThreads + threadIdx.x, ff = c0 + f;
+                                g[u] = 0;
+                                j[u] = -1;
+                                if (f < m) {
+#pragma unroll
+                                    for (int step = kGroup / 2; step > 0; step >>= 1)
+                                        if (gpre[g[u] + step] <= ff) g[u] += step;
+                                    j[u] = a.bin_atoms[gstart[g[u]] + (ff - gpre[g[u]])];
+                                }
                             }
-                            const unsigned keep = __ballot_sync(0xffffffffu, in);
+#pragma unroll
+                            for (int u = 0; u < kStageEach; ++u)
+                                cp[u] = j[u] >= 0 ? a.local[j[u]] : make_float4(0.f, 0.f, 0.f, 0.f);
+                            int total_kept = 0;
+#pragma unroll
+                            for (int u = 0; u < kStageEach; ++u) {
+                                cp[u] = make_float4(cp[u].x + goff[g[u]], cp[u].y + goff[kGroup + g[u]],
+                                                    cp[u].z + goff[2 * kGroup + g[u]], __int_as_float(j[u]));
+                                // distance to the box: no atom in it is nearer
+                                const float ex = fmaxf(fmaxf(bx0 - cp[u].x, cp[u].x - bx1), 0.f),
+                                            ey = fmaxf(fmaxf(by0 - cp[u].y, cp[u].y - by1), 0.f),
+                                            ez = fmaxf(fmaxf(bz0 - cp[u].z, cp[u].z - bz1), 0.f);
+                                if (!(ex * ex + ey * ey + ez * ez <= a.cull2)) j[u] = -1;
+                                keep[u] = __ballot_sync(0xffffffffu, j[u] >= 0);
+                                total_kept += __popc(keep[u]);
+                            }
                             int at = 0;
-                            if (lane == 0 && keep) at = atomicAdd(&s_count, __popc(keep));
-                            at = __shfl_sync(0xffffffffu, at, 0) + __popc(keep & ((1u << lane) - 1u));
-                            if (in) {
-                                const int wj = a.atom_wrap[j], tb = gtb[g];
-                                int tz = a.types[j];
-                                tz = tz < 0 ? 0 : (tz >= a.S ? a.S - 1 : tz);  // invalid species are reported by the binning
-                                cpos[at] = cp;
-                                // the key's low word: image shift in bytes 0..2, the neighbour's species in byte 3
-                                // (a function of j: the key order stays (j, s))
-                                cshift[at] = key_shift(unpack(tb, 0) - unpack(wj, 0), unpack(tb, 1) - unpack(wj, 1),
-                                                       unpack(tb, 2) - unpack(wj, 2)) | (tz << 24);
-                                ctb[at] = tb;
+                            if (lane == 0 && total_kept) at = atomicAdd(&s_count, total_kept);
+                            at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+                            for (int u = 0; u < kStageEach; ++u) {
+                                if (j[u] >= 0) {
+                                    const int to = at + __popc(keep[u] & ((1u << lane) - 1u));
+                                    const int wj = a.atom_wrap[j[u]], tb = gtb[g[u]];
+                                    int tz = a.types[j[u]];
+                                    tz = tz < 0 ? 0 : (tz >= a.S ? a.S - 1 : tz);  // invalid species are reported by the binning
+                                    cpos[to] = cp[u];
+                                    // the key's low word: image shift in bytes 0..2, the neighbour's species in
+                                    // byte 3 (a function of j: the key order stays (j, s))
+                                    cshift[to] = key_shift(unpack(tb, 0) - unpack(wj, 0), unpack(tb, 1) - unpack(wj, 1),
+                                                           unpack(tb, 2) - unpack(wj, 2)) | (tz << 24);
+                                    ctb[to] = tb;
+                                }
+                                at += __popc(keep[u]);
                             }
                         }
                         __syncthreads();
