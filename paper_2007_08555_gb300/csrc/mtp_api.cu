@@ -327,19 +327,16 @@ bool reserve_host_flags(mtp_model* M) {
     return M->h_flags == nullptr;
 }
 
-// Waits for the stream, then reports the errors the device recorded.  The two flag words come back
-// by stream-ordered copies into pinned memory before the one synchronisation, and the error word is
-// cleared by a stream-ordered memset, so a synchronous call costs a single wait.
-mtp_status finish(mtp_model* M, cudaStream_t st) {
+// Waits for the stream, then reports the errors the device recorded.  A kernel writes the two flag words
+// (and MD's scalars) to pinned memory before the one synchronisation and clears the error word, so a
+// synchronous call costs a single wait.
+mtp_status finish(mtp_model* M, cudaStream_t st, const double* scalars = nullptr) {
     if (reserve_host_flags(M)) return MTP_ENOMEM;
     M->h_flags[0] = M->h_flags[1] = 0;
     if (M->rev_pending) cudaStreamWaitEvent(st, M->ev_join, 0);  // side-stream work of the last build
-    if (M->nb.err.p) {
-        cudaMemcpyAsync(M->h_flags, M->nb.err.p, sizeof(int), cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(M->h_flags + 1, M->nb.counters.as<int>() + 2, sizeof(int), cudaMemcpyDeviceToHost, st);
-        cudaMemsetAsync(M->nb.err.p, 0, sizeof(int), st);
-    }
-    cudaError_t e = cudaStreamSynchronize(st);
+    cudaError_t e = cudaSuccess;
+    if (M->nb.err.p && M->nb.counters.p) e = mtp::report(M->nb, scalars, M->h_flags, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_status(e);
     collect_profile(M);
     M->last_max = M->h_flags[1];
@@ -1803,8 +1800,7 @@ mtp_status md_impl(mtp_model* M, int n, double* pos, double* vel, const int32_t*
         M->launches += mtp::launch_kick_kinetic(n, M->S, vel, F, types, mass, 0.5 * dt, step > 0, sc + 1, flag, st,
                                                 M->n_sm);
         if (!sel && step < n_steps) drift();
-        scalars();
-        mtp_status s2 = finish(M, st);
+        mtp_status s2 = finish(M, st, sc);
         ep[step] = h_sc[0];
         ek[step] = h_sc[1];
         rebuild = *reinterpret_cast<const int*>(h_sc + 3) != 0;
