@@ -682,7 +682,7 @@ def emit_horner(prog: Program, slot_begin):
     y inside z needs no monomials (a handful of running values instead of up to 165 registers of
     monomials: 72 registers a thread instead of 254 at lev_max 20), and reads dV/dM in the one order in
     which adj_to_shared lays it down.  The force-gradient phase, slices of components against this: lev_max
-    20, 1,048,576 atoms 4.12 against 3.84 ms, 16,384 atoms 104 against 85 us; lev_max 16, 393,000 atoms 447
+    20, 1,048,576 atoms 4.12 against 3.84 ms, 16,384 atoms 104 against 85 us; lev_max 16, 303,000 atoms 447
     against 404 us; lev_max 12, 104,000 atoms 60.6 against 57.5 us; lev_max 10 equal."""
     order = horner_order(prog)
     pos = {t: q for q, t in enumerate(order)}
