@@ -60,8 +60,8 @@ def parse():
 # workload, from one ncu capture of the current kernel (profiles/); None when
 # not captured since the kernel last changed.  The neighbour phase's entry adds its two launches: the
 # cell lists (k_bin_all, 497,920 B) and the list kernel (k_build, 1,463,808 + 329,728 B).
-TRAFFIC = {"k_build": 2291456, "k_pairgrad": 30838272, "k_moments": 12659968, "k_contract_parts": 8654080,
-           "k_gather": 29120000}
+TRAFFIC = {"k_build": 2486784, "k_pairgrad": 30847488, "k_moments": 12667392, "k_contract_parts": 8653568,
+           "k_gather": 29134592}
 # DRAM bytes per row of the tensor-core grade (rows of 116 doubles read once, one grade written), from
 # one ncu capture of the current kernel at 200,000 rows (profiles/); None when
 # not captured since the kernel last changed
