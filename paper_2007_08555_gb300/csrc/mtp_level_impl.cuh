@@ -1471,15 +1471,15 @@ struct TanSink;
 template <>
 struct TanSink<float> {
     using Pair = float2;
-    float eh, el;  // ek as a float pair; zero for a lane without an atom
-    float keep;    // 1, or 0 for a lane without an atom
+    float eh, el;  // ek as a float pair
+    bool act;      // a lane without an atom adds zero, whatever its (unwritten) moments hold
     float2* s;     // [MAXDALPHA][33]
     int* alpha;    // [MAXDALPHA]
     int lane;
     __device__ __forceinline__ void put(int q, int al, float v, float t) {
         const Df p = df_mulf({eh, el}, v);
-        const Df d = df_add(p, {-keep * t, 0.f});
-        s[q * 33 + lane] = make_float2(d.hi, d.lo);
+        const Df d = df_add(p, {-t, 0.f});
+        s[q * 33 + lane] = act ? make_float2(d.hi, d.lo) : make_float2(0.f, 0.f);
         if (lane == 0) alpha[q] = al;
     }
     __device__ __forceinline__ double sum(int q) const {
@@ -1488,18 +1488,19 @@ struct TanSink<float> {
         for (int l = 0; l < 32; ++l) d = df_add(d, {s[q * 33 + l].x, s[q * 33 + l].y});
         return (double)d.hi + (double)d.lo;
     }
-    __device__ __forceinline__ TanSink(double ek, bool act, Pair* st, int* al, int ln)
-        : eh((float)ek), el((float)(ek - (double)(float)ek)), keep(act ? 1.f : 0.f), s(st), alpha(al), lane(ln) {}
+    __device__ __forceinline__ TanSink(double ek, bool has, Pair* st, int* al, int ln)
+        : eh((float)ek), el((float)(ek - (double)(float)ek)), act(has), s(st), alpha(al), lane(ln) {}
 };
 template <>
 struct TanSink<double> {
     using Pair = double;
-    double ek, keep;
+    double ek;
+    bool act;
     double* s;
     int* alpha;
     int lane;
     __device__ __forceinline__ void put(int q, int al, double v, double t) {
-        s[q * 33 + lane] = ek * v - keep * t;
+        s[q * 33 + lane] = act ? ek * v - t : 0.0;
         if (lane == 0) alpha[q] = al;
     }
     __device__ __forceinline__ double sum(int q) const {
@@ -1508,8 +1509,8 @@ struct TanSink<double> {
         for (int l = 0; l < 32; ++l) d += s[q * 33 + l];
         return d;
     }
-    __device__ __forceinline__ TanSink(double e, bool act, Pair* st, int* al, int ln)
-        : ek(e), keep(act ? 1.0 : 0.0), s(st), alpha(al), lane(ln) {}
+    __device__ __forceinline__ TanSink(double e, bool has, Pair* st, int* al, int ln)
+        : ek(e), act(has), s(st), alpha(al), lane(ln) {}
 };
 constexpr int kTanWarps = 4;
 constexpr size_t kTanWarpBytes = (size_t)::MTP_GEN_NS::MAXDALPHA * (33 * 8 + 8);
