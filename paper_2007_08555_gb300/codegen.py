@@ -1109,6 +1109,21 @@ def emit_dual_parts(prog: Program, parts: int):
         out.append("  }")
         out.append("};")
     out.append(f"constexpr int MAXDALPHA = {max(len(alphas) for _, alphas in groups)};")
+    # dL/dxi of a part over a tile: put() takes the value and tangent of a basis function for one lane's
+    # atom, sum() adds the lanes' ek v - t; double precision, whatever that of v and t
+    out.append("struct DxiSink {")
+    out.append("  double ek; bool act;  // a lane without an atom adds zero, whatever its moments hold")
+    out.append("  double* s; int* alpha; int lane;  // [MAXDALPHA][33], [MAXDALPHA]")
+    out.append("  template <class T> __device__ __forceinline__ void put(int q, int al, T v, T t) {")
+    out.append("    s[q * 33 + lane] = act ? ek * (double)v - (double)t : 0.0;")
+    out.append("    if (lane == 0) alpha[q] = al;")
+    out.append("  }")
+    out.append("  __device__ __forceinline__ double sum(int q) const {")
+    out.append("    double d = 0.0;")
+    out.append("    for (int l = 0; l < 32; ++l) d += s[q * 33 + l];")
+    out.append("    return d;")
+    out.append("  }")
+    out.append("};")
     out.append("template <class Sink, class T>")
     out.append("__device__ __forceinline__ int dual_part(int part, const T* m, const T* mt, T* adj, T* adt, "
                "const T* xi, Sink& sink) {")
@@ -1118,20 +1133,15 @@ def emit_dual_parts(prog: Program, parts: int):
     out.append("  }")
     out.append("  return 0;")
     out.append("}")
-    # the same with ek v - t summed over the warp one basis function at a time
-    out.append("struct WarpSink {")
-    out.append("  double ek; bool act, lane0; double* dxt;")
-    out.append("  template <class T> __device__ __forceinline__ void put(int, int alpha, T v, T t) {")
-    out.append("    double d = act ? ek * (double)v - (double)t : 0.0;")
-    out.append("    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);")
-    out.append("    if (lane0) dxt[alpha] = d;")
-    out.append("  }")
-    out.append("};")
+    # one lane's share of dL/dxi alone (the other 31 lanes of the tile hold no atom)
     out.append("template <class T>")
     out.append("__device__ __forceinline__ void dual_part(int part, const T* m, const T* mt, T* adj, T* adt, "
                "const T* xi, double ek, bool act, bool lane0, double* dxt) {")
-    out.append("  WarpSink sink{ek, act, lane0, dxt};")
-    out.append("  dual_part(part, m, mt, adj, adt, xi, sink);")
+    out.append("  double s[MAXDALPHA * 33]; int alpha[MAXDALPHA];")
+    out.append("  for (int q = 0; q < MAXDALPHA * 33; ++q) s[q] = 0.0;")
+    out.append("  DxiSink sink{ek, act, s, alpha, 0};")
+    out.append("  const int n = dual_part(part, m, mt, adj, adt, xi, sink);")
+    out.append("  for (int q = 0; lane0 && q < n; ++q) dxt[alpha[q]] = sink.sum(q);")
     out.append("}")
     return out
 

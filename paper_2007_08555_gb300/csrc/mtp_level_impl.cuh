@@ -1462,65 +1462,19 @@ constexpr int kAdjRow = (G::C_ + 3) / 4 * 4;
 // Tangent contraction of the loss gradient, split into NDPART generated parts like the
 // forward contraction: warp w runs part w / n_tiles for the 32 atoms of tile w % n_tiles.  Each part
 // writes dV/dM and its tangent for its moments to dual slots and its basis functions' shares of
-// dL/dxi (summed over the tile's atoms) to dxt[tile].  Every lane forms its atom's ek B - dB/dt as a
-// double-float pair in shared memory, then a lane per basis function sums the 32 atoms in double-float
-// arithmetic: warp sums in double cost ten instructions of the double-precision pipe per basis function,
-// 16 clocks of the SM each (2048 cells, lev_max 20: 3.79 ms, with these sums 2.98).
-template <class T>
-struct TanSink;
-template <>
-struct TanSink<float> {
-    using Pair = float2;
-    float eh, el;  // ek as a float pair
-    bool act;      // a lane without an atom adds zero, whatever its (unwritten) moments hold
-    float2* s;     // [MAXDALPHA][33]
-    int* alpha;    // [MAXDALPHA]
-    int lane;
-    __device__ __forceinline__ void put(int q, int al, float v, float t) {
-        const Df p = df_mulf({eh, el}, v);
-        const Df d = df_add(p, {-t, 0.f});
-        s[q * 33 + lane] = act ? make_float2(d.hi, d.lo) : make_float2(0.f, 0.f);
-        if (lane == 0) alpha[q] = al;
-    }
-    __device__ __forceinline__ double sum(int q) const {
-        Df d = {0.f, 0.f};
-#pragma unroll 4
-        for (int l = 0; l < 32; ++l) d = df_add(d, {s[q * 33 + l].x, s[q * 33 + l].y});
-        return (double)d.hi + (double)d.lo;
-    }
-    __device__ __forceinline__ TanSink(double ek, bool has, Pair* st, int* al, int ln)
-        : eh((float)ek), el((float)(ek - (double)(float)ek)), act(has), s(st), alpha(al), lane(ln) {}
-};
-template <>
-struct TanSink<double> {
-    using Pair = double;
-    double ek;
-    bool act;
-    double* s;
-    int* alpha;
-    int lane;
-    __device__ __forceinline__ void put(int q, int al, double v, double t) {
-        s[q * 33 + lane] = act ? ek * v - t : 0.0;
-        if (lane == 0) alpha[q] = al;
-    }
-    __device__ __forceinline__ double sum(int q) const {
-        double d = 0.0;
-#pragma unroll 4
-        for (int l = 0; l < 32; ++l) d += s[q * 33 + l];
-        return d;
-    }
-    __device__ __forceinline__ TanSink(double e, bool has, Pair* st, int* al, int ln)
-        : ek(e), act(has), s(st), alpha(al), lane(ln) {}
-};
+// dL/dxi (summed over the tile's atoms) to dxt[tile].  Every lane leaves its atom's ek B - dB/dt in shared
+// memory, then a lane per basis function sums the 32 atoms (the generated DxiSink), all in double: four
+// instructions of the double-precision pipe, 16 clocks of the SM each, per basis function, where warp sums
+// by shuffles took ten.  The gradient of 2048 cells at lev_max 20 takes 7.45 ms; with double-float sums (44
+// bits) it took 7.30, and this kernel 3.0 ms where the shuffles took 3.8.
 constexpr int kTanWarps = 4;
 constexpr size_t kTanWarpBytes = (size_t)::MTP_GEN_NS::MAXDALPHA * (33 * 8 + 8);
 
 template <class T>
 __global__ void __launch_bounds__(32 * kTanWarps) k_contract_tan_parts(const EvalCtx<T> a) {
-    using Pair = typename TanSink<T>::Pair;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
-    Pair* stage = reinterpret_cast<Pair*>(smem_raw + (threadIdx.x >> 5) * kTanWarpBytes);
+    double* stage = reinterpret_cast<double*>(smem_raw + (threadIdx.x >> 5) * kTanWarpBytes);
     int* alpha = reinterpret_cast<int*>(stage + ::MTP_GEN_NS::MAXDALPHA * 33);
     const int n_tiles = (a.n_atoms + 31) >> 5;
     const int total = n_tiles * G::NDPART_;
@@ -1530,7 +1484,7 @@ __global__ void __launch_bounds__(32 * kTanWarps) k_contract_tan_parts(const Eva
         const int i = tile * 32 + lane;
         const bool act = i < a.n_atoms;
         const double ek = act ? a.gew[a.cfg_of[i]] : 0.0;
-        TanSink<T> sink(ek, act, stage, alpha, lane);
+        ::MTP_GEN_NS::DxiSink sink{ek, act, stage, alpha, lane};
         const size_t mo = (size_t)tile * G::C_ * 32 + lane;
         const size_t so = (size_t)tile * G::NDSLOT_ * 32 + lane;
         const int na = ::MTP_GEN_NS::dual_part(part, a.mom + mo, a.momt + mo, a.dslots + so, a.dslots + half + so, a.xi,
