@@ -80,21 +80,6 @@ __device__ __forceinline__ int clamp_species(int z, int S) { return z < 0 ? 0 : 
 __device__ __forceinline__ float my_sqrt(float x) { return sqrtf(x); }
 __device__ __forceinline__ double my_sqrt(double x) { return sqrt(x); }
 
-// |r| and x / |r| of a pair: in double from one reciprocal square root (a square root and a division take
-// some thirty more instructions of the slow double-precision pipe)
-struct Length {
-    double r, inv;
-    __device__ __forceinline__ explicit Length(double r2) : inv(rsqrt(r2)) { r = r2 * inv; }
-    __device__ __forceinline__ double over(double x) const { return x * inv; }
-};
-struct LengthF {
-    float r;
-    __device__ __forceinline__ explicit LengthF(float r2) : r(sqrtf(r2)) {}
-    __device__ __forceinline__ float over(float x) const { return x / r; }
-};
-template <class T>
-using LengthOf = std::conditional_t<sizeof(T) == 4, LengthF, Length>;
-
 // Double-float numbers (hi + lo, |lo| <= ulp(hi) / 2): Knuth's TwoSum and the FMA form of Dekker's
 // TwoProduct give the exact rounding errors, so sums and products keep ~44 significant bits on the
 // FP32 pipe (GB300 issues double precision at a small fraction of the FP32 rate).
@@ -441,8 +426,8 @@ __device__ void moments_split(const EvalCtx<double>& a, const double* cs, double
                 double* mine = buf + (size_t)(half * NS + S) * W * 32 + lane;
                 double f[G::NMU_];
                 if (t < trips) {
-                    const Length len(cur.x * cur.x + cur.y * cur.y + cur.z * cur.z);
-                    radial<double, false>(len.r, cs + (zi * a.S + cur.zj) * csz, a.NQ, a.rmin, a.rcut, a.inv_span, f,
+                    const double r = my_sqrt(cur.x * cur.x + cur.y * cur.y + cur.z * cur.z);
+                    radial<double, false>(r, cs + (zi * a.S + cur.zj) * csz, a.NQ, a.rmin, a.rcut, a.inv_span, f,
                                           nullptr);
                     mine[0] = cur.x;
                     mine[32] = cur.y;
@@ -750,13 +735,12 @@ __device__ __forceinline__ void pairgrad_pairs(const EvalCtx<T>& a, int i, int s
         const PairIn<T> cur = nx;
         if (p + TPA < cnt) nx = load_pair(a, (size_t)(p + TPA) * n + i);
         const T x = cur.x, y = cur.y, z = cur.z;
-        const LengthOf<T> len(x * x + y * y + z * z);
-        const T r = len.r;
+        const T r = my_sqrt(x * x + y * y + z * z);
         T f[G::NMU_], df[G::NMU_];
         radial<T, true>(r, cs + (zi * a.S + cur.zj) * csz, a.NQ, a.rmin, a.rcut, a.inv_span, f, df);
         T s = T(0), gx = T(0), gy = T(0), gz = T(0);
         SliceSel<T, S>::type::template grad<T>(x, y, z, f, df, adj, s, gx, gy, gz);
-        const T sr = len.over(s);
+        const T sr = s / r;
         gx += sr * x;
         gy += sr * y;
         gz += sr * z;
@@ -853,8 +837,7 @@ __device__ __forceinline__ void pairgrad_merged(const EvalCtx<T>& a, int i, int 
         const PairIn<T> cur = nx;
         if (p + TPA < cnt) nx = load_pair(a, (size_t)(p + TPA) * n + i);
         const T x = cur.x, y = cur.y, z = cur.z;
-        const LengthOf<T> len(x * x + y * y + z * z);
-        const T r = len.r;
+        const T r = my_sqrt(x * x + y * y + z * z);
         T f[G::NMU_], df[G::NMU_];
         radial<T, true>(r, cs + (zi * a.S + cur.zj) * csz, a.NQ, a.rmin, a.rcut, a.inv_span, f, df);
         T s = T(0), gx = T(0), gy = T(0), gz = T(0);
@@ -862,7 +845,7 @@ __device__ __forceinline__ void pairgrad_merged(const EvalCtx<T>& a, int i, int 
             ::MTP_GEN_NS::HornerF::grad<T>(x, y, z, f, df, SharedAdj<T, NSA>{q}, s, gx, gy, gz);
         else
             grad_all_slices<T, 0, NSA>(x, y, z, f, df, q, s, gx, gy, gz);
-        const T sr = len.over(s);
+        const T sr = s / r;
         a.g[idx] = Vec4<T>{gx + sr * x, gy + sr * y, gz + sr * z, T(0)};
     }
 }
