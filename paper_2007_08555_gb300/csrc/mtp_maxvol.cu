@@ -497,6 +497,11 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
         }
     }
     __syncthreads();
+    // The shares of A's rows begin elsewhere than those of B's.  In global memory (matrices of some 10,000
+    // rows and more) a block's first rows of A lie among another's rows of B, so everyone finishes first: one
+    // round of the exchange, a few microseconds of such a phase's milliseconds.
+    const bool shared = g.rows_in && g.col_in;
+    if (!shared && !x.barrier()) return;
     // 2. the inverse of A = B[sel]
     const auto load = [&](int j, int c) { return g.B[(size_t)sel[j] * m + c] * D[c]; };
     own(m, Rm);
@@ -587,6 +592,7 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
     __syncthreads();
     // A^-1 = D (A D)^-1, computed from scratch, and the unscaled A (possibly over the exchange's rows:
     // after every block has read the last of them)
+    if (!shared && !x.barrier()) return;
     own(m, Rm);
     if (!invert_rows(x, a, orig, g.Ai, g.status, load, [&](int row) { return D[row]; })) return;
     if (!x.barrier()) return;
