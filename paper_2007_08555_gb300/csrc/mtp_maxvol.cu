@@ -192,9 +192,9 @@ struct Exchange {
 };
 
 // The candidate of a pivot step: largest |w[r][k]| among the block's rows at positions >= k (ties to the
-// smaller position; NaN is no candidate).  Warp 0 publishes it with its row from column c0 on and, while
-// the record travels, the reciprocal of the pivot.  The block is in step before and after is not.
-__device__ void publish_pivot(Exchange& x, const Rows& a, int k, int c0) {
+// smaller position; NaN is no candidate).  Warp 0 publishes it with its row from column c0 on and, if asked
+// to, while the record travels, the reciprocal of the pivot.  The block is in step before and after is not.
+__device__ void publish_pivot(Exchange& x, const Rows& a, int k, int c0, bool reciprocal) {
     ++x.t;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     unsigned long long bv = 0;
@@ -238,7 +238,7 @@ __device__ void publish_pivot(Exchange& x, const Rows& a, int k, int c0) {
             const double* row = a.w + (size_t)br * a.m;
             for (int c = c0 + lane; c < a.m; c += 32) x.send(c, row[c]);
             if (lane == 0) x.send(a.m, (double)(a.first + br));
-            if (lane == 1) x.send(a.m + 1, 1.0 / row[k]);
+            if (reciprocal && lane == 1) x.send(a.m + 1, 1.0 / row[k]);
         }
     }
 }
@@ -293,7 +293,7 @@ __device__ bool invert_rows(Exchange& x, Rows& a, int* orig, double* Ai, int* st
     for (int r = tid; r < a.R; r += nt) a.pos[r] = a.first + r;
     __syncthreads();
     for (int k = 0; k < m; ++k) {
-        publish_pivot(x, a, k, 0);
+        publish_pivot(x, a, k, 0, true);
         double v;
         unsigned p;
         const int q = x.winner(&v, &p);
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
         for (int r = tid; r < a.R; r += nt) a.pos[r] = a.first + r;
         __syncthreads();
         for (int k = 0; k < m; ++k) {
-            publish_pivot(x, a, k, k + 1);
+            publish_pivot(x, a, k, k, false);
             double v;
             unsigned p;
             const int q = x.winner(&v, &p);
@@ -480,13 +480,13 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
             bool bad = false;
             for (int c = k + 1 + tid; c < m; c += nt) a.prow[c] = x.receive(q, c, &bad);
             if (tid == nt - 1) sel[k] = (int)x.receive(q, m, &bad);
-            const double inv = tid < a.R ? x.receive(q, m + 1, &bad) : 0.0;
+            const double pivot = tid < a.R ? x.receive(q, k, &bad) : 1.0;
             for (int r = tid; r < a.R; r += nt) {
                 if (a.pos[r] == (int)p)
                     a.pos[r] = k;
                 else if (a.pos[r] == k)
                     a.pos[r] = (int)p;
-                a.col[r] = a.w[(size_t)r * m + k] * inv;
+                a.col[r] = a.w[(size_t)r * m + k] / pivot;
             }
             if (__syncthreads_or(bad)) {
                 if (bad) atomicOr(g.status, kErrTimeout);
