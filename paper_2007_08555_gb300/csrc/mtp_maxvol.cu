@@ -243,11 +243,11 @@ __device__ void publish_pivot(Exchange& x, const Rows& a, int k, int c0, bool re
     }
 }
 
-// w[r][c] <- w[r][c] - col[r] prow[c] for the block's rows that keep(r) takes and columns c0 <= c < m;
+// w[r][c] <- update(w[r][c], col[r], prow[c]) for the block's rows that keep(r) takes and columns c0 <= c < m;
 // seen(value, r, c) gets every new value.  Warps take rows, and parts of a row where there are more warps
 // than rows.
-template <class Keep, class Seen>
-__device__ __forceinline__ void rank_one(const Rows& a, int c0, Keep keep, Seen seen) {
+template <class Keep, class Update, class Seen>
+__device__ __forceinline__ void rank_one(const Rows& a, int c0, Keep keep, Update update, Seen seen) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     if (a.R < 1) return;
     const int parts = a.R < nw ? nw / a.R : 1;
@@ -258,12 +258,13 @@ __device__ __forceinline__ void rank_one(const Rows& a, int c0, Keep keep, Seen 
         const double l = a.col[r];
         double* w = a.w + (size_t)r * a.m;
         for (int c = c0 + part * 32 + lane; c < a.m; c += parts * 32) {
-            const double v = fma(-l, a.prow[c], w[c]);
+            const double v = update(w[c], l, a.prow[c]);
             w[c] = v;
             seen(v, r, c);
         }
     }
 }
+__device__ __forceinline__ double eliminate(double w, double l, double p) { return fma(-l, p, w); }
 
 // NR rows of C = B A^-1 (chunk: NR rows of B, scaled): a thread per column, k in order.
 template <int NR, class Put>
@@ -317,7 +318,7 @@ __device__ bool invert_rows(Exchange& x, Rows& a, int* orig, double* Ai, int* st
             if (bad) atomicOr(x.err, kErrTimeout);
             return false;
         }
-        rank_one(a, 0, [&](int r) { return a.pos[r] != k; }, [](double, int, int) {});
+        rank_one(a, 0, [&](int r) { return a.pos[r] != k; }, eliminate, [](double, int, int) {});
         if (q == (int)blockIdx.x)
             for (int r = 0; r < a.R; ++r)
                 if (a.pos[r] == k)
@@ -492,7 +493,7 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
                 if (bad) atomicOr(g.status, kErrTimeout);
                 return;
             }
-            rank_one(a, k + 1, [&](int r) { return a.pos[r] > k; }, [](double, int, int) {});
+            rank_one(a, k + 1, [&](int r) { return a.pos[r] > k; }, eliminate, [](double, int, int) {});
             __syncthreads();
         }
     }
@@ -578,7 +579,7 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
         bool bad = false;
         const double ckj = x.receive(q, j, &bad);
         for (int c = tid; c < m; c += nt) a.prow[c] = x.receive(q, c, &bad) - (c == j ? 1.0 : 0.0);
-        for (int r = tid; r < a.R; r += nt) a.col[r] = a.w[(size_t)r * m + j] / ckj;
+        for (int r = tid; r < a.R; r += nt) a.col[r] = a.w[(size_t)r * m + j];
         if (tid == 0) sel[j] = (int)e / m;
         if (__syncthreads_or(bad)) {
             if (bad) atomicOr(g.status, kErrTimeout);
@@ -586,7 +587,9 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
         }
         best = -1.0;
         at = 0;
-        rank_one(a, 0, [](int) { return true; }, [&](double v, int r, int c) { track(v, (a.first + r) * m + c); });
+        // (product, then quotient, then difference: with the factor divided beforehand ties fall differently)
+        rank_one(a, 0, [](int) { return true; }, [&](double w, double l, double p) { return w - l * p / ckj; },
+                 [&](double v, int r, int c) { track(v, (a.first + r) * m + c); });
         ++swaps;
     }
     __syncthreads();

@@ -113,9 +113,7 @@ def restated(tmp_path_factory):
     return run
 
 
-@pytest.mark.parametrize("kind", ["signs", "bits", "wide", "rank_lost"])
-@pytest.mark.parametrize("seed", range(40))
-def test_selection_of_integer_matrices(gpu_lib, restated, kind, seed):
+def _compare(restated, kind, seed):
     rng = np.random.default_rng([seed, len(kind)])
     m = int(rng.integers(2, 80))
     n = int(m + rng.integers(0, 2 * m + 1))
@@ -132,3 +130,14 @@ def test_selection_of_integer_matrices(gpu_lib, restated, kind, seed):
     assert got == want
     if want >= 0:
         assert sel.cpu().tolist() == rows
+
+
+@pytest.mark.parametrize("kind", ["signs", "bits", "wide", "rank_lost"])
+@pytest.mark.parametrize("seed", range(40))
+def test_selection_of_integer_matrices(gpu_lib, restated, kind, seed):
+    _compare(restated, kind, seed)
+
+
+@pytest.mark.parametrize("seed", [68, 4675, 5032])
+def test_swaps_that_the_last_bit_decides(gpu_lib, restated, seed):
+    _compare(restated, "bits", seed)
