@@ -350,8 +350,9 @@ inline Layout mv_layout(int n, int m, int G, bool full) {
     l.R = mv_rows(n > m ? n : m, G);
     l.br = full ? (m <= 1024 ? 8 : 1) : 0;
     size_t b = 32 + 32 * 16 + (G == 1 ? 32 + 32 * (size_t)(m + 2) : 0);
-    b += 8 * (size_t)m + 8 * (size_t)m;                                     // prow, orig (8-byte slots)
-    if (full) b += 8 * (size_t)m + 8 * (size_t)m + 8 * (size_t)m * l.br;    // D, sel, chunk
+    const size_t ints = 8 * ((size_t)(m + 1) / 2);                    // m ints in 8-byte slots
+    b += 8 * (size_t)m + ints;                                        // prow, orig
+    if (full) b += 8 * (size_t)m + ints + 8 * (size_t)m * l.br;       // D, sel, chunk
     l.col_in = b + 16 * (size_t)l.R <= kMvSharedMost;
     if (l.col_in) b += 16 * (size_t)l.R;
     l.rows_in = b + 8 * (size_t)l.R * m <= kMvSharedMost;
@@ -381,7 +382,7 @@ __device__ void carve_common(Carve& s, Exchange& x, Rows& a, int** orig) {
         for (int e = threadIdx.x; e < 4 + 4 * (x.m + 2); e += blockDim.x) x.rec[e] = 0;
     }
     a.prow = s.take<double>(x.m);
-    *orig = s.take<int>(2 * x.m);
+    *orig = s.take<int>(x.m);
 }
 
 struct MaxvolArgs {
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
     int* orig;
     carve_common(sh, x, a, &orig);
     double* D = sh.take<double>(m);
-    int* sel = sh.take<int>(2 * m);
+    int* sel = sh.take<int>(m);
     double* chunk = sh.take<double>((size_t)m * g.br);
     const int Rn = mv_rows(n, g.G), Rm = mv_rows(m, g.G), Rmost = Rn > Rm ? Rn : Rm;
     double* col_s = g.col_in ? sh.take<double>(Rmost) : nullptr;
@@ -741,7 +742,7 @@ int launch_invert(int m, const double* A, double* Ai, double* W, int* status, cu
         G = blocks(mm);
         l = mv_layout(m, m, G, false);
     }
-    if (!l.col_in || l.bytes > kMvSharedMost) return -1;  // not reachable for the widths of a model
+    if (!l.col_in || l.bytes > kMvSharedMost) return -1;  // above m = 16,000
     auto* rec = reinterpret_cast<unsigned long long*>(W);
     InvertArgs g{m, G, l.rows_in, l.col_in, A, Ai, W + mm, nullptr, rec + 4 * (size_t)G, rec, status};
     return mv_launch(k_invert, g, G, l.bytes, st);
@@ -760,7 +761,7 @@ int launch_maxvol(int n, int m, const double* B, double* W, int* pos, int* sel, 
         G = mv_blocks(m, mm - 1);  // (A need not be 16-byte aligned)
         l = mv_layout(n, m, G, true);
     }
-    if (l.bytes > kMvSharedMost) return -1;  // not reachable for the widths of a model
+    if (l.bytes > kMvSharedMost) return -1;  // above m = 6382; a model's widest active set is 5580 columns
     auto* rec = reinterpret_cast<unsigned long long*>(W);
     double* rest = W + 2 * (size_t)m;
     auto* in_A = reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(A) + 15) & ~(uintptr_t)15);
