@@ -716,13 +716,14 @@ size_t mv_slot_bytes(int m, int G) { return 32 * (size_t)G * (m + 2); }
 
 template <class K, class Args>
 int mv_launch(K kernel, Args& g, int G, size_t smem, cudaStream_t st) {
-    if (G > 1 && (cudaMemsetAsync(g.rec, 0, 32 * (size_t)G, st) != cudaSuccess ||
-                  cudaMemsetAsync(g.slots, 0, mv_slot_bytes(g.m, G), st) != cudaSuccess))
-        return -1;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMvSharedMost) != cudaSuccess)
-        return -1;
     void* args[] = {&g};
-    return cudaLaunchCooperativeKernel((void*)kernel, dim3(G), dim3(kMvThreads), args, smem, st) == cudaSuccess ? 1 : -1;
+    const bool ok =
+        (G == 1 || (cudaMemsetAsync(g.rec, 0, 32 * (size_t)G, st) == cudaSuccess &&
+                    cudaMemsetAsync(g.slots, 0, mv_slot_bytes(g.m, G), st) == cudaSuccess)) &&
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMvSharedMost) == cudaSuccess &&
+        cudaLaunchCooperativeKernel((void*)kernel, dim3(G), dim3(kMvThreads), args, smem, st) == cudaSuccess;
+    if (!ok) cudaGetLastError();
+    return ok ? 1 : -1;
 }
 
 }  // namespace
