@@ -317,7 +317,9 @@ mtp_status mtp_param_grad(mtp_model* model, int n_cfg, int n_atoms, const int32_
  * masses [S] (host, amu).  Requires mtp_set_skin() > 0: the neighbour list is rebuilt when an atom
  * has moved more than skin / 2 since the last build, otherwise refreshed.  e_pot and e_kin (host,
  * [n_steps + 1], eV, step 0 = initial state) and n_rebuilds (host) may be NULL.  Energies and the
- * kinetic sum are accumulated in double precision; forces are the model's precision.
+ * kinetic sum are accumulated in double precision; forces are the model's precision.  When a step
+ * fails (MTP_EOVERFLOW, a non-finite position), pos holds that step's positions; if it is the starting
+ * configuration that fails, pos and vel are as they came in.
  */
 mtp_status mtp_md_run(mtp_model* model, int n_atoms, double* pos, double* vel, const int32_t* types,
                       const double* cell, const double* masses, double dt, int n_steps, double* e_pot,

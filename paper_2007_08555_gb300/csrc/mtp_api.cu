@@ -1759,7 +1759,7 @@ mtp_status md_impl(mtp_model* M, int n, double* pos, double* vel, const int32_t*
     cudaMemcpyAsync(M->s_off.p, off_h, sizeof off_h, cudaMemcpyHostToDevice, st);
     const int* off = M->s_off.as<int>();
     double* F = M->md_F.as<double>();
-    double* sc = M->md_scalars.as<double>();  // [0] E_pot, [1] E_kin, [2] grade, [3] the rebuild flag
+    double* sc = M->md_scalars.as<double>();  // [0] E_pot, [1] E_kin, [2] grade, [3] two ints: the rebuild flag, errors
     int* flag = reinterpret_cast<int*>(sc + 3);
     const double* mass = M->md_masses.as<double>();
     const double lim2 = 0.25 * M->skin * M->skin;
@@ -1794,10 +1794,11 @@ mtp_status md_impl(mtp_model* M, int n, double* pos, double* vel, const int32_t*
     };
     auto scalars = [&]() { cudaMemcpyAsync(M->h_flags + 4, sc, 4 * sizeof(double), cudaMemcpyDeviceToHost, st); };
     // Ends a step: the second half kick (not for step 0) and the energies, and the drift of the next step
-    // when nothing can stop the run here, so that one wait covers both.
+    // when no grade can stop the run here, so that one wait covers both (the drift does nothing if the
+    // evaluation reported an error).
     auto record = [&](int step) -> mtp_status {
         cudaMemsetAsync(sc + 1, 0, sizeof(double), st);
-        M->launches += mtp::launch_kick_kinetic(n, M->S, vel, F, types, mass, 0.5 * dt, step > 0, sc + 1, flag, st,
+        M->launches += mtp::launch_kick_kinetic(M->nb, M->S, vel, F, types, mass, 0.5 * dt, step > 0, sc + 1, flag, st,
                                                 M->n_sm);
         if (!sel && step < n_steps) drift();
         mtp_status s2 = finish(M, st, sc);

@@ -120,7 +120,9 @@ int launch_lbfgs_pair(int P, const double* theta, const double* trial, const dou
 // Molecular dynamics helpers (mtp_md.cu).  The refreshed pairs go to nb.cpr, from the displacements in
 // nb.disp (have_u: already there from launch_kick_drift).
 int launch_update_pairs(const NbrState& nb, const double* x, bool have_u, cudaStream_t st, int n_sm);
-int launch_kick_kinetic(int n, int S, double* v, const double* F, const int* types, const double* masses,
+// flag: two ints, written by launch_kick_kinetic (the error word of the evaluation before it in flag[1]) and
+// read by launch_kick_drift (which sets flag[0] when the lists must be rebuilt).
+int launch_kick_kinetic(const NbrState& nb, int S, double* v, const double* F, const int* types, const double* masses,
                         double half_dt, bool kick, double* e_kin, int* flag, cudaStream_t st, int n_sm);
 int launch_kick_drift(const NbrState& nb, int S, double* x, double* v, const double* F, const int* types,
                       const double* masses, double dt, double lim2, int* flag, cudaStream_t st, int n_sm);

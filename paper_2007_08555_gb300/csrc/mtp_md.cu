@@ -67,11 +67,15 @@ __device__ __forceinline__ int species(const int* types, int i, int S) {
 }
 
 // Second half kick of a step and the kinetic energy of the new velocities (kick = false: the kinetic
-// energy alone); clears the rebuild flag for the drift that follows.
+// energy alone); clears the rebuild flag (flag[0]) for the drift that follows and keeps the error word of the
+// evaluation for it (flag[1]).
 __global__ void k_kick_kinetic(int n, int S, double* v, const double* F, const int* types, const double* masses,
-                               double half_dt, bool kick, double* out, int* flag) {
+                               double half_dt, bool kick, double* out, int* flag, const int* err) {
     __shared__ double s[256];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        flag[0] = 0;
+        flag[1] = *err;
+    }
     double acc = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const double m = masses[species(types, i, S)];
@@ -96,11 +100,14 @@ __global__ void k_kick_kinetic(int n, int S, double* v, const double* F, const i
 }
 
 // First half kick, x += dt v, and the displacements since the build for the refresh of the pairs; flags
-// a rebuild when |x - x0| exceeds skin / 2
+// a rebuild when |x - x0| exceeds skin / 2.  Launched before the host has seen whether the evaluation that
+// gave F succeeded: if it did not (flag[1], which this kernel does not write: all blocks agree), positions and
+// velocities stay those of the failing step.
 template <class T>
 __global__ void k_kick_drift(int n, int S, double* x, double* v, const double* F, const int* types,
                              const double* masses, double half_dt, const double* x0, double dt, double lim2,
                              Vec4<T>* u, int* flag, int* err) {
+    if (flag[1] != 0) return;
     bool far = false;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const double q = half_dt / (masses[species(types, i, S)] * kMvv2eV);
@@ -147,9 +154,11 @@ int launch_update_pairs(const NbrState& nb, const double* x, bool have_u, cudaSt
     return have_u ? 1 : 2;
 }
 
-int launch_kick_kinetic(int n, int S, double* v, const double* F, const int* types, const double* masses,
+int launch_kick_kinetic(const NbrState& nb, int S, double* v, const double* F, const int* types, const double* masses,
                         double half_dt, bool kick, double* e_kin, int* flag, cudaStream_t st, int n_sm) {
-    k_kick_kinetic<<<grid_for(n, 256, n_sm), 256, 0, st>>>(n, S, v, F, types, masses, half_dt, kick, e_kin, flag);
+    const int n = nb.n_atoms;
+    k_kick_kinetic<<<grid_for(n, 256, n_sm), 256, 0, st>>>(n, S, v, F, types, masses, half_dt, kick, e_kin, flag,
+                                                          nb.err.as<int>());
     return 1;
 }
 
