@@ -1855,10 +1855,19 @@ int grad_all(EvalCtx<T>& a, const LossArgs& L, cudaStream_t st, int n_sm) {
         ++launches;
     }
     {
-        // one warp per block; atoms per block: enough blocks for eight warps per SM, four atoms at least
+        // One warp per block; atoms per block: enough blocks for eight warps per SM, four atoms at least.  In float,
+        // where the shared memory holds fewer warps and each has a full chunk or more to do, a whole number of
+        // long chunks for each, since the sums are combined once per species and chunk: 1024 cells, 8 species, 16
+        // radial functions at lev_max 20 (one resident warp) 10.2 -> 9.3 ms, 16 and 10 (two and three) 3.70 ->
+        // 3.21 and 2.00 -> 1.81 ms.  In double the arithmetic takes longer than the combining, and shorter chunks
+        // share it better: 400 such cells at lev_max 16 21.4 against 22.2 ms.
         const size_t smem = dc_bytes<T>(a.S, a.NQ);
-        const long per = ((long)a.n_atoms + n_sm * 8 - 1) / (n_sm * 8);
-        const int chunk = (int)(per < kDcAtoms ? kDcAtoms : per > kDcChunkMax ? kDcChunkMax : (per + 3) / 4 * 4);
+        const int warps = n_sm * (int)std::max<size_t>(1, std::min<size_t>(8, 227 * 1024 / (smem + 1024)));
+        const int each = (a.n_atoms + warps - 1) / warps;  // atoms of a resident warp
+        const bool few = sizeof(T) == 4 && warps < n_sm * 8 && each >= kDcChunkMax;
+        const int per = few ? each / ((each + kDcChunkMax - 1) / kDcChunkMax)
+                            : std::min((a.n_atoms + n_sm * 8 - 1) / (n_sm * 8), kDcChunkMax);
+        const int chunk = (per + kDcAtoms - 1) / kDcAtoms * kDcAtoms;
         const int blocks = (a.n_atoms + chunk - 1) / chunk;
         auto go = [&](void (*k)(const EvalCtx<T>, int)) {
             if (smem > 48 * 1024)
