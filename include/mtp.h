@@ -250,7 +250,7 @@ mtp_status mtp_grade_columns(const mtp_model* model, int32_t* cols /* host [mtp_
  * Jacobian rows of the nonlinear criterion (Sec. 2.3) for a batch (layout of mtp_eval_batch, device
  * arrays): rows [n_cfg][mtp_grade_width()] (double, device), the columns selected by
  * mtp_set_grade_kind() of [b(cfg_k), dE_k/dc] with b(cfg_k) = sum_i B(n_i) = dE_k/dxi (Eq. 2) and
- * dE_k/dc from the adjoint kernels of mtp_param_grad, summed per configuration in double precision.
+ * dE_k/dc from the adjoint kernels of mtp_param_grad, summed per configuration as there.
  * In the linear kind the rows are [b(cfg_k), dE_k/dc] in full.  Flags: MTP_ASYNC.
  */
 mtp_status mtp_jacobian_rows(mtp_model* model, int n_cfg, int n_atoms, const int32_t* cfg_off, const double* pos,
@@ -303,7 +303,8 @@ mtp_status mtp_grade(mtp_model* model, int n_rows, const double* b_rows, double*
  * f_ref [n_atoms][3], w_ref [n_cfg][9].  Outputs: loss [1], d_xi [m], d_c [S][S][N_mu][N_Q] (each may
  * be NULL; with both d_xi and d_c NULL only the evaluation and the loss run).  The force and stress terms are obtained as the derivative of the pair gradients along
  * the residual displacements (the mixed second derivative), recomputed rather than stored.
- * Device arrays unless MTP_HOST_MEMORY.  Gradient sums are accumulated in double precision.
+ * Device arrays unless MTP_HOST_MEMORY.  The sums over atoms are accumulated in double precision; in the float
+ * path those of d_c are float over the pairs of up to eight atoms first.
  */
 mtp_status mtp_param_grad(mtp_model* model, int n_cfg, int n_atoms, const int32_t* cfg_off, const double* pos,
                           const int32_t* types, const double* cells, const double* e_ref, const double* f_ref,

@@ -127,10 +127,10 @@ int launch_kick_kinetic(const NbrState& nb, int S, double* v, const double* F, c
 int launch_kick_drift(const NbrState& nb, int S, double* x, double* v, const double* F, const int* types,
                       const double* masses, double dt, double lim2, int* flag, cudaStream_t st, int n_sm);
 
-// CSR export of the neighbour list with exact double-precision r_ij.
-// error word and largest neighbour count of the last build to pinned host memory (host[0], host[1]; the former is
-// cleared), and four doubles from `scalars`, if given, to byte 16
+// Error word and largest neighbour count of the last build to pinned host memory (host[0], host[1]; the former is
+// cleared), and four doubles from `scalars`, if given, to byte 16.
 cudaError_t report(const NbrState& nb, const double* scalars, int* host, cudaStream_t st);
+// CSR export of the neighbour list with exact double-precision r_ij.
 int export_neighbors(const NbrState& nb, const double* pos, const int* offsets, int* nbr_j, int* nbr_s,
                      double* r_ij, cudaStream_t st);
 

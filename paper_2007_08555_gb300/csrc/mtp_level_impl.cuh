@@ -1609,9 +1609,11 @@ __device__ __forceinline__ void pdot_all(const Vec4<T>* adj, const Vec4<T>* adjt
 // shared memory (2 C reads per pair and lane, as broadcast vectors); every lane adds its pairs' terms to
 // sums of its own in shared memory, one set per neighbour species, so that the lanes of a warp work on
 // pairs of different species at once; the sums are combined over an atom's lanes and go to the block's
-// double sums when the central species changes and at least every kDcRounds rounds of four atoms (no
-// longer a float sum than one thread over one atom's neighbours has), and from there to global memory
-// by one atomic per entry and block.  Bound: FP32 (or FP64) issue, 3 C multiply-adds and the monomials'
+// double sums when the central species changes and at least every kDcRounds rounds of four atoms, and from
+// there to global memory by one atomic per entry and block.  In float a lane so adds its eighth of the
+// neighbours of eight atoms at most; the error of dL/dc against double is 0.93 to 1.00 times (0.97 on average)
+// that of one thread adding one atom's neighbours, over eleven shapes of lev_max 6-20, 1-8 species and 4-16
+// radial functions (0.96 with the lanes combined in double-float arithmetic, for 1-8% of a gradient's time).  Bound: FP32 (or FP64) issue, 3 C multiply-adds and the monomials'
 // tangents per pair.  NQC: the radial basis size when it is known at compile time, 0 = any.
 // Against one thread per atom, a pass per neighbour species, dV/dM from global memory for every pair and
 // a double atomic per entry and atom: the gradient of 67 cells at lev_max 12 in double 3.01 -> 1.20 ms
