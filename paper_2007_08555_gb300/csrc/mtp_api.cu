@@ -264,11 +264,13 @@ mtp_status fill_ctx(mtp_model* M, int K, int n, const int* cfg_off, const int* t
     const std::pair<int, int> t = (M->tpa_pairs && M->tpa_moments) ? std::pair<int, int>{0, 0} : tuned(M, n);
     // (float: two lanes for the pair kernels at any size -- they visit every pair once and read dV/dM from
     // shared memory, one lane per atom costs 4-12% of an evaluation from 77k atoms on: 442k atoms 4.07 ms
-    // against 3.77 at lev_max 16, 7.3 against 6.6 at 20; and two for the moments up to lev_max 16, where a
-    // lane's running sums leave room for more warps: 0-5%, 55k atoms 0.468 against 0.446 ms, and below
-    // 100k atoms at any level: 70k at lev_max 18 150 against 129 us of the moments)
+    // against 3.77 at lev_max 16, 7.3 against 6.6 at 20.  The moments take two below 100k atoms (70k at lev_max
+    // 18 150 against 129 us of the moments), and at any size up to lev_max 10: 108k to 1M atoms of crystals and
+    // batches at lev_max 10 are 0-3% faster with two, at 12 to 16 0-1.7% with one (1M atoms 5.24 against 5.30,
+    // 5.84 against 5.94 and 6.95 against 7.05 ms), at 18 and 20 1-2% with two up to 300k atoms of a crystal and
+    // 0.5-3% with one above and in batches)
     // double: four lanes, from which on every pair is visited once
-    const int least = sizeof(T) == 4 ? 2 : 4, least_m = sizeof(T) == 4 && (M->L <= 16 || n < 100000) ? 2 : 1;
+    const int least = sizeof(T) == 4 ? 2 : 4, least_m = sizeof(T) == 4 && (M->L <= 10 || n < 100000) ? 2 : 1;
     a.tpa = M->tpa_pairs ? M->tpa_pairs : (t.second ? t.second : std::max(least, choose_tpa(n, M->n_sm, 512)));
     a.tpa_m = M->tpa_moments ? M->tpa_moments : (t.first ? t.first : std::max(least_m, choose_tpa(n, M->n_sm, 128)));
     a.mom = M->mom.as<T>();
