@@ -59,7 +59,7 @@ def launchers(tmp_path_factory):
         build.build()
     d = tmp_path_factory.mktemp("fake")
     (d / "fake.cpp").write_text(FAKE)
-    subprocess.run(["g++", "-shared", "-fPIC", "-o", str(d / "fake.so"), str(d / "fake.cpp"), obj], check=True)
+    subprocess.run(["g++", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-o", str(d / "fake.so"), str(d / "fake.cpp"), obj], check=True)
     return ctypes.CDLL(str(d / "fake.so"))
 
 
