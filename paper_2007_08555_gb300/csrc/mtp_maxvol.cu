@@ -22,9 +22,9 @@
 // inverse are the same operations in the same order as elimination by one block with explicit
 // interchanges, so the selection does not depend on the number of blocks.
 // Bound: one exchange per step (a trip to the L2 for the records and one for the winner's row) and the
-// step's FMAs on the double-precision pipe (~2 per clock and SM).  Measured with all grades of the rows:
-// 232 x 116 in 1.51 ms, 920 x 460 in 8.0 ms; with flags and fences instead of tagged words 2.81 and 13.7;
-// one block with every matrix in global memory 11.3 and 482 ms.
+// step's FMAs and the swaps' divisions on the double-precision pipe (~2 FMAs per clock and SM).  Measured with
+// all grades of the rows: 232 x 116 in 1.66 ms, 920 x 460 in 8.4 ms; with flags and fences instead of tagged
+// words (and without the divisions) 2.81 and 13.7; one block with every matrix in global memory 10.8 and 451.
 // k_grade: gamma_r = max_j |(b_r A^-1)_j| for many rows; 64x64 output tiles through shared memory,
 //   the row maxima are combined with an atomic max on the bit pattern (gamma >= 0); a NaN in a row
 //   of b A^-1 gives gamma = +inf, so a broken configuration reads as extrapolating.
@@ -703,14 +703,15 @@ int mv_sm_count() {
     return n > 0 ? n : 1;
 }
 
-// Blocks of a cooperative kernel: as many as have two rows of A each and room for their exchange rows, two
-// for three SMs at most: fewer blocks take longer over their rows, more of them over the exchange (920 x 460:
-// 10.2 ms with 32 blocks, 7.5 with 64, 6.8 with 100, 7.6 with 128, 8.7 with 152; 232 x 116: 1.73 ms with 8,
-// 1.37 with 32, 1.31 with 58).  Where the exchange rows lie in memory matters too: of eight allocations seven
-// gave 6.7 against 8.5 ms, one 7.4 ms with either number of blocks.
+// Blocks of a cooperative kernel: as many as have two rows of A each and room for their exchange rows, one for
+// every SM at most.  More blocks take longer over the exchange and shorter over their rows, which also fit in
+// shared memory sooner: with 76, 101 (two thirds of the SMs), 128 and 152 blocks at most 920 x 460 takes 9.0,
+// 8.7, 8.5 and 8.6 ms, 2000 x 1000 70, 63, 49 and 33, 3000 x 2000 308, 270, 206 and 195, 20000 x 460 92, 73, 65
+// and 65; 232 x 116 (57 blocks by the room) 1.48 with all of them, 1.51 with 50.  Where the exchange rows lie in
+// memory moves 920 x 460 by up to 10%.
 int mv_blocks(int m, size_t slot_doubles) {
     const long by_slots = (long)(slot_doubles / (4 * (size_t)(m + 2)));
-    return (int)std::max(1l, std::min({(long)mv_sm_count() * 2 / 3, (long)m / 2, by_slots}));
+    return (int)std::max(1l, std::min({(long)mv_sm_count(), (long)m / 2, by_slots}));
 }
 size_t mv_slot_bytes(int m, int G) { return 32 * (size_t)G * (m + 2); }
 
@@ -735,7 +736,7 @@ int launch_invert(int m, const double* A, double* Ai, double* W, int* status, cu
     // W = [records 4 G | slots 4 G (m + 2) | rows m^2 if they do not fit in shared memory]
     const size_t mm = (size_t)m * m, per = 4 + 4 * (size_t)(m + 2);
     auto blocks = [&](size_t room) {
-        return (int)std::max(1l, std::min({(long)mv_sm_count() * 2 / 3, (long)m / 2, (long)(room / per)}));
+        return (int)std::max(1l, std::min({(long)mv_sm_count(), (long)m / 2, (long)(room / per)}));
     };
     int G = blocks(2 * mm);
     Layout l = mv_layout(m, m, G, false);

@@ -1062,8 +1062,8 @@ int build_neighbors(NbrState& nb, int K, int n, const int* cfg_off, const double
 }
 
 // Error word, largest neighbour count and (MD) four scalars to pinned host memory, the error word cleared:
-// one launch instead of a copy each and a memset (128 atoms at lev_max 10 120 -> 111 us a call, 16,384 atoms
-// at lev_max 16 242 -> 234 us, 16,384 atoms of MD 1.64 -> 1.57 ms for 10 steps).
+// one launch instead of a copy each and a memset (128 atoms at lev_max 10 120 -> 111 us a call, 16,384 atoms of
+// MD 1.64 -> 1.57 ms for 10 steps; on a call of 0.25 ms the gain is within the spread).
 __global__ void k_report(int* err, const int* max_seen, const double* scalars, int* host) {
     const int q = threadIdx.x;
     if (scalars && q < 4) reinterpret_cast<double*>(host + 4)[q] = scalars[q];
