@@ -86,7 +86,7 @@ struct mtp_model {
     bool tc_ready = false;
     std::vector<int> active_rows;
     DevBuf g_energy, g_forces, g_virial, g_D, g_eps, g_ew, g_momt, g_adjmt, g_out, g_refs;
-    DevBuf d_A, d_Ai, mv_W, mv_pos, mv_sel, mv_status, mv_swaps, mv_gmax, s_rows, s_gamma, g_brows, g_batoms;
+    DevBuf d_A, d_Ai, mv_W, mv_X, mv_pos, mv_sel, mv_status, mv_swaps, mv_gmax, s_rows, s_gamma, g_brows, g_batoms;
     // profiling: events around the neighbour build and each evaluation phase
     bool profiling = false;
     cudaEvent_t ev_nbr[2] = {nullptr, nullptr};
@@ -441,7 +441,7 @@ void mtp_destroy(mtp_model* M) {
                       &M->nb.bin_count, &M->nb.bin_start, &M->nb.atom_slot, &M->nb.bin_atoms, &M->nb.counters,
                       &M->nb.err, &M->g_energy, &M->g_forces, &M->g_virial, &M->g_D, &M->g_eps, &M->g_ew,
                       &M->g_momt, &M->g_adjmt, &M->g_out, &M->g_refs, &M->md_F, &M->md_scalars, &M->md_masses,
-                      &M->nb.x0, &M->nb.disp, &M->nb.cpr, &M->d_A, &M->d_Ai, &M->mv_W, &M->mv_pos, &M->mv_sel,
+                      &M->nb.x0, &M->nb.disp, &M->nb.cpr, &M->d_A, &M->d_Ai, &M->mv_W, &M->mv_X, &M->mv_pos, &M->mv_sel,
                       &M->mv_status, &M->mv_swaps, &M->mv_gmax, &M->s_rows, &M->s_gamma, &M->g_brows,
                       &M->g_batoms};
     for (DevBuf* b : bufs) b->release();
@@ -1313,8 +1313,8 @@ mtp_status mtp_select_active_set(mtp_model* M, int n_rows, const double* b_rows,
     M->g_sig.clear();  // A^-1 may move: no replay of an older graph
     cudaStream_t st = (cudaStream_t)stream;
     const int m = M->gw, n = n_rows;
-    const size_t wsz = std::max((size_t)n * m, (size_t)2 * m * m) + 2 * (size_t)m + n + 16;
-    if (M->mv_W.reserve(sizeof(double) * wsz) || M->mv_pos.reserve(sizeof(int) * n) ||
+    const size_t wsz = (size_t)n * m + n + 16, xsz = mtp::maxvol_exchange_doubles(n, m);
+    if (M->mv_W.reserve(sizeof(double) * wsz) || M->mv_X.reserve(sizeof(double) * xsz) || M->mv_pos.reserve(sizeof(int) * n) ||
         M->mv_sel.reserve(sizeof(int) * m) || M->d_A.reserve(sizeof(double) * m * m) ||
         M->d_Ai.reserve(sizeof(double) * m * m) ||
         M->mv_status.reserve(16) || M->mv_swaps.reserve(16) || M->mv_gmax.reserve(16))
@@ -1326,7 +1326,7 @@ mtp_status mtp_select_active_set(mtp_model* M, int n_rows, const double* b_rows,
         B = M->s_rows.as<double>();
     }
     cudaMemsetAsync(M->mv_status.p, 0, sizeof(int), st);
-    const int lm = mtp::launch_maxvol(n, m, B, M->mv_W.as<double>(), M->mv_pos.as<int>(), M->mv_sel.as<int>(),
+    const int lm = mtp::launch_maxvol(n, m, B, M->mv_W.as<double>(), M->mv_X.as<double>(), xsz, M->mv_pos.as<int>(), M->mv_sel.as<int>(),
                                       M->d_A.as<double>(), M->d_Ai.as<double>(), 1e-3, 100 * m,
                                       M->mv_status.as<int>(), M->mv_swaps.as<int>(), M->mv_gmax.as<double>(), st);
     if (lm < 0) {
@@ -1372,8 +1372,8 @@ mtp_status mtp_select_add(mtp_model* M, int n_cand, const double* cand_rows, int
     M->g_sig.clear();  // A^-1 moves: no replay of an older graph
     cudaStream_t st = (cudaStream_t)stream;
     const int m = M->gw, n = m + n_cand;
-    const size_t wsz = std::max((size_t)n * m, (size_t)2 * m * m) + 2 * (size_t)m + n + 16;
-    if (M->mv_W.reserve(sizeof(double) * wsz) || M->mv_pos.reserve(sizeof(int) * n) ||
+    const size_t wsz = (size_t)n * m + n + 16, xsz = mtp::maxvol_exchange_doubles(n, m);
+    if (M->mv_W.reserve(sizeof(double) * wsz) || M->mv_X.reserve(sizeof(double) * xsz) || M->mv_pos.reserve(sizeof(int) * n) ||
         M->mv_sel.reserve(sizeof(int) * m) ||
         M->mv_status.reserve(16) || M->mv_swaps.reserve(16) || M->mv_gmax.reserve(16) ||
         M->s_rows.reserve(sizeof(double) * (size_t)n * m))
@@ -1386,7 +1386,7 @@ mtp_status mtp_select_add(mtp_model* M, int n_cand, const double* cand_rows, int
         cudaMemcpyAsync(B + mm, cand_rows, sizeof(double) * (size_t)n_cand * m,
                         (flags & MTP_HOST_MEMORY) ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st);
     cudaMemsetAsync(M->mv_status.p, 0, sizeof(int), st);
-    const int lm = mtp::launch_maxvol(n, m, B, M->mv_W.as<double>(), M->mv_pos.as<int>(), M->mv_sel.as<int>(),
+    const int lm = mtp::launch_maxvol(n, m, B, M->mv_W.as<double>(), M->mv_X.as<double>(), xsz, M->mv_pos.as<int>(), M->mv_sel.as<int>(),
                                       M->d_A.as<double>(), M->d_Ai.as<double>(), 1e-3, 100 * m,
                                       M->mv_status.as<int>(), M->mv_swaps.as<int>(), M->mv_gmax.as<double>(), st, 1);
     if (lm < 0) {

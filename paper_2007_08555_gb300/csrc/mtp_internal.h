@@ -69,8 +69,10 @@ size_t scan_tmp_ints(int n);
 int scan_exclusive(const int* in, int* out, int n, int* tmp, cudaStream_t st);
 
 // Active set (mtp_maxvol.cu)
-int launch_maxvol(int n, int m, const double* B, double* W, int* pos, int* sel, double* A, double* Ai, double tol,
-                  int max_iter, int* status, int* swaps, double* gmax, cudaStream_t st, int start_given = 0);
+size_t maxvol_exchange_doubles(int n, int m);  // of X, for as many blocks as the sizes are worth
+int launch_maxvol(int n, int m, const double* B, double* W, double* X, size_t x_doubles, int* pos, int* sel, double* A,
+                  double* Ai, double tol, int max_iter, int* status, int* swaps, double* gmax, cudaStream_t st,
+                  int start_given = 0);
 int launch_invert(int m, const double* A, double* Ai, double* W, int* status, cudaStream_t st);
 template <class T>
 int launch_grade(int n, int m, const T* B, int ldb, const T* Ai, unsigned long long* gbits, cudaStream_t st);

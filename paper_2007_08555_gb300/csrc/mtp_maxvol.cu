@@ -393,7 +393,7 @@ struct MaxvolArgs {
     double* col;               // [max(n, m)], likewise
     int* pos;                  // [n], likewise
     unsigned long long* rec;   // [2][G][2], zero at the start (G > 1)
-    unsigned long long* slots; // [2][G][m + 2][2], zero at the start (G > 1); may lie in A
+    unsigned long long* slots; // [2][G][m + 2][2], zero at the start (G > 1)
     int* sel;                  // [m]
     double* A;                 // [m][m]
     double* Ai;                // [m][m]
@@ -594,12 +594,10 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
         ++swaps;
     }
     __syncthreads();
-    // A^-1 = D (A D)^-1, computed from scratch, and the unscaled A (possibly over the exchange's rows:
-    // after every block has read the last of them)
+    // A^-1 = D (A D)^-1, computed from scratch, and the unscaled A
     if (!shared && !x.barrier()) return;
     own(m, Rm);
     if (!invert_rows(x, a, orig, g.Ai, g.status, load, [&](int row) { return D[row]; })) return;
-    if (!x.barrier()) return;
     for (int e = tid; e < a.R * m; e += nt)
         g.A[(size_t)a.first * m + e] = g.B[(size_t)sel[a.first + e / m] * m + e % m];
     if (blockIdx.x == 0) {
@@ -703,15 +701,23 @@ int mv_sm_count() {
     return n > 0 ? n : 1;
 }
 
-// Blocks of a cooperative kernel: as many as have two rows of A each and room for their exchange rows, one for
-// every SM at most.  More blocks take longer over the exchange and shorter over their rows, which also fit in
-// shared memory sooner: with 76, 101 (two thirds of the SMs), 128 and 152 blocks at most 920 x 460 takes 9.0,
-// 8.7, 8.5 and 8.6 ms, 2000 x 1000 70, 63, 49 and 33, 3000 x 2000 308, 270, 206 and 195, 20000 x 460 92, 73, 65
-// and 65; 232 x 116 (57 blocks by the room) 1.48 with all of them, 1.51 with 50.  Where the exchange rows lie in
-// memory moves 920 x 460 by up to 10%.
-int mv_blocks(int m, size_t slot_doubles) {
-    const long by_slots = (long)(slot_doubles / (4 * (size_t)(m + 2)));
-    return (int)std::max(1l, std::min({(long)mv_sm_count(), (long)m / 2, by_slots}));
+// Blocks of a cooperative kernel: as many as have room for their exchange rows and two rows of A or 16 rows of B
+// each, one for two of three SMs at most if a block then has no more than 64 rows and shared memory holds them, else
+// one for every SM.  More blocks take longer over the exchange and shorter over their rows: with 76, 101, 128 and 152 of them 920 x 460 takes 9.0,
+// 8.7, 8.5 and 8.6 ms on one box, 101 8.8 against 9.3 with 152 on another, but 2000 x 1000 70, 63, 49 and 33 (in
+// shared memory at last), 3000 x 2000 308, 270, 206 and 195, 20000 x 460 92, 73, 65 and 65; 232 x 116 1.48 with 57,
+// 1.51 with 50.  Rows of B count for tall, narrow matrices (a block for 16, 64, 256 and 1024 of them): 1000 x 9 0.24,
+// 0.28, 0.52, 0.51 ms, 3000 x 17 0.47, 0.49, 1.01, 1.27, 100000 x 9 1.27, 1.26, 1.27, 1.75 (1.69 with 101 blocks at
+// most; by the rows of A alone, one block, 113).  Where the exchange rows lie in memory moves 920 x 460 by up to 15%.
+size_t mv_exchange(int m) { return 4 * (size_t)m + 12; }  // doubles of a block: two records, two rows
+int mv_blocks(int n, int m, size_t room, bool full) {
+    const long sms = mv_sm_count(), by_room = (long)(room / mv_exchange(m));
+    const auto most = [&](long limit) {
+        return (int)std::max(1l, std::min({limit, std::max((long)m / 2, (long)n / 16), by_room}));
+    };
+    const int few = most(sms * 2 / 3);
+    const Layout l = mv_layout(n, m, few, full);
+    return l.rows_in && l.col_in && l.R <= 64 ? few : most(sms);
 }
 size_t mv_slot_bytes(int m, int G) { return 32 * (size_t)G * (m + 2); }
 
@@ -734,14 +740,11 @@ int mv_launch(K kernel, Args& g, int G, size_t smem, cudaStream_t st) {
 // W: 2 m^2 + 4 doubles, 16-byte aligned.
 int launch_invert(int m, const double* A, double* Ai, double* W, int* status, cudaStream_t st) {
     // W = [records 4 G | slots 4 G (m + 2) | rows m^2 if they do not fit in shared memory]
-    const size_t mm = (size_t)m * m, per = 4 + 4 * (size_t)(m + 2);
-    auto blocks = [&](size_t room) {
-        return (int)std::max(1l, std::min({(long)mv_sm_count(), (long)m / 2, (long)(room / per)}));
-    };
-    int G = blocks(2 * mm);
+    const size_t mm = (size_t)m * m;
+    int G = mv_blocks(m, m, 2 * mm, false);
     Layout l = mv_layout(m, m, G, false);
     if (!l.rows_in) {
-        G = blocks(mm);
+        G = mv_blocks(m, m, mm, false);
         l = mv_layout(m, m, G, false);
     }
     if (!l.col_in || l.bytes > kMvSharedMost) return -1;  // above m = 16,000
@@ -750,26 +753,18 @@ int launch_invert(int m, const double* A, double* Ai, double* W, int* status, cu
     return mv_launch(k_invert, g, G, l.bytes, st);
 }
 
-// W: max(n m, 2 m^2) + 2 m + n doubles, 16-byte aligned, pos: n ints.
-int launch_maxvol(int n, int m, const double* B, double* W, int* pos, int* sel, double* A, double* Ai, double tol,
-                  int max_iter, int* status, int* swaps, double* gmax, cudaStream_t st, int start_given) {
-    const size_t nm = (size_t)n * m, mm = (size_t)m * m;
-    // records at the start of W (4 G <= 2 m doubles); then the exchange's rows, where the matrix's rows
-    // are in shared memory, else the matrix's rows and column, with the exchange's rows in A
-    int G = mv_blocks(m, std::max(nm, 2 * mm));
-    Layout l = mv_layout(n, m, G, true);
-    const bool in = l.rows_in && l.col_in;
-    if (!in) {
-        G = mv_blocks(m, mm - 1);  // (A need not be 16-byte aligned)
-        l = mv_layout(n, m, G, true);
-    }
+size_t maxvol_exchange_doubles(int n, int m) { return mv_exchange(m) * (size_t)mv_blocks(n, m, ~(size_t)0 / 2, true); }
+
+// W: n m + n doubles; X: x_doubles doubles (any number: fewer give fewer blocks), 16-byte aligned; pos: n ints.
+int launch_maxvol(int n, int m, const double* B, double* W, double* X, size_t x_doubles, int* pos, int* sel, double* A,
+                  double* Ai, double tol, int max_iter, int* status, int* swaps, double* gmax, cudaStream_t st,
+                  int start_given) {
+    const int G = mv_blocks(n, m, x_doubles, true);
+    const Layout l = mv_layout(n, m, G, true);
     if (l.bytes > kMvSharedMost) return -1;  // above m = 6382; a model's widest active set is 5580 columns
-    auto* rec = reinterpret_cast<unsigned long long*>(W);
-    double* rest = W + 2 * (size_t)m;
-    auto* in_A = reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(A) + 15) & ~(uintptr_t)15);
-    MaxvolArgs g{n, m, G, l.br, l.rows_in, l.col_in, B, rest, rest + std::max(nm, 2 * mm), pos, rec,
-                 in ? reinterpret_cast<unsigned long long*>(rest) : in_A, sel, A, Ai, tol, max_iter, start_given, status,
-                 swaps, gmax};
+    auto* rec = reinterpret_cast<unsigned long long*>(X);
+    MaxvolArgs g{n, m, G, l.br, l.rows_in, l.col_in, B, W, W + (size_t)n * m, pos, rec, rec + 4 * (size_t)G, sel, A, Ai, tol,
+                 max_iter, start_given, status, swaps, gmax};
     return mv_launch(k_maxvol, g, G, l.bytes, st);
 }
 
@@ -850,9 +845,8 @@ extern "C" mtp_status mtp_select_active_set_noalloc(int n_rows, int m, const dou
                                                     double* a_inv, int* n_swaps, void* stream) {
     using namespace mtp;
     if (m < 1 || n_rows < m || !b_rows || !selected) return MTP_EINVAL;
-    // the documented limit (2 n m + m doubles of it are unused); layout inside the fixed array (in
-    // doubles): W [max(n m, 2 m m) + 2 m + n]; A, A^-1 [m m]; then ints: pos [n], sel [m], status,
-    // swaps; then gmax.
+    // the documented limit; layout inside the fixed array (in doubles): W [max(n m, 2 m m) + 2 m + n]; A,
+    // A^-1 [m m]; then ints: pos [n], sel [m], status, swaps; then the exchange (2 n m + m); then gmax.
     const size_t nm = (size_t)n_rows * m, mm = (size_t)m * m;
     const size_t w = (nm > 2 * mm ? nm : 2 * mm) + 2 * (size_t)m + n_rows;
     const size_t ints = (size_t)n_rows + m + 2;
@@ -867,10 +861,12 @@ extern "C" mtp_status mtp_select_active_set_noalloc(int n_rows, int m, const dou
     int* sel = pos + n_rows;
     int* status = sel + m;
     int* swaps = status + 1;
+    const size_t x0 = (w + 2 * mm + (ints + 1) / 2 + 1) & ~(size_t)1;  // 16-byte aligned
+    const size_t x_doubles = x0 < need - 1 ? need - 1 - x0 : 0;
     double* gmax = reinterpret_cast<double*>(base + (need - 1));
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaMemsetAsync(status, 0, 2 * sizeof(int), st) != cudaSuccess) return MTP_ECUDA;
-    if (launch_maxvol(n_rows, m, b_rows, W, pos, sel, A, Ai, 1e-3, 100 * m, status, swaps, gmax, st, 0) < 0)
+    if (launch_maxvol(n_rows, m, b_rows, W, base + x0, x_doubles, pos, sel, A, Ai, 1e-3, 100 * m, status, swaps, gmax, st, 0) < 0)
         return MTP_ECUDA;
     int h[2] = {0, 0};
     if (cudaMemcpyAsync(h, status, sizeof h, cudaMemcpyDeviceToHost, st) != cudaSuccess) return MTP_ECUDA;

@@ -1,5 +1,5 @@
-"""MaxVol of so many rows that the blocks' rows, and their positions, lie in global memory (Sec. 2.3): several blocks
-whose shares of B and of A overlap.  The selection equals a plain restatement (elimination with partial
+"""MaxVol of so many rows that the blocks' rows, and their positions, lie in global memory (Sec. 2.3), so that the
+blocks' shares of B and of A overlap, and of tall, narrow matrices with more blocks than columns.  The selection equals a plain restatement (elimination with partial
 pivoting, then swaps by C = B A^-1 from scratch); A A^-1 = 1 within 64 eps m cond(A)."""
 
 import numpy as np
@@ -29,7 +29,8 @@ def _maxvol(B):
         swaps += 1
 
 
-@pytest.mark.parametrize("n,m", [(20011, 29), (90001, 29), (120007, 32), (200003, 61)])
+@pytest.mark.parametrize("n,m", [(20011, 29), (90001, 29), (120007, 32), (200003, 61), (33, 1), (517, 2),
+                                 (1000, 9), (100003, 9), (3001, 17)])
 def test_selection_from_many_rows(gpu_lib, n, m):
     model = mtp.Model(12, 2, 8, 2.0, 5.0)
     model.set_grade_kind(True, np.arange(m, dtype=np.int32))

@@ -35,8 +35,8 @@ void __cudaRegisterFunction(...) {}
 void __cudaRegisterVar(...) {}
 }
 namespace mtp {
-int launch_maxvol(int, int, const double*, double*, int*, int*, double*, double*, double, int, int*, int*, double*,
-                  CUstream_st*, int);
+int launch_maxvol(int, int, const double*, double*, double*, size_t, int*, int*, double*, double*, double, int, int*, int*,
+                  double*, CUstream_st*, int);
 int launch_invert(int, const double*, double*, double*, int*, CUstream_st*);
 }
 extern "C" int run(int invert, int n, int m, int fail, int* left) {
@@ -45,7 +45,8 @@ extern "C" int run(int invert, int n, int m, int fail, int* left) {
   fail_at = fail;
   calls = pending = 0;
   int r = invert ? mtp::launch_invert(m, none, none, none, &zero, nullptr)
-                 : mtp::launch_maxvol(n, m, none, none, &zero, &zero, none, none, 1e-3, 100, &zero, &zero, none, nullptr, 0);
+                 : mtp::launch_maxvol(n, m, none, none, none, 1 << 20, &zero, &zero, none, none, 1e-3, 100, &zero, &zero, none,
+                                      nullptr, 0);
   *left = pending;
   return r;
 }
@@ -64,7 +65,7 @@ def launchers(tmp_path_factory):
 
 
 @pytest.mark.parametrize("invert", [0, 1])
-@pytest.mark.parametrize("n,m,steps", [(40, 3, 2), (232, 116, 4)])  # one block; several: two memsets come first
+@pytest.mark.parametrize("n,m,steps", [(9, 3, 2), (232, 116, 4)])  # one block; several: two memsets come first
 def test_a_failed_launch_leaves_no_error(launchers, invert, n, m, steps):
     left = ctypes.c_int()
     for fail in range(steps + 1):  # the last one lets every call pass
