@@ -481,9 +481,11 @@ __global__ void __launch_bounds__(kMvThreads) k_maxvol(const MaxvolArgs g) {
             }
             bool bad = false;
             for (int c = k + 1 + tid; c < m; c += nt) a.prow[c] = x.receive(q, c, &bad);
-            if (tid == nt - 1) sel[k] = (int)x.receive(q, m, &bad);
-            const double pivot = tid < a.R ? x.receive(q, k, &bad) : 1.0;
-            for (int r = tid; r < a.R; r += nt) {
+            if (tid == nt / 2) sel[k] = (int)x.receive(q, m, &bad);
+            // (the last warps: the division, over a thousand clocks, runs beside the row's arrival)
+            const int rt = nt - 1 - tid;
+            const double pivot = rt < a.R ? x.receive(q, k, &bad) : 1.0;
+            for (int r = rt; r < a.R; r += nt) {
                 if (a.pos[r] == (int)p)
                     a.pos[r] = k;
                 else if (a.pos[r] == k)
