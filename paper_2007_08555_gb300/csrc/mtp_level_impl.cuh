@@ -1151,7 +1151,20 @@ int launch_pairs(const EvalCtx<T>& a, cudaStream_t st, int n_sm, bool moments) {
             cudaFuncSetAttribute(k_pairgrad<T, TPA>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
             attr_set = true;
         }
-        launch_pdl(k_pairgrad<T, TPA>, blocks, threads, smem, st, a);
+        // Started early, its blocks go to whichever SMs the contraction leaves first and crowd there, where a
+        // grid of a few waves then runs as long as the fullest SM.  In double (sixteen clocks a warp instruction)
+        // from lev_max 12 on that always costs more than the launch's latency: lanes 2, 1 on 9322 atoms at lev_max 20
+        // 12.9 -> 6.9 ms, 2048 atoms at 16 0.51 -> 0.40; below between one and four blocks per SM: 6912 atoms at 10
+        // 434 -> 409 us (16,384 would lose, 747 -> 767).  In float from lev_max 16 on between
+        // half a wave and four blocks per SM: 6912 atoms at 16, 18, 20 129 -> 119, 167 -> 148, 240 -> 191 us, 2048
+        // atoms at 18, 20 118 -> 109, 144 -> 131; elsewhere the early start gains 1-5 us.
+        constexpr bool heavy = sizeof(T) == 8 && G::L_ >= 12;
+        const int from = sizeof(T) == 8 ? n_sm : n_sm / 2;
+        const bool apart = heavy || ((sizeof(T) == 8 || G::L_ >= 16) && blocks >= from && blocks <= n_sm * 4);
+        if (apart)
+            k_pairgrad<T, TPA><<<blocks, threads, smem, st>>>(a);
+        else
+            launch_pdl(k_pairgrad<T, TPA>, blocks, threads, smem, st, a);
     }
     return 1;
 }
