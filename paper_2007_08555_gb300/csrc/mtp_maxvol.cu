@@ -23,7 +23,7 @@
 // interchanges, so the selection does not depend on the number of blocks.
 // Bound: one exchange per step (a trip to the L2 for the records and one for the winner's row) and the
 // step's FMAs and the swaps' divisions on the double-precision pipe (~2 FMAs per clock and SM).  Measured with
-// all grades of the rows: 232 x 116 in 1.66 ms, 920 x 460 in 8.4 ms; with flags and fences instead of tagged
+// all grades of the rows: 232 x 116 in 1.68 ms, 920 x 460 in 8.2 ms; with flags and fences instead of tagged
 // words (and without the divisions) 2.81 and 13.7; one block with every matrix in global memory 10.8 and 451.
 // k_grade: gamma_r = max_j |(b_r A^-1)_j| for many rows; 64x64 output tiles through shared memory,
 //   the row maxima are combined with an atomic max on the bit pattern (gamma >= 0); a NaN in a row
